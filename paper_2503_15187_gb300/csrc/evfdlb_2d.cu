@@ -45,7 +45,19 @@ struct Slab2 {
     long long N;          // nodes, nx * ny
     int nft, nfm;         // force and Fischer-Methfessel taps
     int Mf, mfm;          // their radii in nodes
-    double dx, inv_dx, dt, weno_eps, b, eta_coef, mu0_coef;
+    double dx;
+};
+
+// The model constants a kernel multiplies by, in its precision R, rounded on
+// the host.  An FP32 kernel that takes them as doubles converts them on the
+// FP64 pipe, and the compiler forms such conversions (and a compare of a
+// double stage weight) again inside the plane loop instead of holding their
+// results: they kept that pipe 65 % busy in k2_adv2.
+template <typename R>
+struct Par2 {
+    R inv_dx, k12, dt, weno_eps, b, eta_coef, mu0_coef;   // k12 = 1 / (12 dx)
+    R alpha, beta;                                         // Shu-Osher weights of the stage (k2_adv, k2_adv2)
+    int with_base;                                         // alpha != 0
 };
 
 // raw moment sums per node ([kNumMom2][N], FP64)
@@ -362,7 +374,7 @@ __host__ __device__ inline size_t fields_smem_bytes(int Mf, int mfm) {
 
 template <typename R>
 __global__ void __launch_bounds__(256)
-k2_fields(Slab2 s, const double* __restrict__ mom, const float* __restrict__ prf, const R* __restrict__ ftw,
+k2_fields(Slab2 s, const Par2<R> pr, const double* __restrict__ mom, const float* __restrict__ prf, const R* __restrict__ ftw,
           const int* __restrict__ fplan, const int* __restrict__ fm_off, const R* __restrict__ fm_w,
           R* __restrict__ fld, unsigned* err) {
     constexpr bool F32 = std::is_same<R, float>::value;
@@ -411,7 +423,7 @@ k2_fields(Slab2 s, const double* __restrict__ mom, const float* __restrict__ prf
         const int hy = cy - 2 + H, hx = cx - 2 + H;   // position in the halo array
         R nb = R(0);
         for (int t = 0; t < s.nfm; ++t) nb = fma(fm_w[t], Nr[(hy + fm_off[2 * t + 1]) * Wr + hx + fm_off[2 * t]], nb);
-        const R eta = (R)s.eta_coef * nb, om = R(1) - eta;
+        const R eta = pr.eta_coef * nb, om = R(1) - eta;
         const R chi = (R(2) - eta) / (R(2) * om * om * om);
         const R n = Nr[hy * Wr + hx];
         Ct[e] = chi;
@@ -475,7 +487,7 @@ k2_fields(Slab2 s, const double* __restrict__ mom, const float* __restrict__ prf
     if (x >= nx || y >= ny) return;
     const long long i = (long long)y * nx + x;
     const int c = (ty + 2) * E + (tx + 2);
-    const R k12 = (R)(s.inv_dx / 12.0);
+    const R k12 = pr.k12;
     auto d4x = [&](const R* f) { return (f[c - 2] - R(8) * f[c - 1] + R(8) * f[c + 1] - f[c + 2]) * k12; };
     auto d4y = [&](const R* f) { return (f[c - 2 * E] - R(8) * f[c - E] + R(8) * f[c + E] - f[c + 2 * E]) * k12; };
     const R ux = U[c], uy = V[c], T = Tt[c], X = Xt[c], chi = Ct[c];
@@ -500,8 +512,8 @@ k2_fields(Slab2 s, const double* __restrict__ mom, const float* __restrict__ prf
     }
     // transport, Eqs. (viscosity), (tau), (prandtl)
     const R c16 = R((4.0 / 25.0) * (1.0 + 12.0 / M_PI)), c9 = R((9.0 / 25.0) * (1.0 + 32.0 / (9.0 * M_PI)));
-    const R bn = (R)s.b * n, xx = bn * chi;
-    const R mu = (R)s.mu0_coef * sqrt(T) * (R(1) / chi + R(0.8) * bn + c16 * bn * bn * chi);
+    const R bn = pr.b * n, xx = bn * chi;
+    const R mu = pr.mu0_coef * sqrt(T) * (R(1) / chi + R(0.8) * bn + c16 * bn * bn * chi);
     const R tau = mu / (n * T * (R(1) + R(0.4) * xx));
     const R Pr = R(2.0 / 3.0) * (R(1) + R(0.6) * xx) * (R(1) + R(0.8) * xx + c16 * xx * xx) /
                  ((R(1) + R(0.4) * xx) * (R(1) + R(1.2) * xx + c9 * xx * xx));
@@ -848,8 +860,8 @@ constexpr int adv_min_blocks() { return std::is_same<R, float>::value ? 4 : 2; }
 
 template <typename R, int Q, bool RHS>
 __global__ void __launch_bounds__(256, adv_min_blocks<R>())
-k2_adv(Slab2 s, const R* __restrict__ rtab, const R* __restrict__ src, const R* base, R* out,
-       const R* __restrict__ RL, double* rhs_out, double alpha, double beta) {
+k2_adv(Slab2 s, const Par2<R> pr, const R* __restrict__ rtab, const R* __restrict__ src, const R* base, R* out,
+       const R* __restrict__ RL, double* rhs_out) {
     constexpr int WX = kAdvX + 6, WY = kAdvY + 6, NH = WX * WY;
     constexpr int NHR = (NH + 255) / 256;                   // halo loads per thread
     constexpr int RPW = kAdvY / 8;                          // output rows per warp
@@ -878,8 +890,8 @@ k2_adv(Slab2 s, const R* __restrict__ rtab, const R* __restrict__ src, const R* 
         const int e = threadIdx.x + 256 * j;
         hoff[j] = (e < NH) ? rowoff[e / WX] + coloff[e % WX] : 0;
     }
-    const R eps = (R)s.weno_eps, idx = (R)s.inv_dx, dt = (R)s.dt, ralpha = (R)alpha, rbeta = (R)beta;
-    const bool with_base = (alpha != 0.0);
+    const R eps = pr.weno_eps, idx = pr.inv_dx, dt = pr.dt, ralpha = pr.alpha, rbeta = pr.beta;
+    const bool with_base = pr.with_base != 0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // this thread's run of faces: along x (threads 0-127) or y (128-255)
     const bool xrun = threadIdx.x < 128;
@@ -1140,8 +1152,8 @@ __device__ __forceinline__ void adv2_issue(float* buf, const float* src, const f
 // per SM the kernel executed 9 % more instructions and took 10 % longer)
 template <int Q>
 __global__ void __launch_bounds__(256, 3)
-k2_adv2(Slab2 s, const float* __restrict__ rtab, const float* __restrict__ src, const float* base, float* out,
-        const float* __restrict__ RL, double alpha, double beta) {
+k2_adv2(Slab2 s, const Par2<float> pr, const float* __restrict__ rtab, const float* __restrict__ src,
+        const float* base, float* out, const float* __restrict__ RL) {
     constexpr int K = Q * Q, RPW = kAdvY / 8;
     static_assert(kAdvX == 32 && kAdvY == 16, "run split: 33 = 5 + 7 x 4 x-faces, 17 = 5 + 3 x 4 y-faces");
     extern __shared__ __align__(16) double sma[];
@@ -1162,9 +1174,8 @@ k2_adv2(Slab2 s, const float* __restrict__ rtab, const float* __restrict__ src, 
     __syncthreads();
     const bool fast = (nx % 4 == 0) && (x0 + kAdvX <= nx) && (y0 + kAdvY <= ny);
     const Adv2Copies cplan = adv2_plan(rowoff, coloff, x0, y0, nx);
-    const float eps = (float)s.weno_eps, idx = (float)s.inv_dx, dt = (float)s.dt, ralpha = (float)alpha,
-                rbeta = (float)beta;
-    const bool with_base = (alpha != 0.0);
+    const float eps = pr.weno_eps, idx = pr.inv_dx, dt = pr.dt, ralpha = pr.alpha, rbeta = pr.beta;
+    const bool with_base = pr.with_base != 0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool xrun = threadIdx.x < 128;
     const int rj = xrun ? (threadIdx.x >> 4) : ((threadIdx.x - 128) >> 5);
@@ -1584,6 +1595,7 @@ struct Ctx2 {
     evfdlb_params p;
     Slab2 s;
     int prec = EVFDLB_FP32;
+    double dt = 0.0;
     size_t esize = 4;
     cudaStream_t user = nullptr, cap = nullptr;
     void* state[3] = {nullptr, nullptr, nullptr};
@@ -1603,6 +1615,20 @@ struct Ctx2 {
     unsigned* err = nullptr;
     cudaGraphExec_t g_one = nullptr;
     size_t smem_fields = 0, smem_coll = 0;
+    // the model constants in precision R (the stage weights are the caller's)
+    template <typename R>
+    Par2<R> par() const {
+        Par2<R> q{};
+        const double sg = p.sigma, idx = 1.0 / p.dx;
+        q.inv_dx = (R)idx;
+        q.k12 = (R)(idx / 12.0);
+        q.dt = (R)dt;
+        q.weno_eps = (R)p.weno_eps;
+        q.b = (R)(2.0 * M_PI * sg * sg * sg / 3.0);
+        q.eta_coef = (R)(M_PI * sg * sg * sg / 6.0);
+        q.mu0_coef = (R)(5.0 / (16.0 * sg * sg * sqrt(M_PI)));
+        return q;
+    }
 };
 
 namespace {
@@ -1624,38 +1650,38 @@ void launch_coll(int Q, int nc, size_t smem, cudaStream_t st, const Slab2& s, co
 // k2_adv is compiled for each even Q of the 2D model (4 .. 16) and both
 // output forms
 template <typename R, bool RHS>
-void launch_adv_t(int Q, dim3 g, cudaStream_t st, const Slab2& s, const R* rtab, const R* src, const R* base,
-                  R* out, const R* RL, double* rhs_out, double alpha, double beta) {
+void launch_adv_t(int Q, dim3 g, cudaStream_t st, const Slab2& s, const Par2<R>& pr, const R* rtab, const R* src,
+                  const R* base, R* out, const R* RL, double* rhs_out) {
     switch (Q) {
-        case 4: k2_adv<R, 4, RHS><<<g, 256, 0, st>>>(s, rtab, src, base, out, RL, rhs_out, alpha, beta); break;
-        case 6: k2_adv<R, 6, RHS><<<g, 256, 0, st>>>(s, rtab, src, base, out, RL, rhs_out, alpha, beta); break;
-        case 8: k2_adv<R, 8, RHS><<<g, 256, 0, st>>>(s, rtab, src, base, out, RL, rhs_out, alpha, beta); break;
-        case 10: k2_adv<R, 10, RHS><<<g, 256, 0, st>>>(s, rtab, src, base, out, RL, rhs_out, alpha, beta); break;
-        case 12: k2_adv<R, 12, RHS><<<g, 256, 0, st>>>(s, rtab, src, base, out, RL, rhs_out, alpha, beta); break;
-        case 14: k2_adv<R, 14, RHS><<<g, 256, 0, st>>>(s, rtab, src, base, out, RL, rhs_out, alpha, beta); break;
-        default: k2_adv<R, 16, RHS><<<g, 256, 0, st>>>(s, rtab, src, base, out, RL, rhs_out, alpha, beta); break;
+        case 4: k2_adv<R, 4, RHS><<<g, 256, 0, st>>>(s, pr, rtab, src, base, out, RL, rhs_out); break;
+        case 6: k2_adv<R, 6, RHS><<<g, 256, 0, st>>>(s, pr, rtab, src, base, out, RL, rhs_out); break;
+        case 8: k2_adv<R, 8, RHS><<<g, 256, 0, st>>>(s, pr, rtab, src, base, out, RL, rhs_out); break;
+        case 10: k2_adv<R, 10, RHS><<<g, 256, 0, st>>>(s, pr, rtab, src, base, out, RL, rhs_out); break;
+        case 12: k2_adv<R, 12, RHS><<<g, 256, 0, st>>>(s, pr, rtab, src, base, out, RL, rhs_out); break;
+        case 14: k2_adv<R, 14, RHS><<<g, 256, 0, st>>>(s, pr, rtab, src, base, out, RL, rhs_out); break;
+        default: k2_adv<R, 16, RHS><<<g, 256, 0, st>>>(s, pr, rtab, src, base, out, RL, rhs_out); break;
     }
 }
 
 // the FP32 stage form: F and G of a velocity as float2 pairs
-void launch_adv2(int Q, dim3 g, cudaStream_t st, const Slab2& s, const float* rtab, const float* src,
-                 const float* base, float* out, const float* RL, double alpha, double beta) {
+void launch_adv2(int Q, dim3 g, cudaStream_t st, const Slab2& s, const Par2<float>& pr, const float* rtab,
+                 const float* src, const float* base, float* out, const float* RL) {
     switch (Q) {
-        case 4: k2_adv2<4><<<g, 256, kA2Smem, st>>>(s, rtab, src, base, out, RL, alpha, beta); break;
-        case 6: k2_adv2<6><<<g, 256, kA2Smem, st>>>(s, rtab, src, base, out, RL, alpha, beta); break;
-        case 8: k2_adv2<8><<<g, 256, kA2Smem, st>>>(s, rtab, src, base, out, RL, alpha, beta); break;
-        case 10: k2_adv2<10><<<g, 256, kA2Smem, st>>>(s, rtab, src, base, out, RL, alpha, beta); break;
-        case 12: k2_adv2<12><<<g, 256, kA2Smem, st>>>(s, rtab, src, base, out, RL, alpha, beta); break;
-        case 14: k2_adv2<14><<<g, 256, kA2Smem, st>>>(s, rtab, src, base, out, RL, alpha, beta); break;
-        default: k2_adv2<16><<<g, 256, kA2Smem, st>>>(s, rtab, src, base, out, RL, alpha, beta); break;
+        case 4: k2_adv2<4><<<g, 256, kA2Smem, st>>>(s, pr, rtab, src, base, out, RL); break;
+        case 6: k2_adv2<6><<<g, 256, kA2Smem, st>>>(s, pr, rtab, src, base, out, RL); break;
+        case 8: k2_adv2<8><<<g, 256, kA2Smem, st>>>(s, pr, rtab, src, base, out, RL); break;
+        case 10: k2_adv2<10><<<g, 256, kA2Smem, st>>>(s, pr, rtab, src, base, out, RL); break;
+        case 12: k2_adv2<12><<<g, 256, kA2Smem, st>>>(s, pr, rtab, src, base, out, RL); break;
+        case 14: k2_adv2<14><<<g, 256, kA2Smem, st>>>(s, pr, rtab, src, base, out, RL); break;
+        default: k2_adv2<16><<<g, 256, kA2Smem, st>>>(s, pr, rtab, src, base, out, RL); break;
     }
 }
 
 template <typename R>
-void launch_adv(int Q, dim3 g, cudaStream_t st, const Slab2& s, const R* rtab, const R* src, const R* base, R* out,
-                const R* RL, double* rhs_out, double alpha, double beta, int mode) {
-    if (mode == 1) launch_adv_t<R, true>(Q, g, st, s, rtab, src, base, out, RL, rhs_out, alpha, beta);
-    else launch_adv_t<R, false>(Q, g, st, s, rtab, src, base, out, RL, rhs_out, alpha, beta);
+void launch_adv(int Q, dim3 g, cudaStream_t st, const Slab2& s, const Par2<R>& pr, const R* rtab, const R* src,
+                const R* base, R* out, const R* RL, double* rhs_out, int mode) {
+    if (mode == 1) launch_adv_t<R, true>(Q, g, st, s, pr, rtab, src, base, out, RL, rhs_out);
+    else launch_adv_t<R, false>(Q, g, st, s, pr, rtab, src, base, out, RL, rhs_out);
 }
 
 // k2_moments: 128 nodes per CTA pass (grid-stride beyond 8192 CTAs)
@@ -1699,23 +1725,29 @@ void queue_stage_t(Ctx2* c, cudaStream_t st, const void* src, const void* base, 
     // FP32: the field kernel reads the FP32 primitives; the FP64 raw sums are
     // only needed by the FP64 build and by the diagnostics
     const int nbm = moments_grid(s.N);
+    Par2<R> pr = c->template par<R>();
+    pr.alpha = (R)alpha;
+    pr.beta = (R)beta;
+    pr.with_base = alpha != 0.0;
     if constexpr (F32) launch_moments<float>(Q, nbm, st, s, c->pwf, (const float*)src, nullptr, c->prf, c->err);
     else launch_moments<double>(Q, nbm, st, s, c->pwd, (const double*)src, c->mom, nullptr, c->err);
     dim3 gf((s.nx + kTile2 - 1) / kTile2, (s.ny + kTile2 - 1) / kTile2);
-    k2_fields<R><<<gf, 256, c->smem_fields, st>>>(s, c->mom, c->prf, (const R*)c->ftw, c->fplan, c->fm_off,
+    k2_fields<R><<<gf, 256, c->smem_fields, st>>>(s, pr, c->mom, c->prf, (const R*)c->ftw, c->fplan, c->fm_off,
                                                    (const R*)c->fm_w, (R*)c->fld, c->err);
     int nc = (int)((s.N + kNB - 1) / kNB);
     launch_coll<R>(Q, nc, c->smem_coll, st, s, (const R*)c->rtab, (const R*)src, (const R*)c->fld, (R*)c->RL);
     const int tiles = ((s.nx + kAdvX - 1) / kAdvX) * ((s.ny + kAdvY - 1) / kAdvY);
-    if (F32 && mode == 0) {   // the FP32 stage form: one CTA column per group of velocities, F and G paired
-        dim3 ga(tiles, (Q * Q + kAdvPlanes - 1) / kAdvPlanes);
-        launch_adv2(Q, ga, st, s, (const float*)c->rtab, (const float*)src, (const float*)base, (float*)out,
-                    (const float*)c->RL, alpha, beta);
-    } else {
-        dim3 ga(tiles, (2 * Q * Q + kAdvPlanes - 1) / kAdvPlanes);
-        launch_adv<R>(Q, ga, st, s, (const R*)c->rtab, (const R*)src, (const R*)base, (R*)out, (const R*)c->RL,
-                      rhs_out, alpha, beta, mode);
+    if constexpr (F32) {
+        if (mode == 0) {   // the FP32 stage form: one CTA column per group of velocities, F and G paired
+            dim3 ga(tiles, (Q * Q + kAdvPlanes - 1) / kAdvPlanes);
+            launch_adv2(Q, ga, st, s, pr, (const float*)c->rtab, (const float*)src, (const float*)base, (float*)out,
+                        (const float*)c->RL);
+            return;
+        }
     }
+    dim3 ga(tiles, (2 * Q * Q + kAdvPlanes - 1) / kAdvPlanes);
+    launch_adv<R>(Q, ga, st, s, pr, (const R*)c->rtab, (const R*)src, (const R*)base, (R*)out, (const R*)c->RL,
+                  rhs_out, mode);
 }
 
 void queue_stage(Ctx2* c, cudaStream_t st, const void* src, const void* base, void* out, double* rhs_out,
@@ -1772,12 +1804,7 @@ evfdlb_status create_2d(const evfdlb_params& p, void* stream, Ctx2** out) {
     s.relax = p.relax_mode;
     s.N = (long long)p.nx * p.ny;
     s.dx = p.dx;
-    s.inv_dx = 1.0 / p.dx;
-    s.dt = resolved_dt_2d(p);
-    s.weno_eps = p.weno_eps;
-    s.b = 2.0 * M_PI * p.sigma * p.sigma * p.sigma / 3.0;
-    s.eta_coef = M_PI * p.sigma * p.sigma * p.sigma / 6.0;
-    s.mu0_coef = 5.0 / (16.0 * p.sigma * p.sigma * sqrt(M_PI));
+    c->dt = resolved_dt_2d(p);
     Taps2 t = taps_2d(p);
     s.nft = (int)(t.fg.size() / 2);
     s.nfm = (int)t.mw.size();
@@ -1884,7 +1911,7 @@ evfdlb_status check_2d(Ctx2* c) {
 
 long long nodes_2d(const Ctx2* c) { return c->s.N; }
 long long dist_2d(const Ctx2* c) { return (long long)c->s.Q * c->s.Q * c->s.N; }
-double dt_2d(const Ctx2* c) { return c->s.dt; }
+double dt_2d(const Ctx2* c) { return c->dt; }
 
 evfdlb_status init_2d(Ctx2* c, const double* n0, const double* u0, const double* T0, int on_device) {
     const long long N = c->s.N;
