@@ -583,6 +583,7 @@ evfdlb_status evfdlb_create(const evfdlb_params* p, int32_t nbatch, const evfdlb
         d.eta_coef = M_PI * q.sigma * q.sigma * q.sigma / 6.0;
         d.mu0_coef = 5.0 / (16.0 * q.sigma * q.sigma * sqrt(M_PI));
         d.T_iso = q.T_iso;
+        d.round_f32();
         if (q.T_iso > 0.0) c->iso = true;
         NF += (long long)q.Q * q.nx;
         NN += q.nx;

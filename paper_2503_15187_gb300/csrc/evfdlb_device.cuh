@@ -162,6 +162,27 @@ __device__ __forceinline__ bool positive(double x) {
     return b > 0 && b <= 0x7ff0000000000000ll;
 }
 
+// x != 0 by the bit pattern (+-0 are zero), off the FP64 pipe
+__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
+__device__ __forceinline__ bool nonzero(float x) { return x != 0.0f; }
+
+// The slab constants in R (see SlabDesc).
+template <typename R>
+__device__ __forceinline__ R slab_inv_dx(const SlabDesc& sd) {
+    if constexpr (std::is_same<R, float>::value) return sd.inv_dx_f;
+    else return sd.inv_dx;
+}
+template <typename R>
+__device__ __forceinline__ R slab_dt(const SlabDesc& sd) {
+    if constexpr (std::is_same<R, float>::value) return sd.dt_f;
+    else return sd.dt;
+}
+template <typename R>
+__device__ __forceinline__ R slab_weno_eps(const SlabDesc& sd) {
+    if constexpr (std::is_same<R, float>::value) return sd.weno_eps_f;
+    else return sd.weno_eps;
+}
+
 // Global load of data that other CTAs of the same launch may have written
 // (CG: cached in L2 only, never a stale L1 line), or an ordinary load.
 template <bool CG, typename T>
@@ -924,7 +945,7 @@ __device__ void faces(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, 
     const int nruns = (nf + kRun - 1) / kRun;
     TableLayout L(Q);
     const R* xi = rtab + sd.tab_off + L.xi;
-    const R eps = (R)sd.weno_eps;
+    const R eps = slab_weno_eps<R>(sd);
     for (int e = tid; e < rows * nruns; e += nth) {
         const int r = e % rows, run = e / rows;
         const int k = r % Q;
@@ -1172,8 +1193,8 @@ __device__ __forceinline__ double moment_sum(int which, int Q, const R* h, long 
                 G, [&](int g) { return 2 * g + 1 < H ? __dadd_rn(term(2 * g), term(2 * g + 1)) : term(2 * g); });
         }
         auto term = [&](int j) { return pair_term_f32(which, j, Q, ha(j), hb(j), xr); };
-        return (double)sum_chains4<float>(
-            G, [&](int g) { return 2 * g + 1 < H ? __fadd_rn(term(2 * g), term(2 * g + 1)) : term(2 * g); });
+        return f2d_bits(sum_chains4<float>(
+            G, [&](int g) { return 2 * g + 1 < H ? __fadd_rn(term(2 * g), term(2 * g + 1)) : term(2 * g); }));
     }
 }
 

@@ -97,6 +97,14 @@ struct SlabDesc {
     double eta_coef;     // pi sigma^3 / 6
     double mu0_coef;     // 5 / (16 sigma^2 sqrt(pi)), Eq. (viscosity)
     double T_iso;        // > 0: node fields formed at this temperature (isothermal mode)
+    // inv_dx, dt and weno_eps rounded to FP32 on the host: a conversion
+    // instruction of the FP32 stage would run on the FP64 pipe, once per warp
+    float inv_dx_f, dt_f, weno_eps_f;
+    void round_f32() {
+        inv_dx_f = (float)inv_dx;
+        dt_f = (float)dt;
+        weno_eps_f = (float)weno_eps;
+    }
 };
 
 // One CTA's share of work: nodes [i0, i0 + nz) of slab `slab`.

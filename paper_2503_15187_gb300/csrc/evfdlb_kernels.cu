@@ -67,7 +67,7 @@ __device__ __forceinline__ void stage_body(const SlabDesc& sd, const WorkItem& i
                                            const double* __restrict__ taps, const R* __restrict__ rtaps,
                                            const R* src, const R* base, R* out, double* rhs_out,
                                            const double* mom_in, double* mom_out, double* fields_out,
-                                           long long NF, long long NN, double alpha, double beta, int mode, int Z,
+                                           long long NF, long long NN, R alpha, R beta, int mode, int Z,
                                            unsigned* err) {
     const int Q = sd.Q, W = Z + 6, nz = it.nz;
     Smem<R> s = carve<R>(smem, Q, Z, sd.M);
@@ -164,8 +164,8 @@ __device__ __forceinline__ void stage_body(const SlabDesc& sd, const WorkItem& i
 
     // Phase 5: synthesis, advection, relaxation and the RK stage.
     const R* xi = rt + L.xi;
-    const R dt = (R)sd.dt, inv_dx = (R)sd.inv_dx, ralpha = (R)alpha, rbeta = (R)beta;
-    const bool rhs_form = (mode == 1), with_base = (alpha != 0.0);
+    const R dt = slab_dt<R>(sd), inv_dx = slab_inv_dx<R>(sd), ralpha = alpha, rbeta = beta;
+    const bool rhs_form = (mode == 1), with_base = nonzero(alpha);
     // The stage out = alpha base + beta (h + dt R) with
     // R = -xi_k/dx (f_{t+1/2} - f_{t-1/2}) - nu h + syn is formed as
     // fma(cx_k, df, fma(cs, syn, fma(ch, h, alpha base))): cs = beta dt,
@@ -345,7 +345,7 @@ __device__ __forceinline__ void stage_body(const SlabDesc& sd, const WorkItem& i
             const int which = e / nz, t = e - which * nz;
             double v;
             if (which == MOM_S3 || which == MOM_G1)
-                v = (double)sum_pair_terms<float>(s.Mp32 + (which == MOM_S3 ? 0 : blk) + t, G, Z);
+                v = f2d_bits(sum_pair_terms<float>(s.Mp32 + (which == MOM_S3 ? 0 : blk) + t, G, Z));
             else
                 v = sum_pair_terms<double>(s.Mp64 + (which == MOM_G0 ? 3 : which) * blk + t, G, Z);
             mom_out[which * NN + sd.node_off + it.i0 + t] = v;
@@ -362,7 +362,7 @@ stage_kernel(const SlabDesc* __restrict__ slabs, const WorkItem* __restrict__ it
              const double* __restrict__ taps, const R* __restrict__ rtaps,
              const R* __restrict__ src, const R* base, R* out, double* rhs_out,
              const double* __restrict__ mom_in, double* __restrict__ mom_out,
-             long long NF, long long NN, double alpha, double beta, int mode, int Z, unsigned* err) {
+             long long NF, long long NN, R alpha, R beta, int mode, int Z, unsigned* err) {
     extern __shared__ __align__(16) double smem[];
     const WorkItem it = items[blockIdx.x];
     const SlabDesc sd = slabs[it.slab];
@@ -845,11 +845,11 @@ void launch_stage_p(int prec, int nitems, size_t smem, cudaStream_t st, const Sl
         if (nitems <= sm_count())
             launch_pdl(stage_kernel<float>, nitems, StageThreads<float>::value, smem, st, slabs, items, tables,
                        (const float*)rtab, taps, (const float*)rtaps, (const float*)src, (const float*)base,
-                       (float*)out, rhs_out, mom_in, mom_out, NF, NN, alpha, beta, mode, Z, err);
+                       (float*)out, rhs_out, mom_in, mom_out, NF, NN, (float)alpha, (float)beta, mode, Z, err);
         else
             launch_pdl(stage_kernel<float, false, 256>, nitems, 256, smem, st, slabs, items, tables,
                        (const float*)rtab, taps, (const float*)rtaps, (const float*)src, (const float*)base,
-                       (float*)out, rhs_out, mom_in, mom_out, NF, NN, alpha, beta, mode, Z, err);
+                       (float*)out, rhs_out, mom_in, mom_out, NF, NN, (float)alpha, (float)beta, mode, Z, err);
     } else
         launch_stage_fp64(nitems, smem, st, slabs, items, tables, (const double*)rtab, taps, (const double*)rtaps,
                           (const double*)src, (const double*)base, (double*)out, rhs_out, mom_in, mom_out, NF, NN,
