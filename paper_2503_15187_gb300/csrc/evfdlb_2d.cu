@@ -21,11 +21,11 @@
 //   k2_fields   node fields per 16x16 node tile (force disc, FM average, chi,
 //               gradients, transport) and the polynomial coefficients of the
 //               equilibria;
-//   k2_coll     per group of 8 nodes, all Q^2 velocities: separable Hermite
-//               analysis, coefficients (equilibria + force), separable
-//               synthesis; writes the local part -nu h + sum S c;
-//   k2_adv      per 32x16 node tile and 8 velocity planes: WENO-5 faces along
-//               x and y, the full right-hand side and the Shu-Osher combine.
+//   k2_coll     per group of 16 nodes, all Q^2 velocities: force and collision
+//               in velocity space, written with the Runge-Kutta base as the
+//               stage's local increment V into the stage's output;
+//   k2_adv      per 32x32 node tile and a run of velocities: WENO-5 faces along
+//               x and y, added to V and the input in place.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <string.h>
@@ -52,13 +52,38 @@ struct Slab2 {
 // the host.  An FP32 kernel that takes them as doubles converts them on the
 // FP64 pipe, and the compiler forms such conversions (and a compare of a
 // double stage weight) again inside the plane loop instead of holding their
-// results: they kept that pipe 65 % busy in k2_adv2.
+// results: they kept that pipe 65 % busy in the FP32 advection.
 template <typename R>
 struct Par2 {
-    R inv_dx, k12, dt, weno_eps, b, eta_coef, mu0_coef;   // k12 = 1 / (12 dx)
-    R alpha, beta;                                         // Shu-Osher weights of the stage (k2_adv, k2_adv2)
+    R k12, weno_eps, b, eta_coef, mu0_coef;               // k12 = 1 / (12 dx)
+    // one Shu-Osher stage alpha base + beta (h + dt R) in increment form,
+    //   h + (V + ca (xi_x df_x + xi_y df_y)),  V = alpha (base - h) + cb RL
+    // (alpha + beta = 1): cb = beta dt, ca = -beta dt / dx.  The right-hand
+    // side itself is cb = 1, ca = -1 / dx without h.
+    R alpha, cb, ca, hs;                                   // hs: 1 for a stage, 0 for a right-hand side
     int with_base;                                         // alpha != 0
 };
+
+// The 2D state interleaves the distributions: pair (F, G) of velocity k at
+// node i is element k N + i of an R2 array, so that every kernel moves both
+// with one 8-byte (FP32) or 16-byte (FP64) access.
+template <typename R>
+using Pair = typename std::conditional<std::is_same<R, float>::value, float2, double2>::type;
+
+// Arithmetic on pairs: FP32 in packed instructions (two lanes each; one may
+// take a literal for both), FP64 componentwise.
+__device__ __forceinline__ float2 splat(float a) { return make_float2(a, a); }
+__device__ __forceinline__ double2 splat(double a) { return make_double2(a, a); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ double2 add2(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, splat(-1.f), a); }
+__device__ __forceinline__ double2 sub2(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ double2 mul2(double2 a, double2 b) { return make_double2(a.x * b.x, a.y * b.y); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ double2 fma2(double2 a, double2 b, double2 c) {
+    return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
+}
 
 // raw moment sums per node ([kNumMom2][N], FP64)
 enum { M2_S0 = 0, M2_S1X, M2_S1Y, M2_S2XX, M2_S2YY, M2_G0, M2_S2XY, M2_S3X, M2_S3Y, M2_G1X, M2_G1Y, kNumMom2 };
@@ -69,9 +94,7 @@ enum { F2_N = 0, F2_UX, F2_UY, F2_T, F2_NU, F2_FX, F2_FY, F2_PF = 7, F2_PG = 17,
 
 constexpr int kTile2 = 16;     // k2_fields tile edge
 constexpr int kNB = 16;        // nodes per k2_coll CTA (half a warp: a lane per node and distribution)
-static_assert(kNB == 16, "k2_coll maps the 32 lanes of a warp to 2 distributions x 16 nodes");
-constexpr int kAdvX = 32, kAdvY = 16, kAdvPlanes = 8;
-static_assert(kAdvX == 32 && kAdvY % 8 == 0, "k2_adv maps a warp (256 threads per CTA) to tile rows");
+static_assert(kNB == 16, "k2_coll maps the 32 lanes of a warp to 16 nodes x 2 distributions");
 
 __device__ __forceinline__ int wrapi(int i, int n) {
     int r = i % n;
@@ -153,18 +176,29 @@ struct MomPart {
 constexpr int kMomX = 17;                    // values exchanged between the halves
 
 template <typename R, int Q, int K0>
-__device__ __forceinline__ void moments_half(const R* __restrict__ f, long long N, long long NF, const Pow2<R>& pw,
+__device__ __forceinline__ void moments_half(const Pair<R>* __restrict__ f, long long N, const Pow2<R>& pw,
                                              const R (*sv)[Q], const float (*sh)[Q], MomPart<R>& P) {
     constexpr bool F32 = std::is_same<R, float>::value;
     constexpr int QH = Q / 2;
     CompSum<R> col[QH];
+    // the next row's loads are in flight while a row is summed
+    Pair<R> hn[QH];
+#pragma unroll
+    for (int j = 0; j < QH; ++j) hn[j] = f[(long long)(K0 + j) * N];
     for (int kx = 0; kx < Q; ++kx) {
         CompSum<R> rowF, rowG;
         R p1 = 0, p2 = 0, p3 = 0, pg = 0;          // sum y f, y^2 f, y^3 f, y g over the half row
+        Pair<R> hc[QH];
+#pragma unroll
+        for (int j = 0; j < QH; ++j) hc[j] = hn[j];
+        if (kx + 1 < Q) {
+            const Pair<R>* q = f + (long long)((kx + 1) * Q + K0) * N;
+#pragma unroll
+            for (int j = 0; j < QH; ++j) hn[j] = q[j * N];
+        }
 #pragma unroll
         for (int j = 0; j < QH; ++j) {
-            const long long o = (long long)(kx * Q + K0 + j) * N;
-            const R fv = f[o], gv = f[NF + o];
+            const R fv = hc[j].x, gv = hc[j].y;
             rowF.add(fv);
             rowG.add(gv);
             col[j].add(fv);
@@ -209,10 +243,10 @@ __device__ __forceinline__ void moments_half(const R* __restrict__ f, long long 
     }
 }
 
-// FP32: four CTAs per SM keep more loads in flight; the FP64 build (parity
-// checks) keeps its registers
+// FP32: three CTAs per SM, with the registers of two rows of loads; the FP64
+// build (parity checks) keeps its registers
 template <typename R>
-constexpr int moments_min_blocks() { return std::is_same<R, float>::value ? 4 : 1; }
+constexpr int moments_min_blocks() { return std::is_same<R, float>::value ? 3 : 1; }
 
 // Per CTA pass 128 nodes: warp pair (2p, 2p+1) takes nodes 32p .. 32p+31,
 // the even warp the y velocities of the first half, the odd warp the second
@@ -220,12 +254,12 @@ constexpr int moments_min_blocks() { return std::is_same<R, float>::value ? 4 : 
 // odd warp hands its partial sums to the even one through shared memory.
 template <typename R, int Q>
 __global__ void __launch_bounds__(256, moments_min_blocks<R>())
-k2_moments(Slab2 s, const Pow2<R> pw, const R* __restrict__ st, double* __restrict__ mom, float* __restrict__ prf,
+k2_moments(Slab2 s, const Pow2<R> pw, const Pair<R>* __restrict__ st, double* __restrict__ mom, float* __restrict__ prf,
            unsigned* err) {
     constexpr bool F32 = std::is_same<R, float>::value;
     constexpr int kNodes = 128;
     static_assert(Q % 2 == 0, "the y velocities split in two halves");
-    const long long N = s.N, NF = (long long)Q * Q * N;
+    const long long N = s.N;
     // the row loop indexes the powers at run time: from shared memory
     __shared__ R sv[2][Q];
     __shared__ float sh[4][Q];
@@ -246,8 +280,8 @@ k2_moments(Slab2 s, const Pow2<R> pw, const R* __restrict__ st, double* __restri
         const long long i = b0 + slot;
         MomPart<R> P;
         if (i < N) {
-            if (half == 0) moments_half<R, Q, 0>(st + i, N, NF, pw, sv, sh, P);
-            else moments_half<R, Q, Q / 2>(st + i, N, NF, pw, sv, sh, P);
+            if (half == 0) moments_half<R, Q, 0>(st + i, N, pw, sv, sh, P);
+            else moments_half<R, Q, Q / 2>(st + i, N, pw, sv, sh, P);
         }
         if (half == 1) {
             R v[kMomX];
@@ -583,62 +617,141 @@ k2_fields(Slab2 s, const Par2<R> pr, const double* __restrict__ mom, const float
 // (Q/2)^2 blocks instead of Q^2 products per line, and a synthesis is
 // (S c)_k = e_k + o_k, (S c)_{Q-1-k} = e_k - o_k over the even and odd orders.
 //
-// Work layout: a lane owns one (distribution, node) pair -- the 32 lanes of
-// a warp are the 2 x 16 pairs of the group -- and the state sits plane-major
-// in shared memory (16 nodes of a plane contiguous, staged by 16-byte
-// asynchronous copies), so a warp's shared accesses are conflict-free and its
-// global stores are 16 consecutive nodes of one plane per distribution.  A
-// warp takes velocity rows w, w + 8, ... (then columns): a line of Q values
-// is loaded, split into E and O and multiplied by DA and DB, whose entries
-// sit in the constant bank -- uniform across the warp at compile-time
-// indices, they are operands of the multiply-adds, with no load instructions
-// (the syntheses of phi and chi use S from the constant bank the same way).
+// Work layout: a half-warp owns one line (velocity row, then column) of the
+// group's 16 nodes, a lane the (F, G) pairs of its node, and the state sits
+// plane-major in shared memory (the 16 nodes of a plane in 128 bytes), so
+// shared accesses are conflict-free and global accesses whole lines.  A line
+// of Q pairs is loaded, split into E and O and multiplied by DA and DB, whose
+// entries are literals of the packed multiply-adds: half the instructions of
+// scalar arithmetic, and none to fetch the matrices.
 //   pass 1 (rows, D along y):  Y = -nu h + F_y (I (x) D) h + sum_b pr_b chi^b
-//   pass 2 (columns, along x): RL = Y + F_x (D (x) I) h, to global memory.
+//   pass 2 (columns, along x): RL = Y + F_x (D (x) I) h, and to global
+//   memory the stage's local increment V = alpha (base - h) + cb RL, where the
+//   advection adds its part in place (base may be the output itself: every
+//   element is read and written by the same thread).
 // ---------------------------------------------------------------------------
-// per even Q of the 2D model (4 .. 16), at coll_coff(Q): DA, DB [(Q/2)^2
-// each], then S [Q][Q] (S[k][l] = w_k psi_l(xi_k))
+// The matrices of one Q: DA, DB [(Q/2)^2 each], then S [Q][Q] (S[k][l] = w_k
+// psi_l(xi_k)).  FP32: evaluated at compile time, so that their entries are
+// literals of the multiply-adds (a line of 16 takes 163 instructions; with
+// constant-bank entries 204, in scalar and packed arithmetic alike).  FP64: in the constant bank, at
+// coll_coff(Q), from the host's extended precision.
 __host__ __device__ constexpr int coll_coff(int Q) {
     int o = 0;
     for (int q = 4; q < Q; q += 2) o += q * q / 2 + q * q;
     return o;
 }
 constexpr int kCollConst = coll_coff(18);
-__constant__ float c_coll_f[kCollConst];
 __constant__ double c_coll_d[kCollConst];
-template <typename R>
-__device__ __forceinline__ R ccoll(int i);
-template <>
-__device__ __forceinline__ float ccoll<float>(int i) { return c_coll_f[i]; }
-template <>
-__device__ __forceinline__ double ccoll<double>(int i) { return c_coll_d[i]; }
+
+constexpr double ct_sqrt(double x) {
+    double r = x > 1.0 ? x : 1.0;
+    for (int i = 0; i < 60; ++i) r = 0.5 * (r + x / r);
+    return r;
+}
+template <int Q>
+struct CollLit {
+    float v[Q * Q / 2 + Q * Q];
+    float rec[5 * Q];   // 1/sqrt(l+1), sqrt(l/(l+1)), sqrt(l), sqrt(l(l-1)), sqrt(l(l-1)(l-2))
+    constexpr CollLit() : v{}, rec{} {
+        // orthonormal Hermite polynomials psi_0 .. psi_Q at x
+        struct Psi {
+            double p[Q + 1];
+            constexpr Psi(double x, const double* r) : p{} {
+                p[0] = 1.0;
+                p[1] = x;
+                for (int l = 1; l < Q; ++l) p[l + 1] = (x * p[l] - r[l] * p[l - 1]) / r[l + 1];
+            }
+        };
+        double r[Q + 1] = {};
+        for (int l = 0; l <= Q; ++l) r[l] = l ? ct_sqrt((double)l) : 0.0;
+        for (int l = 0; l < Q; ++l) {
+            rec[l] = (float)(1.0 / r[l + 1]);
+            rec[Q + l] = (float)(r[l] / r[l + 1]);
+            rec[2 * Q + l] = (float)r[l];
+            rec[3 * Q + l] = l >= 1 ? (float)(r[l] * r[l - 1]) : 0.f;
+            rec[4 * Q + l] = l >= 2 ? (float)(r[l] * r[l - 1] * r[l - 2]) : 0.f;
+        }
+        // the Q/2 positive roots of psi_Q, ascending: sign changes on a grid
+        // finer than their spacing, then bisection
+        double xi[Q] = {}, w[Q] = {};
+        int found = 0;
+        double a = 0.0, fa = Psi(0.0, r).p[Q];
+        for (int i = 1; found < Q / 2; ++i) {
+            const double b = 0.1 * i, fb = Psi(b, r).p[Q];
+            if ((fa < 0.0) != (fb < 0.0)) {
+                double lo = a, hi = b;
+                for (int it = 0; it < 52; ++it) {
+                    const double m = 0.5 * (lo + hi);
+                    if ((Psi(m, r).p[Q] < 0.0) == (fa < 0.0)) lo = m;
+                    else hi = m;
+                }
+                xi[Q / 2 + found] = 0.5 * (lo + hi);
+                xi[Q / 2 - 1 - found] = -0.5 * (lo + hi);
+                ++found;
+            }
+            a = b;
+            fa = fb;
+        }
+        // w_k = 1 / sum_{l<Q} psi_l(xi_k)^2 (Christoffel)
+        double ps[Q][Q] = {};
+        for (int k = 0; k < Q; ++k) {
+            const Psi p(xi[k], r);
+            double sum = 0.0;
+            for (int l = 0; l < Q; ++l) {
+                ps[k][l] = p.p[l];
+                sum += p.p[l] * p.p[l];
+            }
+            w[k] = 1.0 / sum;
+        }
+        constexpr int QH = Q / 2;
+        for (int k = 0; k < QH; ++k)
+            for (int j = 0; j < QH; ++j) {
+                double d0 = 0.0, d1 = 0.0;
+                for (int l = 1; l < Q; ++l) {
+                    const double c = w[k] * ps[k][l] * r[l];
+                    d0 += c * ps[j][l - 1];
+                    d1 += c * ps[Q - 1 - j][l - 1];
+                }
+                v[k * QH + j] = (float)(0.5 * (d0 - d1));
+                v[QH * QH + k * QH + j] = (float)(0.5 * (d0 + d1));
+            }
+        for (int k = 0; k < Q; ++k)
+            for (int l = 0; l < Q; ++l) v[2 * QH * QH + k * Q + l] = (float)(w[k] * ps[k][l]);
+    }
+};
+// entry i of the matrices of order Q (i a constant once the loops are unrolled)
+template <typename R, int Q>
+__device__ __forceinline__ R ccoll(int i) {
+    if constexpr (std::is_same<R, float>::value) {
+        static constexpr CollLit<Q> lit{};
+        return lit.v[i];
+    } else {
+        return c_coll_d[coll_coff(Q) + i];
+    }
+}
 
 template <int Q>
 struct Coll2Lay {
     static constexpr int K = Q * Q, QH = Q / 2;
-    // Xp, Yp [2][K][kNB] (+16 per distribution: the two halves of a warp on
-    // opposite bank halves); chi4 [kNB][PS] (chi^b at column k: k 4 + b; PS an
-    // odd count of 16-byte units); phi [4][PH] (phi^a_k of node n at k kNB + n;
-    // PH = 8 mod 32: the 4 a of 8 nodes on distinct banks); mu [2][Q][kNB][4]
-    // (axis, order, node, a); sc [kNumFld2][kNB]; rinv, rr, r1, r2, r3 [Q]
-    static constexpr int XD = K * kNB + 16, PS = 4 * (Q + 1), PH = Q * kNB + 8;
+    // in values: state tile [K][kNB] pairs; chi4 [kNB][PS] (chi^b at column k,
+    // twice, at k 8 + 2 b: the pair operand of both distributions; PS an odd
+    // count of 16-byte units in FP32); phi [4][PH] (phi^a_k of node n at
+    // k kNB + n; PH = 8 mod 32); mu [2][Q][kNB][4] (axis, order, node, a);
+    // sc [kNumFld2][kNB]; rinv, rr, r1, r2, r3 [Q]
+    static constexpr int XN = K * 2 * kNB, PS = 8 * Q + 4, PH = Q * kNB + 8;
+    static constexpr int CHI = kNB * PS, PHI = 4 * PH, MU = 2 * Q * kNB * 4, SC = kNumFld2 * kNB;
+    static constexpr int ONE = 2 * XN + CHI + PHI + SC + MU + 5 * Q;         // k2_coll
+    static constexpr int PIPE = 5 * XN + 2 * (CHI + PHI + SC) + MU;          // k2_coll_pipe: two buffers of
+                                                                             // what a group brings with it
 };
 
-template <typename R>
-__host__ __device__ inline size_t coll_smem_bytes(int Q) {
-    const size_t K = (size_t)Q * Q, XD = K * kNB + 16, PS = 4 * ((size_t)Q + 1), PH = (size_t)Q * kNB + 8;
-    return sizeof(R) * (4 * XD + kNB * PS + 4 * PH + 2 * (size_t)Q * kNB * 4 + kNumFld2 * kNB + 5 * (size_t)Q);
+// two consecutive pairs
+__device__ __forceinline__ void ld_pairs(const float* p, float2& a, float2& b) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    a = make_float2(v.x, v.y), b = make_float2(v.z, v.w);
 }
-
-template <typename R>
-__device__ __forceinline__ void ld4(const R* p, R& a, R& b, R& c, R& d) {
-    if constexpr (std::is_same<R, float>::value) {
-        const float4 v = *reinterpret_cast<const float4*>(p);
-        a = v.x, b = v.y, c = v.z, d = v.w;
-    } else {
-        const double2 v0 = reinterpret_cast<const double2*>(p)[0], v1 = reinterpret_cast<const double2*>(p)[1];
-        a = v0.x, b = v0.y, c = v1.x, d = v1.y;
-    }
+__device__ __forceinline__ void ld_pairs(const double* p, double2& a, double2& b) {
+    a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
 }
 
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
@@ -646,371 +759,386 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gsrc) : "memory");
 }
 
-// D h along one line of Q values hv: out[k] = sum_j D_kj hv[j]
+// D h along one line of Q pairs hv: out[k] = sum_j D_kj hv[j]
 template <typename R, int Q>
-__device__ __forceinline__ void d_line(const R (&hv)[Q], R (&out)[Q]) {
-    constexpr int QH = Q / 2, O0 = coll_coff(Q), O1 = O0 + QH * QH;
-    R E[QH], Od[QH];
+__device__ __forceinline__ void d_line(const Pair<R> (&hv)[Q], Pair<R> (&out)[Q]) {
+    constexpr int QH = Q / 2, O1 = QH * QH;
+    Pair<R> E[QH], Od[QH];
 #pragma unroll
     for (int j = 0; j < QH; ++j) {
-        E[j] = hv[j] + hv[Q - 1 - j];
-        Od[j] = hv[j] - hv[Q - 1 - j];
+        E[j] = add2(hv[j], hv[Q - 1 - j]);
+        Od[j] = sub2(hv[j], hv[Q - 1 - j]);
     }
 #pragma unroll
     for (int k = 0; k < QH; ++k) {
-        R u = R(0), v = R(0);
+        Pair<R> u = mul2(splat(ccoll<R, Q>(k * QH)), Od[0]), v = mul2(splat(ccoll<R, Q>(O1 + k * QH)), E[0]);
 #pragma unroll
-        for (int j = 0; j < QH; ++j) {
-            u = fma(ccoll<R>(O0 + k * QH + j), Od[j], u);
-            v = fma(ccoll<R>(O1 + k * QH + j), E[j], v);
+        for (int j = 1; j < QH; ++j) {
+            u = fma2(splat(ccoll<R, Q>(k * QH + j)), Od[j], u);
+            v = fma2(splat(ccoll<R, Q>(O1 + k * QH + j)), E[j], v);
         }
-        out[k] = v + u;
-        out[Q - 1 - k] = u - v;
+        out[k] = add2(v, u);
+        out[Q - 1 - k] = sub2(u, v);
     }
 }
 
 // S c for one vector of Q orders: out[k] = sum_l S_kl c[l]
 template <typename R, int Q>
 __device__ __forceinline__ void s_line(const R (&c)[Q], R (&out)[Q]) {
-    constexpr int QH = Q / 2, OS = coll_coff(Q) + 2 * QH * QH;
+    constexpr int QH = Q / 2, OS = 2 * QH * QH;
 #pragma unroll
     for (int k = 0; k < QH; ++k) {
         R e = R(0), o = R(0);
 #pragma unroll
         for (int l = 0; l < Q; l += 2) {
-            e = fma(ccoll<R>(OS + k * Q + l), c[l], e);
-            o = fma(ccoll<R>(OS + k * Q + l + 1), c[l + 1], o);
+            e = fma(ccoll<R, Q>(OS + k * Q + l), c[l], e);
+            o = fma(ccoll<R, Q>(OS + k * Q + l + 1), c[l + 1], o);
         }
         out[k] = e + o;
         out[Q - 1 - k] = e - o;
     }
 }
 
-// FP32: two CTAs per SM (85 KB of shared memory each at Q = 16); FP64: one
+// The parts of a group's work, shared by the two kernels below.  sc: the
+// group's node fields [kNumFld2][kNB]; lane = 2 n + d.
+//
+// node fields of nodes i0 .. i0 + nb - 1 (the rest benign), by threads tid, tid + nth, ...
 template <typename R>
-constexpr int coll_min_blocks() { return std::is_same<R, float>::value ? 2 : 1; }
-
-template <typename R, int Q>
-__global__ void __launch_bounds__(256, coll_min_blocks<R>())
-k2_coll(Slab2 s, const R* __restrict__ rtab, const R* __restrict__ st, const R* __restrict__ fld,
-        R* __restrict__ RL) {
-    using Lay = Coll2Lay<Q>;
-    constexpr int K = Lay::K, XD = Lay::XD, PS = Lay::PS, PH = Lay::PH, NT = 256;
-    extern __shared__ __align__(16) double smc[];
-    R* Xp = reinterpret_cast<R*>(smc);                         // [2][K][kNB] (+16 per distribution)
-    R* Yp = Xp + 2 * XD;
-    R* chi4 = Yp + 2 * XD;                                      // [kNB][PS]
-    R* phi = chi4 + kNB * PS;                                   // [4][PH]
-    R* mu = phi + 4 * PH;                                       // [2][Q][kNB][4]
-    R* sc = mu + 2 * Q * kNB * 4;                               // [kNumFld2][kNB]
-    R* rinv = sc + kNumFld2 * kNB;
-    R* rr = rinv + Q;
-    R* r1 = rr + Q;
-    R* r2 = r1 + Q;
-    R* r3 = r2 + Q;
-    const long long N = s.N, NF = (long long)K * N;
-    const long long i0 = (long long)blockIdx.x * kNB;
-    const int nb = (int)min((long long)kNB, N - i0);
-    TableLayout L(Q);
-    // the group's state, plane-major: 16-byte copies when whole aligned
-    // chunks of 4 nodes exist (N a multiple of 4, a full group), else per element
-    constexpr int CH = 16 / (int)sizeof(R);                     // elements per 16-byte chunk
-    if (nb == kNB && (N % CH) == 0) {
-        for (int e = threadIdx.x; e < 2 * K * (kNB / CH); e += NT) {
-            const int c = e % (kNB / CH), k = (e / (kNB / CH)) % K, d = e / ((kNB / CH) * K);
-            cp_async16(Xp + d * XD + k * kNB + c * CH, st + d * NF + (long long)k * N + i0 + c * CH);
-        }
-    } else {
-        for (int e = threadIdx.x; e < 2 * K * kNB; e += NT) {
-            const int n = e % kNB, k = (e / kNB) % K, d = e / (kNB * K);
-            R* dst = Xp + d * XD + k * kNB + n;
-            if (n < nb) cp_async_elem<R>(dst, st + d * NF + (long long)k * N + i0 + n);
-            else *dst = R(0);
-        }
-    }
-    cp_async_commit();
-    for (int e = threadIdx.x; e < Q; e += NT) {
-        rinv[e] = rtab[L.rinv + e];
-        rr[e] = rtab[L.rr + e];
-        r1[e] = rtab[L.r1 + e];
-        r2[e] = rtab[L.r2 + e];
-        r3[e] = rtab[L.r3 + e];
-    }
-    for (int e = threadIdx.x; e < kNumFld2 * kNB; e += NT) {
+__device__ __forceinline__ void coll_fields(const R* __restrict__ fld, long long N, long long i0, int nb, R* sc, int tid,
+                                            int nth) {
+    for (int e = tid; e < kNumFld2 * kNB; e += nth) {
         const int n = e % kNB, f = e / kNB;
         sc[e] = (n < nb) ? fld[f * N + i0 + n] : (f == F2_N || f == F2_T ? R(1) : R(0));
     }
-    __syncthreads();
-    // one-axis Gaussian moments mu^a_l, one node and axis per thread
-    if (threadIdx.x < 2 * kNB) {
-        const int n = threadIdx.x % kNB, axis = threadIdx.x / kNB;
-        const R u = sc[(axis ? F2_UY : F2_UX) * kNB + n], T = sc[F2_T * kNB + n], Tm1 = T - R(1);
-        R* out = mu + (axis * Q * kNB + n) * 4;
-        R m1v = 0, m2v = 0, m3v = 0;                            // m_{l-1}, m_{l-2}, m_{l-3}
-        R m0 = 1;                                               // m_l
-        for (int l = 0; l < Q; ++l) {
-            R* o = out + l * kNB * 4;
-            o[0] = m0;
-            o[1] = T * r1[l] * m1v;
-            o[2] = T * m0 + T * T * r2[l] * m2v;
-            o[3] = R(3) * T * T * r1[l] * m1v + T * T * T * r3[l] * m3v;
-            const R mn = fma(u * rinv[l], m0, Tm1 * rr[l] * m1v);
-            m3v = m2v;
-            m2v = m1v;
-            m1v = m0;
-            m0 = mn;
-        }
-    }
-    __syncthreads();
-    // one-axis syntheses, one vector (axis, node, a) per thread:
-    // phi^a = S mu^a(u_x) to phi, chi^b = S mu^b(u_y) to chi4
-    if (threadIdx.x < 2 * kNB * 4) {
-        const int a = threadIdx.x % 4, n = (threadIdx.x / 4) % kNB, axis = threadIdx.x / (4 * kNB);
-        R c[Q], out[Q];
-#pragma unroll
-        for (int l = 0; l < Q; ++l) c[l] = mu[((axis * Q + l) * kNB + n) * 4 + a];
-        s_line<R, Q>(c, out);
-        if (axis == 0) {
-#pragma unroll
-            for (int k = 0; k < Q; ++k) phi[a * PH + k * kNB + n] = out[k];
+}
+
+// one-axis Gaussian moments mu^a_l, one node and axis per thread (32
+// threads); rec (FP64; FP32 has literals): the recurrence constants of CollLit
+template <typename R, int Q>
+__device__ __forceinline__ void coll_mu(const R* sc, const R* rec, R* mu, int tid) {
+    auto c = [&](int which, int l) -> R {
+        if constexpr (std::is_same<R, float>::value) {
+            static constexpr CollLit<Q> lit{};
+            return lit.rec[which * Q + l];
         } else {
-#pragma unroll
-            for (int k = 0; k < Q; ++k) chi4[n * PS + k * 4 + a] = out[k];
+            return rec[which * Q + l];
         }
+    };
+    const int n = tid % kNB, axis = tid / kNB;
+    const R u = sc[(axis ? F2_UY : F2_UX) * kNB + n], T = sc[F2_T * kNB + n], Tm1 = T - R(1);
+    R* out = mu + (axis * Q * kNB + n) * 4;
+    R m1v = 0, m2v = 0, m3v = 0;                            // m_{l-1}, m_{l-2}, m_{l-3}
+    R m0 = 1;                                               // m_l
+#pragma unroll
+    for (int l = 0; l < Q; ++l) {
+        R* o = out + l * kNB * 4;
+        o[0] = m0;
+        o[1] = T * c(2, l) * m1v;
+        o[2] = T * m0 + T * T * c(3, l) * m2v;
+        o[3] = R(3) * T * T * c(2, l) * m1v + T * T * T * c(4, l) * m3v;
+        const R mn = fma(u * c(0, l), m0, Tm1 * c(1, l) * m1v);
+        m3v = m2v;
+        m2v = m1v;
+        m1v = m0;
+        m0 = mn;
     }
+}
+
+// one-axis syntheses, vector `tid` (axis, node, a) of 128:
+// phi^a = S mu^a(u_x) to phi, chi^b = S mu^b(u_y) to chi4
+template <typename R, int Q>
+__device__ __forceinline__ void coll_synth(const R* mu, R* phi, R* chi4, int tid) {
+    using Lay = Coll2Lay<Q>;
+    const int a = tid % 4, n = (tid / 4) % kNB, axis = tid / (4 * kNB);
+    R c[Q], out[Q];
+#pragma unroll
+    for (int l = 0; l < Q; ++l) c[l] = mu[((axis * Q + l) * kNB + n) * 4 + a];
+    s_line<R, Q>(c, out);
+    if (axis == 0) {
+#pragma unroll
+        for (int k = 0; k < Q; ++k) phi[a * Lay::PH + k * kNB + n] = out[k];
+    } else {
+#pragma unroll
+        for (int k = 0; k < Q; ++k) chi4[n * Lay::PS + k * 8 + 2 * a] = chi4[n * Lay::PS + k * 8 + 2 * a + 1] = out[k];
+    }
+}
+
+// pass 1 on row r (fixed kx) of node n, D along y: from X to Y
+template <typename R, int Q>
+__device__ __forceinline__ void coll_row(int r, int n, const Pair<R>* X, Pair<R>* Y, const R* sc, const R* phi,
+                                         const R* chi4) {
+    using Lay = Coll2Lay<Q>;
+    using R2 = Pair<R>;
+    const R2* h = X + r * Q * kNB + n;
+    R2* y = Y + r * Q * kNB + n;
+    R2 hv[Q], dy[Q];
+#pragma unroll
+    for (int j = 0; j < Q; ++j) hv[j] = h[j * kNB];
+    d_line<R, Q>(hv, dy);
+    const R2 mnu = splat(-sc[F2_NU * kNB + n]), fy = splat(sc[F2_FY * kNB + n]);
+    // P_ab (the equilibrium polynomials' coefficients of c_x^a c_y^b, times
+    // n) at (a+b)(a+b+1)/2 + b of the order (0,0) (1,0) (0,1) (2,0) (1,1)
+    // (0,2) (3,0) (2,1) (1,2) (0,3)
+    auto P = [&](int i) {
+        R2 p;
+        p.x = sc[(F2_PF + i) * kNB + n];
+        p.y = sc[(F2_PG + i) * kNB + n];
+        return p;
+    };
+    const R2 p0 = splat(phi[0 * Lay::PH + r * kNB + n]), p1 = splat(phi[1 * Lay::PH + r * kNB + n]);
+    const R2 p2 = splat(phi[2 * Lay::PH + r * kNB + n]), p3 = splat(phi[3 * Lay::PH + r * kNB + n]);
+    // pr_b = sum_{a <= 3-b} phi^a_r P_ab
+    const R2 pr0 = fma2(p3, P(6), fma2(p2, P(3), fma2(p1, P(1), mul2(p0, P(0)))));
+    const R2 pr1 = fma2(p2, P(7), fma2(p1, P(4), mul2(p0, P(2))));
+    const R2 pr2 = fma2(p1, P(8), mul2(p0, P(5)));
+    const R2 pr3 = mul2(p0, P(9));
+    const R* ch = chi4 + n * Lay::PS;
+#pragma unroll
+    for (int c = 0; c < Q; ++c) {
+        R2 q0, q1, q2, q3;
+        ld_pairs(ch + c * 8, q0, q1);
+        ld_pairs(ch + c * 8 + 4, q2, q3);
+        R2 eq = mul2(pr0, q0);
+        eq = fma2(pr1, q1, eq);
+        eq = fma2(pr2, q2, eq);
+        eq = fma2(pr3, q3, eq);
+        y[c * kNB] = fma2(fy, dy[c], fma2(mnu, hv[c], eq));
+    }
+}
+
+// pass 2 on column c (fixed ky) of node n, D along x, and the store of V at
+// g + k N; bv(k): base at plane k of this node
+template <typename R, int Q, typename B>
+__device__ __forceinline__ void coll_col(int c, int n, const Pair<R>* X, const Pair<R>* Y, const R* sc, bool wb, R cb,
+                                         R al, bool valid, Pair<R>* g, long long N, B bv) {
+    using R2 = Pair<R>;
+    const R2* h = X + c * kNB + n;
+    const R2* y = Y + c * kNB + n;
+    R2 hv[Q], dx[Q];
+#pragma unroll
+    for (int j = 0; j < Q; ++j) hv[j] = h[j * Q * kNB];
+    d_line<R, Q>(hv, dx);
+    const R2 fx = splat(sc[F2_FX * kNB + n]), cb2 = splat(cb), al2 = splat(al);
+    R2* p = g + (long long)c * N;
+#pragma unroll
+    for (int r = 0; r < Q; ++r, p += Q * N) {
+        R2 v = mul2(cb2, fma2(fx, dx[r], y[r * Q * kNB]));
+        if (wb) v = fma2(al2, sub2(bv(r * Q + c), hv[r]), v);
+        if (valid) *p = v;
+    }
+}
+
+// the group's slice of a state, [K][kNB] pairs, by asynchronous copies: 16
+// bytes where they stay aligned in every plane, else one pair at a time
+template <typename R, int Q>
+__device__ __forceinline__ void coll_issue(Pair<R>* dst, const Pair<R>* st, long long N, long long i0, int nb, int tid,
+                                           int nth) {
+    constexpr int K = Q * Q, CH = 16 / (int)sizeof(Pair<R>), CPP = kNB / CH;   // pairs per copy, copies per plane
+    if (CH == 1 || (N & 1) == 0) {                                             // (FP32: nb is even here)
+        const int n = (tid % CPP) * CH;                                        // nth is a multiple of CPP
+        const Pair<R>* g = st + i0 + n;
+        if (n < nb)
+            for (int k = tid / CPP; k < K; k += nth / CPP) cp_async16(dst + k * kNB + n, g + (long long)k * N);
+    } else {
+        const int n = tid % kNB;
+        const Pair<R>* g = st + i0 + n;
+        if (n < nb)
+            for (int k = tid / kNB; k < K; k += nth / kNB)
+                cp_async_elem<double>(reinterpret_cast<double*>(dst + k * kNB + n),
+                                      reinterpret_cast<const double*>(g + (long long)k * N));
+    }
+    cp_async_commit();
+}
+
+template <typename R, int Q>
+__device__ __forceinline__ void coll_tables(const R* __restrict__ rtab, R* rec, int tid, int nth) {
+    TableLayout L(Q);
+    for (int e = tid; e < Q; e += nth) {
+        rec[e] = rtab[L.rinv + e];
+        rec[Q + e] = rtab[L.rr + e];
+        rec[2 * Q + e] = rtab[L.r1 + e];
+        rec[3 * Q + e] = rtab[L.r2 + e];
+        rec[4 * Q + e] = rtab[L.r3 + e];
+    }
+}
+
+// One group per CTA, its phases in sequence: the FP64 build (whose two state
+// buffers and prefetches would not fit).
+template <typename R, int Q>
+__global__ void __launch_bounds__(256, 1)
+k2_coll(Slab2 s, const Par2<R> pr, const R* __restrict__ rtab, const Pair<R>* __restrict__ st,
+        const R* __restrict__ fld, const Pair<R>* base, Pair<R>* V) {
+    using Lay = Coll2Lay<Q>;
+    constexpr int NT = 256;
+    extern __shared__ __align__(16) double smc[];
+    R* chi4 = reinterpret_cast<R*>(smc) + 2 * Lay::XN;
+    Pair<R>* X = reinterpret_cast<Pair<R>*>(smc);
+    Pair<R>* Y = X + Lay::XN / 2;
+    R* phi = chi4 + Lay::CHI;
+    R* sc = phi + Lay::PHI;
+    R* mu = sc + Lay::SC;
+    R* rec = mu + Lay::MU;
+    const long long N = s.N, i0 = (long long)blockIdx.x * kNB;
+    const int nb = (int)min((long long)kNB, N - i0), tid = threadIdx.x;
+    coll_issue<R, Q>(X, st, N, i0, nb, tid, NT);
+    coll_tables<R, Q>(rtab, rec, tid, NT);
+    coll_fields<R>(fld, N, i0, nb, sc, tid, NT);
+    __syncthreads();
+    if (tid < 2 * kNB) coll_mu<R, Q>(sc, rec, mu, tid);
+    __syncthreads();
+    if (tid < 2 * kNB * 4) coll_synth<R, Q>(mu, phi, chi4, tid);
     cp_async_wait_all();
     __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int d = lane >> 4, n = lane & (kNB - 1);
-    const R* h = Xp + d * XD + n;                               // h[k] at k kNB
-    R* y = Yp + d * XD + n;
-    // pass 1: rows r (fixed kx), D along y
-    {
-        const R mnu = -sc[F2_NU * kNB + n], fy = sc[F2_FY * kNB + n];
-        // P^d_ab (the equilibrium polynomial's coefficient of c_x^a c_y^b,
-        // times n) at (a+b)(a+b+1)/2 + b of the order (0,0) (1,0) (0,1)
-        // (2,0) (1,1) (0,2) (3,0) (2,1) (1,2) (0,3)
-        R P[10];
-        const int f0 = d ? F2_PG : F2_PF;
-#pragma unroll
-        for (int i = 0; i < 10; ++i) P[i] = sc[(f0 + i) * kNB + n];
-        const R* ch = chi4 + n * PS;
-        for (int r = warp; r < Q; r += NT / 32) {
-            R hv[Q], dy[Q];
-#pragma unroll
-            for (int j = 0; j < Q; ++j) hv[j] = h[(r * Q + j) * kNB];
-            d_line<R, Q>(hv, dy);
-            const R p0 = phi[0 * PH + r * kNB + n], p1 = phi[1 * PH + r * kNB + n];
-            const R p2 = phi[2 * PH + r * kNB + n], p3 = phi[3 * PH + r * kNB + n];
-            // pr_b = sum_{a <= 3-b} phi^a_r P_ab
-            const R pr0 = fma(p3, P[6], fma(p2, P[3], fma(p1, P[1], p0 * P[0])));
-            const R pr1 = fma(p2, P[7], fma(p1, P[4], p0 * P[2]));
-            const R pr2 = fma(p1, P[8], p0 * P[5]);
-            const R pr3 = p0 * P[9];
-#pragma unroll
-            for (int c = 0; c < Q; ++c) {
-                R q0, q1, q2, q3;
-                ld4<R>(ch + c * 4, q0, q1, q2, q3);
-                R eq = pr0 * q0;
-                eq = fma(pr1, q1, eq);
-                eq = fma(pr2, q2, eq);
-                eq = fma(pr3, q3, eq);
-                const R v = fma(mnu, hv[c], eq);
-                y[(r * Q + c) * kNB] = fma(fy, dy[c], v);
-            }
-        }
-    }
+    const int n = tid % kNB, line = tid / kNB;          // a half-warp per row (column)
+    if (line < Q) coll_row<R, Q>(line, n, X, Y, sc, phi, chi4);
     __syncthreads();
-    // pass 2: columns c (fixed ky), D along x, and the store
-    {
-        const R fx = sc[F2_FX * kNB + n];
-        R* g = RL + d * NF + i0 + n;
-        for (int c = warp; c < Q; c += NT / 32) {
-            R hv[Q], dx[Q];
-#pragma unroll
-            for (int j = 0; j < Q; ++j) hv[j] = h[(j * Q + c) * kNB];
-            d_line<R, Q>(hv, dx);
-#pragma unroll
-            for (int r = 0; r < Q; ++r) {
-                const R v = fma(fx, dx[r], y[(r * Q + c) * kNB]);
-                if (n < nb) g[(long long)(r * Q + c) * N] = v;
-            }
-        }
-    }
+    const bool valid = n < nb;
+    const Pair<R>* bp = base + i0 + n;
+    if (line < Q)
+        coll_col<R, Q>(line, n, X, Y, sc, pr.with_base != 0, pr.cb, pr.alpha, valid, V + i0 + n, N,
+                       [&](int k) { return valid ? bp[(long long)k * N] : splat(R(0)); });
 }
 
-// ---------------------------------------------------------------------------
-// k2_adv: WENO-5 faces along x and y, the right-hand side and the RK combine.
-// ---------------------------------------------------------------------------
-// A 32x16 node tile and a run of velocity planes.  Per plane the halo (tile
-// +-3) is staged in shared memory (its global offsets computed once per CTA),
-// then every thread forms one run of consecutive faces with the difference-
-// form WENO-5 of the 1D kernels (Weno5Run: the differences and the t-terms of
-// each cell formed once and shared by the run's faces): threads 0-127 the x
-// faces (16 rows x runs 5+4+4+4+4+4+4+4 of the 33 faces of a row), threads
-// 128-255 the y faces (32 columns x runs 5+4+4+4 of the 17 faces of a
-// column); for a negative velocity the stencil is mirrored and the run walked
-// down.  Then the right-hand side and the Shu-Osher combine
-//   out = alpha base + beta (h + dt R)   (RHS false),   rhs_out = R (RHS true).
-// Q is a compile-time parameter: the plane index splits by constants.  So is
-// the output form: with a run-time switch the FP32 kernel issued the FP64
-// store's conversion (predicated off) for every output of the combine.
-template <typename R>
-constexpr int adv_min_blocks() { return std::is_same<R, float>::value ? 4 : 2; }
-
-template <typename R, int Q, bool RHS>
-__global__ void __launch_bounds__(256, adv_min_blocks<R>())
-k2_adv(Slab2 s, const Par2<R> pr, const R* __restrict__ rtab, const R* __restrict__ src, const R* base, R* out,
-       const R* __restrict__ RL, double* rhs_out) {
-    constexpr int WX = kAdvX + 6, WY = kAdvY + 6, NH = WX * WY;
-    constexpr int NHR = (NH + 255) / 256;                   // halo loads per thread
-    constexpr int RPW = kAdvY / 8;                          // output rows per warp
-    constexpr int K = Q * Q;
-    static_assert(kAdvX == 32 && kAdvY == 16, "run split: 33 = 5 + 7 x 4 x-faces, 17 = 5 + 3 x 4 y-faces");
-    __shared__ R Hs[NH];
-    __shared__ R FX[kAdvY * (kAdvX + 1)];
-    __shared__ R FY[(kAdvY + 1) * kAdvX];
-    __shared__ int rowoff[WY];
-    __shared__ int coloff[WX];
-    const int nx = s.nx, ny = s.ny;
+// The FP32 form: a resident CTA walks the groups blockIdx.x, + gridDim.x, ...
+// with everything of the next group in preparation while it forms this one:
+//  - its state and base slices (32 KB each at Q = 16) by asynchronous copies
+//    issued a whole group ahead;
+//  - its node fields, Gaussian moments and one-axis syntheses by four extra
+//    warps (the serial recurrence of coll_mu would idle a CTA that formed it
+//    in sequence; with the field loads in that sequence too the preparation
+//    was the longer side: 296 us).
+// Q/2 warps take two velocity rows, then two columns, of each group, F and G
+// in packed arithmetic.
+// Bound by DRAM: 172 us at 384^2, Q 16, 5.3 TB/s with the base (24 bytes per
+// pair).  Two CTAs per SM that ran load, moments and passes in sequence, in
+// scalar arithmetic on constant-bank matrices, took 210 us without the base
+// (and 400 us with it read where it is used).
+constexpr int kCollPrep = 128;               // threads of the preparing warps
+template <int Q>
+constexpr int coll_threads() { return kNB * Q + kCollPrep; }
+template <int Q>
+__global__ void __launch_bounds__(coll_threads<Q>(), 1)
+k2_coll_pipe(Slab2 s, const Par2<float> pr, const float2* __restrict__ st, const float* __restrict__ fld,
+             const float2* base, float2* V, int groups) {
+    using Lay = Coll2Lay<Q>;
+    constexpr int NC = kNB * Q, XP = Lay::XN / 2;          // computing threads, pairs of a slice
+    extern __shared__ __align__(16) double smc[];
+    float2* X = reinterpret_cast<float2*>(smc);            // [2][XP]
+    float2* B = X + 2 * XP;                                // [2][XP]
+    float2* Y = B + 2 * XP;
+    float* chi4 = reinterpret_cast<float*>(Y + XP);        // [2][CHI]
+    float* phi = chi4 + 2 * Lay::CHI;                      // [2][PHI]
+    float* sc = phi + 2 * Lay::PHI;                        // [2][SC]
+    float* mu = sc + 2 * Lay::SC;
     const long long N = s.N;
-    const int tilesx = (nx + kAdvX - 1) / kAdvX;
-    const int x0 = (blockIdx.x % tilesx) * kAdvX, y0 = (blockIdx.x / tilesx) * kAdvY;
-    TableLayout L(Q);
-    // wrapped halo coordinates, shared by every plane of this tile (node
-    // offsets fit 32 bits: the 2D context holds fewer than 2^31 nodes)
-    for (int e = threadIdx.x; e < WY + WX; e += blockDim.x) {
-        if (e < WY) rowoff[e] = wrapi(y0 - 3 + e, ny) * nx;
-        else coloff[e - WY] = wrapi(x0 - 3 + (e - WY), nx);
-    }
-    __syncthreads();
-    int hoff[NHR];
-#pragma unroll
-    for (int j = 0; j < NHR; ++j) {
-        const int e = threadIdx.x + 256 * j;
-        hoff[j] = (e < NH) ? rowoff[e / WX] + coloff[e % WX] : 0;
-    }
-    const R eps = pr.weno_eps, idx = pr.inv_dx, dt = pr.dt, ralpha = pr.alpha, rbeta = pr.beta;
-    const bool with_base = pr.with_base != 0;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // this thread's run of faces: along x (threads 0-127) or y (128-255)
-    const bool xrun = threadIdx.x < 128;
-    const int rj = xrun ? (threadIdx.x >> 4) : ((threadIdx.x - 128) >> 5);   // run index
-    const int rl = xrun ? (threadIdx.x & 15) : (threadIdx.x & 31);           // row (x) or column (y)
-    const int fa = rj == 0 ? 0 : 4 * rj + 1, nrun = rj == 0 ? 5 : 4, fl = fa + nrun - 1;
-    const int hst = xrun ? 1 : WX;                        // halo stride along the run
-    // x face f of row r: stencil from halo (r + 3, f); y face f of column c: from halo (f, c + 3)
-    const R* hrow = xrun ? Hs + (rl + 3) * WX : Hs + rl + 3;
-    R* frow = xrun ? FX + rl * (kAdvX + 1) : FY + rl;
-    const int fst = xrun ? 1 : kAdvX;                     // face stride along the run
-    // output nodes of this thread (rows warp*RPW + rr, column lane) and
-    // their offsets in a velocity plane
-    const int x = x0 + lane;
-    int ooff[RPW];
-    bool oval[RPW];
-#pragma unroll
-    for (int rr = 0; rr < RPW; ++rr) {
-        const int y = y0 + warp * RPW + rr;
-        oval[rr] = (x < nx && y < ny);
-        ooff[rr] = oval[rr] ? y * nx + x : 0;
-    }
-    const int p0 = blockIdx.y * kAdvPlanes, p1 = min(p0 + kAdvPlanes, 2 * K);
-    // plane p (distribution p / K, velocity p % K) starts at p N: the plane
-    // pointers advance by N (no 64-bit products in the loop)
-    const long long off0 = (long long)p0 * N;
-    const R* hp = src + off0;
-    const R* rlp = RL + off0;
-    const R* bsp = base + off0;
-    R* op = out + off0;
-    double* rp = rhs_out ? rhs_out + off0 : nullptr;
-    // the halo of the next plane is loaded into registers while this plane's
-    // faces are formed, and this plane's RL / base values before them
-    R hn[NHR];
-#pragma unroll
-    for (int j = 0; j < NHR; ++j) hn[j] = (threadIdx.x + 256 * j < NH) ? hp[hoff[j]] : R(0);
-    for (int plane = p0; plane < p1; ++plane, hp += N, rlp += N, bsp += N, op += N) {
-        const int k = plane % K;
-        const R vx = rtab[L.xi + k / Q], vy = rtab[L.xi + k % Q];
-        __syncthreads();   // previous plane's faces and halo consumed
-#pragma unroll
-        for (int j = 0; j < NHR; ++j)
-            if (threadIdx.x + 256 * j < NH) Hs[threadIdx.x + 256 * j] = hn[j];
-        if (plane + 1 < p1) {
-            const R* hq = hp + N;
-#pragma unroll
-            for (int j = 0; j < NHR; ++j)
-                if (threadIdx.x + 256 * j < NH) hn[j] = hq[hoff[j]];
+    const int tid = threadIdx.x;
+    const bool wb = pr.with_base != 0;
+    auto nodes_of = [&](int g) { return (int)min((long long)kNB, N - (long long)g * kNB); };
+    if (tid < NC) {
+        auto issue = [&](int g, int b) {
+            const long long i0 = (long long)g * kNB;
+            coll_issue<float, Q>(X + b * XP, st, N, i0, nodes_of(g), tid, NC);
+            if (wb) coll_issue<float, Q>(B + b * XP, base, N, i0, nodes_of(g), tid, NC);
+        };
+        issue(blockIdx.x, 0);
+        const int n = tid % kNB, line = tid / kNB;
+        for (int g = blockIdx.x, b = 0; g < groups; g += gridDim.x, b ^= 1) {
+            cp_async_wait_all();
+            __syncthreads();                 // group g staged and prepared, group g - 1 done
+            if (g + (int)gridDim.x < groups) issue(g + gridDim.x, b ^ 1);
+            const float2* x = X + b * XP;
+            const float* scb = sc + b * Lay::SC;
+            coll_row<float, Q>(line, n, x, Y, scb, phi + b * Lay::PHI, chi4 + b * Lay::CHI);
+            asm volatile("bar.sync 1, %0;" ::"n"(NC) : "memory");
+            const float2* bb = B + b * XP + n;
+            coll_col<float, Q>(line, n, x, Y, scb, wb, pr.cb, pr.alpha, n < nodes_of(g), V + (long long)g * kNB + n, N,
+                               [&](int k) { return bb[k * kNB]; });
         }
-        R rl[RPW], bs[RPW];
+    } else {
+        // the fields of the group after the next are in flight meanwhile
+        constexpr int NV = (Lay::SC + kCollPrep - 1) / kCollPrep;
+        const int t = tid - NC, n = t % kNB;
+        const int step = gridDim.x;
+        float v[NV];
+        auto load = [&](int g) {
+            const bool in = g < groups && n < nodes_of(g);
 #pragma unroll
-        for (int rr = 0; rr < RPW; ++rr) {
-            rl[rr] = oval[rr] ? rlp[ooff[rr]] : R(0);
-            bs[rr] = (oval[rr] && with_base && !RHS) ? bsp[ooff[rr]] : R(0);
-        }
-        __syncthreads();
-        {
-            const bool pos = (xrun ? vx : vy) >= R(0);      // uniform per warp
-            const int dir = pos ? 1 : -1, f0 = pos ? fa : fl;
-            // v >= 0: face f uses halo f .. f+4, walked up; v < 0: f+5 .. f+1, walked down
-            const R* hb = hrow + (pos ? fa : fl + 5) * hst;
-            const int hs = dir * hst;
-            Weno5Run<R> w;
-            w.start(hb[0], hb[hs], hb[2 * hs], hb[3 * hs], hb[4 * hs], eps);
-#pragma unroll
-            for (int q = 0; q < 5; ++q) {
-                if (q >= nrun) break;
-                frow[(f0 + dir * q) * fst] = w.face();
-                if (q + 1 < nrun) w.shift(hb[(q + 5) * hs]);
+            for (int j = 0; j < NV; ++j) {
+                const int f = (t + kCollPrep * j) / kNB;
+                v[j] = (f < kNumFld2 && in) ? fld[f * N + (long long)g * kNB + n]
+                                            : (f == F2_N || f == F2_T ? 1.f : 0.f);
             }
-        }
-        __syncthreads();
+        };
+        auto sync = [] { asm volatile("bar.sync 2, %0;" ::"n"(kCollPrep) : "memory"); };
+        auto prepare = [&](int g, int b) {                   // v: the fields of group g
+            float* scb = sc + b * Lay::SC;
 #pragma unroll
-        for (int rr = 0; rr < RPW; ++rr) {
-            if (!oval[rr]) continue;
-            const int ty = warp * RPW + rr;
-            R Rv = rl[rr];
-            Rv = fma(-vx * idx, FX[ty * (kAdvX + 1) + lane + 1] - FX[ty * (kAdvX + 1) + lane], Rv);
-            Rv = fma(-vy * idx, FY[(ty + 1) * kAdvX + lane] - FY[ty * kAdvX + lane], Rv);
-            if constexpr (RHS) {
-                rp[(plane - p0) * N + ooff[rr]] = (double)Rv;
-                continue;
-            }
-            const R hv = Hs[(ty + 3) * WX + lane + 3];
-            R o = rbeta * fma(dt, Rv, hv);
-            if (with_base) o = fma(ralpha, bs[rr], o);
-            op[ooff[rr]] = o;
+            for (int j = 0; j < NV; ++j)
+                if (t + kCollPrep * j < Lay::SC) scb[t + kCollPrep * j] = v[j];
+            load(g + step);
+            sync();
+            if (t < 2 * kNB) coll_mu<float, Q>(scb, nullptr, mu, t);
+            sync();
+            coll_synth<float, Q>(mu, phi + b * Lay::PHI, chi4 + b * Lay::CHI, t);
+        };
+        load(blockIdx.x);
+        prepare(blockIdx.x, 0);
+        for (int g = blockIdx.x, b = 0; g < groups; g += step, b ^= 1) {
+            __syncthreads();
+            if (g + step < groups) prepare(g + step, b ^ 1);
         }
     }
 }
 
 // ---------------------------------------------------------------------------
-// k2_adv2: the FP32 stage form of k2_adv.  The F and G planes of one
-// velocity are carried together as float2 through packed FP32 arithmetic
-// (two lanes per instruction): both distributions share the velocity, hence
-// the upwind direction of every face, so the pair runs one stencil walk.
-// Each packed operation is the IEEE single-precision operation of each lane
-// in the order of k2_adv (k2_adv's scalar code may also fuse a product into
-// a following add, so the two agree to rounding, not bit for bit).  The
-// halo tile, RL and base of velocity k+2 are copied asynchronously into a
-// second shared buffer while velocity k is formed (two velocities in
-// flight per CTA, no register staging), which keeps enough bytes in flight
-// for the kernel to stream.
+// k2_adv: WENO-5 faces along x and y and the end of the RK stage,
+//   V <- hs h + (V + ca (xi_x df_x + xi_y df_y)),
+// hs = 1 for a stage (V the increment that k2_coll left, here completed in
+// place), 0 for a right-hand side.
+// F and G of one velocity are carried together as a pair (packed FP32
+// arithmetic, two lanes per instruction): both share the velocity, hence the
+// upwind direction of every face, so the pair runs one stencil walk.
+//
+// A CTA of four warps owns a 32x32 node tile and a run of velocities.  Per
+// velocity the halo tile (38x38 pairs) sits in shared memory; the halos of
+// the next two velocities are in flight (cp.async, three buffers).  Each
+// thread walks two runs of nine faces and keeps the face differences in
+// registers:
+//   x: lane = row, warp = 8 columns; the 8 differences go to shared memory;
+//   y: lane = column, warp = 8 rows; per face after the first the thread holds
+//      h and df_y of one node, adds the node's df_x and V and writes it.
+// So a node costs one shared store and two shared loads besides the two
+// stencil loads, two CTA barriers per velocity serve 1024 nodes, and V comes
+// by plain row loads issued before the x walk.  Any nx and ny take this path
+// (copies of single pairs from offsets formed once per CTA).  The odd row
+// pitches keep the accesses of both walks conflict-free.
+// Bound by the FMA pipe (a packed operation holds it two cycles): at 384^2, Q
+// 16, 212 us with the pipe 74 % busy and 4.2 TB/s of DRAM, 110 instructions
+// per node and velocity.  The form before (32x16 tiles, runs of four or five
+// faces, face values in shared memory, separate F and G planes, 16-byte copies
+// on aligned tiles alone) took 345 us and 241 instructions, and 376 us against
+// now 128 us on a 333x250 grid, whose rows are not 16-byte aligned.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float2 f2s(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, f2s(-1.f), a); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float rcp_ftz(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
 
-// Weno5Run on float2 pairs (its operations, lane by lane, none fused)
+// The WENO-5 walk of Weno5Run on pairs.  With g_0 = 2 s_0 - d_1,
+// g_1 = 6 (s_1 + d_2), g_2 = 3 (d_2 - s_2) (60 times the candidate
+// corrections times their linear weights) the face is
+// v2 + (sum a_r g_r) / (6 (a_0 + 6 a_1 + 3 a_2)).  The divisor is at least
+// 10 (4 eps)^4: a normal FP32 number for eps >= kFtzMinEps, where FTZ takes
+// the flushing reciprocal; below, the quotient that also covers subnormals.
+constexpr double kFtzMinEps = 1e-9;
+template <typename R, bool FTZ>
 struct Weno5Run2 {
-    float2 v2, v3, v4, d0, d1, d2, d3, u0, u1, u2, eps4;
-    __device__ __forceinline__ float2 tterm(float2 t) const {
-        return fma2(mul2(f2s(float(13.0 / 3.0)), t), t, eps4);
-    }
-    __device__ __forceinline__ void start(float2 w0, float2 w1, float2 w2, float2 w3, float2 w4, float eps) {
-        eps4 = f2s(4.f * eps);
+    using R2 = Pair<R>;
+    R2 v2, v3, v4, d0, d1, d2, d3, u0, u1, u2, eps4;
+    __device__ __forceinline__ R2 tterm(R2 t) const { return fma2(mul2(splat(R(13.0 / 3.0)), t), t, eps4); }
+    __device__ __forceinline__ void start(R2 w0, R2 w1, R2 w2, R2 w3, R2 w4, R eps) {
+        eps4 = splat(R(4) * eps);
         v2 = w2;
         v3 = w3;
         v4 = w4;
@@ -1022,21 +1150,26 @@ struct Weno5Run2 {
         u1 = tterm(sub2(d2, d1));
         u2 = tterm(sub2(d3, d2));
     }
-    __device__ __forceinline__ float2 face() const {
-        const float2 s0 = fma2(f2s(3.f), d1, neg2(d0)), s1 = add2(d1, d2), s2 = fma2(f2s(-3.f), d2, d3);
-        const float2 e0 = fma2(s0, s0, u0), e1 = fma2(s1, s1, u1), e2 = fma2(s2, s2, u2);
-        const float2 E0 = mul2(e0, e0), E1 = mul2(e1, e1), E2 = mul2(e2, e2);
-        const float2 a0 = mul2(E1, E2), a1 = mul2(E0, E2), a2 = mul2(E0, E1);
-        const float2 c0 = fma2(f2s(float(5.0 / 60.0)), d1, mul2(f2s(float(-2.0 / 60.0)), d0));
-        const float2 p2 = mul2(f2s(0.2f), d2);
-        const float2 c1 = fma2(f2s(0.1f), d1, p2);
-        const float2 c2 = fma2(f2s(-0.05f), d3, p2);
-        const float2 num = fma2(a0, c0, fma2(a1, c1, mul2(a2, c2)));
-        const float2 den = fma2(f2s(0.1f), a0, fma2(f2s(0.6f), a1, mul2(f2s(0.3f), a2)));
-        return add2(v2, make_float2(__fdividef(num.x, den.x), __fdividef(num.y, den.y)));
+    __device__ __forceinline__ R2 quotient(R2 a, R2 b) const {
+        if constexpr (std::is_same<R, double>::value) return make_double2(div_face(a.x, b.x), div_face(a.y, b.y));
+        else if constexpr (FTZ) return mul2(a, make_float2(rcp_ftz(b.x), rcp_ftz(b.y)));
+        else return make_float2(__fdividef(a.x, b.x), __fdividef(a.y, b.y));
     }
-    __device__ __forceinline__ void shift(float2 w5) {
-        const float2 d4 = sub2(w5, v4);
+    __device__ __forceinline__ R2 face() const {
+        // s_0 and the g_r with their signs turned (no negations)
+        const R2 s0 = fma2(splat(R(-3)), d1, d0), s1 = add2(d1, d2), s2 = fma2(splat(R(-3)), d2, d3);
+        const R2 e0 = fma2(s0, s0, u0), e1 = fma2(s1, s1, u1), e2 = fma2(s2, s2, u2);
+        const R2 E0 = mul2(e0, e0), E1 = mul2(e1, e1), E2 = mul2(e2, e2);
+        const R2 a0 = mul2(E1, E2), a1 = mul2(E0, E2), a2 = mul2(E0, E1);
+        const R2 g0 = fma2(splat(R(2)), s0, d1);
+        const R2 g1 = fma2(splat(R(-12)), d2, mul2(splat(R(-6)), d1));
+        const R2 g2 = fma2(splat(R(-12)), d2, mul2(splat(R(3)), d3));
+        const R2 num = fma2(a0, g0, fma2(a1, g1, mul2(a2, g2)));
+        const R2 den = fma2(splat(R(6)), a1, fma2(splat(R(3)), a2, a0));
+        return fma2(splat(R(-1.0 / 6.0)), quotient(num, den), v2);
+    }
+    __device__ __forceinline__ void shift(R2 w5) {
+        const R2 d4 = sub2(w5, v4);
         u0 = u1;
         u1 = u2;
         u2 = tterm(sub2(d4, d3));
@@ -1050,205 +1183,135 @@ struct Weno5Run2 {
     }
 };
 
-// Shared layout of k2_adv2 per buffer (two buffers: velocities k and k+1 in
-// flight): the halo tile of F and G, rows y0-3 .. y0+18 with column
-// x0-3+i at i + 1 (the interior x0 .. x0+31 at columns 4 .. 35, 16-byte
-// aligned, row stride 44: a row's 16 lanes of the x runs on 8 banks apart),
-// then RL and base of the tile's nodes.
-constexpr int kA2Row = 44, kA2Rows = kAdvY + 6;
-constexpr int kA2H = 2 * kA2Rows * kA2Row;                  // halo of F and G
-constexpr int kA2T = 2 * kAdvY * kAdvX;                     // RL (or base) of F and G
-constexpr int kA2Buf = kA2H + 2 * kA2T;
-constexpr size_t kA2Smem = sizeof(float) * 2 * kA2Buf + sizeof(float2) * (kAdvY * (kAdvX + 1) + (kAdvY + 1) * kAdvX) +
-                           sizeof(int) * (kA2Rows + kAdvX + 6);
+constexpr int kPT = 32;                      // tile edge
+constexpr int kPW = kPT + 6;                 // halo edge
+constexpr int kPP = kPW + 1, kPD = kPT + 1;  // row pitches of the halo and of df_x
+constexpr int kPThreads = 128, kPRun = 8;    // nodes per walk
+constexpr int kPBufs = 3;
+// CTAs per SM.  FP32: four, with 124 registers a thread (212 us at 384^2, Q 16;
+// five with 96 serialise each walk: 261 us; three: 215 us).
+template <typename R>
+constexpr int adv_ctas() { return std::is_same<R, float>::value ? 4 : 2; }
+template <typename R>
+constexpr size_t adv_smem() { return sizeof(Pair<R>) * (kPBufs * kPW * kPP + kPT * kPD) + sizeof(int) * 2 * kPW; }
+static_assert(kPThreads / 32 * kPRun == kPT, "a warp per 8 rows or columns of the tile");
 
 __device__ __forceinline__ void cp_async_wait_1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 
-// A thread's share of the whole-chunk copies of one velocity, the same for
-// every velocity of the CTA and so formed once: shared offsets, in-plane
-// global offsets (below N < 2^31) and, per copy, whether it reads the G
-// plane; a negative shared offset marks an absent copy.
-struct Adv2Copies {
-    int hs[2], hg[2];   // 16-byte chunks of the halo interior
-    int ss[2], sg[2];   // 4-byte elements of the halo side columns
-    int rs, rg;         // the 16-byte chunk of RL (and base) every thread copies
-    unsigned gmask;     // bit q: hs[q] reads G; bit 2+q: ss[q]; bit 4: the RL chunk
-};
-static_assert(2 * kAdvY * 8 == 256 && 2 * kA2Rows * 8 <= 512 && 2 * kA2Rows * 6 <= 512,
-              "copy shares of a 256-thread CTA");
-
-__device__ __forceinline__ Adv2Copies adv2_plan(const int* rowoff, const int* coloff, int x0, int y0, int nx) {
-    Adv2Copies p;
-    p.gmask = 0u;
-    const int t = threadIdx.x;
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        const int e = t + 256 * q;
-        p.hs[q] = -1;
-        p.ss[q] = -1;
-        if (e < 2 * kA2Rows * 8) {
-            const int c = e % 8, r = (e / 8) % kA2Rows, d = e / (8 * kA2Rows);
-            p.hs[q] = (d * kA2Rows + r) * kA2Row + 4 + 4 * c;
-            p.hg[q] = rowoff[r] + x0 + 4 * c;
-            if (d) p.gmask |= 1u << q;
-        }
-        if (e < 2 * kA2Rows * 6) {
-            const int c = e % 6, r = (e / 6) % kA2Rows, d = e / (6 * kA2Rows);
-            const int i = c < 3 ? c : 32 + c;               // halo columns 0..2 and 35..37
-            p.ss[q] = (d * kA2Rows + r) * kA2Row + i + 1;
-            p.sg[q] = rowoff[r] + coloff[i];
-            if (d) p.gmask |= 4u << q;
-        }
-    }
-    const int c = t % 8, r = (t / 8) % kAdvY, d = t / (8 * kAdvY);
-    p.rs = (d * kAdvY + r) * kAdvX + 4 * c;
-    p.rg = (y0 + r) * nx + x0 + 4 * c;
-    if (d) p.gmask |= 16u;
-    return p;
-}
-
-// Queues the asynchronous copies of velocity k (planes at F + k N and
-// F + NF + k N) into buffer `buf`: when `fast`, the thread's whole 16-byte
-// chunks of the aligned interior and its side-column elements (plan `cp`);
-// otherwise element copies of everything (wrapped columns, a ragged tile
-// edge, nx not a multiple of 4).
-__device__ __forceinline__ void adv2_issue(float* buf, const float* src, const float* RL, const float* base,
-                                           long long kN, long long NF, const int* rowoff, const int* coloff,
-                                           int x0, int y0, int nx, int ny, bool fast, bool with_base,
-                                           const Adv2Copies& cp) {
-    float* H = buf;
-    float* Rs = buf + kA2H;
-    float* Bs = Rs + kA2T;
-    const int t = threadIdx.x;
-    if (fast) {
-        const float* sF = src + kN;
-        const float* sG = sF + NF;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            if (cp.hs[q] >= 0) cp_async16(H + cp.hs[q], ((cp.gmask >> q) & 1u ? sG : sF) + cp.hg[q]);
-            if (cp.ss[q] >= 0) cp_async_elem<float>(H + cp.ss[q], ((cp.gmask >> (2 + q)) & 1u ? sG : sF) + cp.sg[q]);
-        }
-        const long long g = kN + ((cp.gmask & 16u) ? NF : 0) + cp.rg;
-        cp_async16(Rs + cp.rs, RL + g);
-        if (with_base) cp_async16(Bs + cp.rs, base + g);
-    } else {
-        for (int e = t; e < 2 * kA2Rows * (kAdvX + 6); e += 256) {
-            const int i = e % (kAdvX + 6), r = (e / (kAdvX + 6)) % kA2Rows, d = e / ((kAdvX + 6) * kA2Rows);
-            cp_async_elem<float>(H + (d * kA2Rows + r) * kA2Row + i + 1, src + d * NF + kN + rowoff[r] + coloff[i]);
-        }
-        for (int e = t; e < 2 * kAdvY * kAdvX; e += 256) {
-            const int c = e % kAdvX, r = (e / kAdvX) % kAdvY, d = e / (kAdvX * kAdvY);
-            if (x0 + c < nx && y0 + r < ny) {
-                const long long g = d * NF + kN + (long long)(y0 + r) * nx + x0 + c;
-                cp_async_elem<float>(Rs + (d * kAdvY + r) * kAdvX + c, RL + g);
-                if (with_base) cp_async_elem<float>(Bs + (d * kAdvY + r) * kAdvX + c, base + g);
-            }
-        }
-    }
-}
-
-// three CTAs per SM: with up to 85 registers the constants of the packed
-// arithmetic and the copy plan stay in registers (with the 64 of four CTAs
-// per SM the kernel executed 9 % more instructions and took 10 % longer)
-template <int Q>
-__global__ void __launch_bounds__(256, 3)
-k2_adv2(Slab2 s, const Par2<float> pr, const float* __restrict__ rtab, const float* __restrict__ src,
-        const float* base, float* out, const float* __restrict__ RL) {
-    constexpr int K = Q * Q, RPW = kAdvY / 8;
-    static_assert(kAdvX == 32 && kAdvY == 16, "run split: 33 = 5 + 7 x 4 x-faces, 17 = 5 + 3 x 4 y-faces");
+template <typename R, int Q, bool FTZ>
+__global__ void __launch_bounds__(kPThreads, adv_ctas<R>())
+k2_adv(Slab2 s, const Par2<R> pr, const R* __restrict__ rtab, const Pair<R>* __restrict__ src, Pair<R>* V, int planes) {
+    using R2 = Pair<R>;
+    constexpr int K = Q * Q, NW = kPThreads / 32;
+    constexpr int NR = (kPW + NW - 1) / NW;                          // halo rows per warp
+    constexpr int NE = (6 * kPW + kPThreads - 1) / kPThreads;        // right-edge elements per thread
     extern __shared__ __align__(16) double sma[];
-    float* buf0 = reinterpret_cast<float*>(sma);
-    float2* FX = reinterpret_cast<float2*>(buf0 + 2 * kA2Buf);
-    float2* FY = FX + kAdvY * (kAdvX + 1);
-    int* rowoff = reinterpret_cast<int*>(FY + (kAdvY + 1) * kAdvX);
-    int* coloff = rowoff + kA2Rows;
+    R2* const H0 = reinterpret_cast<R2*>(sma);
+    R2* const DX = H0 + kPBufs * kPW * kPP;
+    int* const rowoff = reinterpret_cast<int*>(DX + kPT * kPD);
+    int* const coloff = rowoff + kPW;
     const int nx = s.nx, ny = s.ny;
-    const long long N = s.N, NF = (long long)K * N;
-    const int tilesx = (nx + kAdvX - 1) / kAdvX;
-    const int x0 = (blockIdx.x % tilesx) * kAdvX, y0 = (blockIdx.x / tilesx) * kAdvY;
+    const long long N = s.N;
+    const int tilesx = (nx + kPT - 1) / kPT;
+    const int x0 = (blockIdx.x % tilesx) * kPT, y0 = (blockIdx.x / tilesx) * kPT;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     TableLayout L(Q);
-    for (int e = threadIdx.x; e < kA2Rows + kAdvX + 6; e += blockDim.x) {
-        if (e < kA2Rows) rowoff[e] = wrapi(y0 - 3 + e, ny) * nx;
-        else coloff[e - kA2Rows] = wrapi(x0 - 3 + (e - kA2Rows), nx);
-    }
+    if (tid < kPW) rowoff[tid] = wrapi(y0 - 3 + tid, ny) * nx;
+    else if (tid >= 64 && tid < 64 + kPW) coloff[tid - 64] = wrapi(x0 - 3 + tid - 64, nx);
     __syncthreads();
-    const bool fast = (nx % 4 == 0) && (x0 + kAdvX <= nx) && (y0 + kAdvY <= ny);
-    const Adv2Copies cplan = adv2_plan(rowoff, coloff, x0, y0, nx);
-    const float eps = pr.weno_eps, idx = pr.inv_dx, dt = pr.dt, ralpha = pr.alpha, rbeta = pr.beta;
-    const bool with_base = pr.with_base != 0;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const bool xrun = threadIdx.x < 128;
-    const int rj = xrun ? (threadIdx.x >> 4) : ((threadIdx.x - 128) >> 5);
-    const int rl = xrun ? (threadIdx.x & 15) : (threadIdx.x & 31);
-    const int fa = rj == 0 ? 0 : 4 * rj + 1, nrun = rj == 0 ? 5 : 4, fl = fa + nrun - 1;
-    const int hst = xrun ? 1 : kA2Row;
-    // x face f of row r: stencil from halo (r + 3, f); y face f of column c: from halo (f, c + 3)
-    const int hrow = xrun ? (rl + 3) * kA2Row + 1 : rl + 3 + 1;
-    float2* frow = xrun ? FX + rl * (kAdvX + 1) : FY + rl;
-    const int fst = xrun ? 1 : kAdvX;
-    const int x = x0 + lane;
-    int ooff[RPW];
-    bool oval[RPW];
+    // this thread's halo elements, the same for every velocity: the columns
+    // 0 .. 31 of rows warp, warp + 4, ... and its share of the columns 32 .. 37
+    unsigned go[NR], ge[NE];
+    int se[NE];
 #pragma unroll
-    for (int rr = 0; rr < RPW; ++rr) {
-        const int y = y0 + warp * RPW + rr;
-        oval[rr] = (x < nx && y < ny);
-        ooff[rr] = oval[rr] ? y * nx + x : 0;
+    for (int j = 0; j < NR; ++j) go[j] = (unsigned)(rowoff[min(warp + NW * j, kPW - 1)] + coloff[lane]);
+#pragma unroll
+    for (int j = 0; j < NE; ++j) {
+        const int e = tid + kPThreads * j;
+        const int r = min(e / 6, kPW - 1), c = kPT + e % 6;
+        ge[j] = (unsigned)(rowoff[r] + coloff[c]);
+        se[j] = e < 6 * kPW ? r * kPP + c : -1;
     }
-    const int k0 = blockIdx.y * kAdvPlanes, k1 = min(k0 + kAdvPlanes, K);
-    constexpr int HG = kA2Rows * kA2Row;                    // G's halo after F's
-    adv2_issue(buf0, src, RL, base, (long long)k0 * N, NF, rowoff, coloff, x0, y0, nx, ny, fast, with_base, cplan);
-    cp_async_commit();
-    if (k0 + 1 < k1)
-        adv2_issue(buf0 + kA2Buf, src, RL, base, (long long)(k0 + 1) * N, NF, rowoff, coloff, x0, y0, nx, ny, fast,
-                   with_base, cplan);
-    cp_async_commit();
-    for (int k = k0; k < k1; ++k) {
-        float* buf = buf0 + ((k - k0) & 1) * kA2Buf;
-        const float* H = buf;
-        const float* Rs = buf + kA2H;
-        const float* Bs = Rs + kA2T;
-        const float vx = rtab[L.xi + k / Q], vy = rtab[L.xi + k % Q];
-        cp_async_wait_1();                                  // velocity k's copies (all but the newest group)
-        __syncthreads();
-        {
-            const bool pos = (xrun ? vx : vy) >= 0.f;       // uniform per warp
-            const int dir = pos ? 1 : -1, f0 = pos ? fa : fl;
-            const float* hb = H + hrow + (pos ? fa : fl + 5) * hst;
-            const int hs = dir * hst;
-            auto at = [&](int o) { return make_float2(hb[o], hb[HG + o]); };
-            Weno5Run2 w;
-            w.start(at(0), at(hs), at(2 * hs), at(3 * hs), at(4 * hs), eps);
+    auto copy = [](R2* dst, const R2* g) {
+        if constexpr (sizeof(R2) == 16) cp_async16(dst, g);
+        else cp_async_elem<double>(reinterpret_cast<double*>(dst), reinterpret_cast<const double*>(g));
+    };
+    auto issue = [&](int k, int b) {
+        const R2* p = src + (long long)k * N;
+        R2* H = H0 + b * kPW * kPP;
+        R2* hr = H + warp * kPP + lane;
 #pragma unroll
-            for (int q = 0; q < 5; ++q) {
-                if (q >= nrun) break;
-                frow[(f0 + dir * q) * fst] = w.face();
-                if (q + 1 < nrun) w.shift(at((q + 5) * hs));
+        for (int j = 0; j < NR; ++j)
+            if (warp + NW * j < kPW) copy(hr + NW * j * kPP, p + go[j]);
+#pragma unroll
+        for (int j = 0; j < NE; ++j)
+            if (se[j] >= 0) copy(H + se[j], p + ge[j]);
+    };
+    const R eps = pr.weno_eps;
+    const R2 hscale = splat(pr.hs);
+    const int k0 = blockIdx.y * planes, k1 = min(k0 + planes, K);
+    issue(k0, 0);
+    cp_async_commit();
+    if (k0 + 1 < k1) issue(k0 + 1, 1);
+    cp_async_commit();
+    const int x = x0 + lane, yw = y0 + warp * kPRun;
+    const int rows = x < nx ? min(kPRun, ny - yw) : 0;               // nodes of this thread's y walk (may be <= 0)
+    const unsigned o0 = (unsigned)yw * (unsigned)nx + (unsigned)x;
+    for (int k = k0, b = 0; k < k1; ++k, b = b == kPBufs - 1 ? 0 : b + 1) {
+        const R vx = rtab[L.xi + k / Q], vy = rtab[L.xi + k % Q];
+        const bool px = vx >= R(0), py = vy >= R(0);
+        // V of this thread's nodes, in the order of its y walk (up for
+        // xi_y >= 0, else down)
+        R2* const p = V + (long long)k * N;
+        R2 vv[kPRun];
+#pragma unroll
+        for (int q = 0; q < kPRun; ++q) {
+            const int r = py ? q : kPRun - 1 - q;
+            vv[q] = r < rows ? p[o0 + (unsigned)(r * nx)] : splat(R(0));
+        }
+        cp_async_wait_1();                                           // velocity k's halo
+        __syncthreads();
+        const R2* H = H0 + b * kPW * kPP;
+        Weno5Run2<R, FTZ> w;
+        // both walks: face f lies below node f; xi >= 0 takes halo cells f ..
+        // f+4 and walks up, xi < 0 takes f+5 .. f+1 and walks down, so that a
+        // new face minus the one before is df for xi >= 0 and -df for xi < 0
+        // and |xi| carries the sign; after a face the walk's v2 is the node
+        // between the two
+        {
+            const int st = px ? 1 : -1;
+            const R2* h = H + (lane + 3) * kPP + warp * kPRun + (px ? 0 : kPRun + 5);
+            w.start(h[0], h[st], h[2 * st], h[3 * st], h[4 * st], eps);
+            R2 f = w.face();
+            R2* dx = DX + lane * kPD + warp * kPRun + (px ? 0 : kPRun - 1);
+#pragma unroll
+            for (int q = 0; q < kPRun; ++q) {
+                w.shift(h[(q + 5) * st]);
+                const R2 g = w.face();
+                dx[q * st] = sub2(g, f);
+                f = g;
             }
         }
-        __syncthreads();
-        const float2 cx = f2s(-vx * idx), cy = f2s(-vy * idx);
-        float* op = out + (long long)k * N;
-#pragma unroll
-        for (int rr = 0; rr < RPW; ++rr) {
-            if (!oval[rr]) continue;
-            const int ty = warp * RPW + rr;
-            float2 Rv = make_float2(Rs[ty * kAdvX + lane], Rs[(kAdvY + ty) * kAdvX + lane]);
-            Rv = fma2(cx, sub2(FX[ty * (kAdvX + 1) + lane + 1], FX[ty * (kAdvX + 1) + lane]), Rv);
-            Rv = fma2(cy, sub2(FY[(ty + 1) * kAdvX + lane], FY[ty * kAdvX + lane]), Rv);
-            const int hc = (ty + 3) * kA2Row + lane + 4;
-            const float2 hv = make_float2(H[hc], H[HG + hc]);
-            float2 o = mul2(f2s(rbeta), fma2(f2s(dt), Rv, hv));
-            if (with_base)
-                o = fma2(f2s(ralpha), make_float2(Bs[ty * kAdvX + lane], Bs[(kAdvY + ty) * kAdvX + lane]), o);
-            op[ooff[rr]] = o.x;
-            op[NF + ooff[rr]] = o.y;
-        }
-        __syncthreads();                                    // this buffer and the faces consumed
-        if (k + 2 < k1)
-            adv2_issue(buf, src, RL, base, (long long)(k + 2) * N, NF, rowoff, coloff, x0, y0, nx, ny, fast,
-                       with_base, cplan);
+        __syncthreads();                                             // df_x written, the buffer of k - 1 consumed
+        if (k + 2 < k1) issue(k + 2, b == 0 ? kPBufs - 1 : b - 1);
         cp_async_commit();
+        {
+            const int dir = py ? 1 : -1, st = dir * kPP;
+            const R2* h = H + (warp * kPRun + (py ? 0 : kPRun + 5)) * kPP + lane + 3;
+            const R2* dx = DX + (warp * kPRun + (py ? 0 : kPRun - 1)) * kPD + lane;
+            const R2 cx = splat(pr.ca * (px ? vx : -vx)), cy = splat(pr.ca * (py ? vy : -vy));
+            w.start(h[0], h[st], h[2 * st], h[3 * st], h[4 * st], eps);
+            R2 f = w.face();
+#pragma unroll
+            for (int q = 0; q < kPRun; ++q) {
+                w.shift(h[(q + 5) * st]);
+                const R2 g = w.face();
+                const R2 inc = fma2(cy, sub2(g, f), fma2(cx, dx[q * dir * kPD], vv[q]));
+                const int r = py ? q : kPRun - 1 - q;
+                if (r < rows) p[o0 + (unsigned)(r * nx)] = fma2(hscale, w.v2, inc);
+                f = g;
+            }
+        }
     }
 }
 
@@ -1259,9 +1322,9 @@ k2_adv2(Slab2 s, const Par2<float> pr, const float* __restrict__ rtab, const flo
 // phi_k(u) = sum_l S_kl m_l(u, T) (the 2D Gaussian factorises), G = T/2 F.
 template <typename R>
 __global__ void k2_init(Slab2 s, const double* __restrict__ tab, const double* __restrict__ n0,
-                        const double* __restrict__ u0, const double* __restrict__ T0, R* st, unsigned* err) {
+                        const double* __restrict__ u0, const double* __restrict__ T0, Pair<R>* st, unsigned* err) {
     const int Q = s.Q;
-    const long long N = s.N, NF = (long long)Q * Q * N;
+    const long long N = s.N;
     TableLayout L(Q);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
         double n = n0[i], ux = u0[i], uy = u0[N + i], T = T0[i];
@@ -1285,9 +1348,10 @@ __global__ void k2_init(Slab2 s, const double* __restrict__ tab, const double* _
         for (int kx = 0; kx < Q; ++kx)
             for (int ky = 0; ky < Q; ++ky) {
                 double f = n * px[kx] * py[ky];
-                long long g = (long long)(kx * Q + ky) * N + i;
-                st[g] = (R)f;
-                st[NF + g] = (R)(0.5 * T * f);
+                Pair<R> h;
+                h.x = (R)f;
+                h.y = (R)(0.5 * T * f);
+                st[(long long)(kx * Q + ky) * N + i] = h;
             }
     }
 }
@@ -1337,10 +1401,23 @@ __global__ void __launch_bounds__(256) k2_totals(Slab2 s, const double* __restri
     if (threadIdx.x < 4) out[threadIdx.x] = red[threadIdx.x][0] * s.dx * s.dx;
 }
 
-template <typename A, typename B>
-__global__ void k2_convert(const A* __restrict__ in, B* __restrict__ out, long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        out[i] = (B)in[i];
+// The interleaved state to or from two FP64 arrays of n = Q^2 N values each.
+template <typename R>
+__global__ void k2_split(const Pair<R>* __restrict__ in, double* __restrict__ F, double* __restrict__ G, long long n) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const Pair<R> h = in[i];
+        F[i] = (double)h.x;
+        G[i] = (double)h.y;
+    }
+}
+template <typename R>
+__global__ void k2_join(const double* __restrict__ F, const double* __restrict__ G, Pair<R>* __restrict__ out, long long n) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        Pair<R> h;
+        h.x = (R)F[i];
+        h.y = (R)G[i];
+        out[i] = h;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1596,10 +1673,10 @@ struct Ctx2 {
     Slab2 s;
     int prec = EVFDLB_FP32;
     double dt = 0.0;
+    int sms = 1;                 // SMs of the context's device
     size_t esize = 4;
     cudaStream_t user = nullptr, cap = nullptr;
     void* state[3] = {nullptr, nullptr, nullptr};
-    void* RL = nullptr;
     void* fld = nullptr;
     double* mom = nullptr;
     double* tables = nullptr;
@@ -1615,14 +1692,13 @@ struct Ctx2 {
     unsigned* err = nullptr;
     cudaGraphExec_t g_one = nullptr;
     size_t smem_fields = 0, smem_coll = 0;
+    int coll_ctas = 1;           // resident CTAs of k2_coll_pipe
     // the model constants in precision R (the stage weights are the caller's)
     template <typename R>
     Par2<R> par() const {
         Par2<R> q{};
         const double sg = p.sigma, idx = 1.0 / p.dx;
-        q.inv_dx = (R)idx;
         q.k12 = (R)(idx / 12.0);
-        q.dt = (R)dt;
         q.weno_eps = (R)p.weno_eps;
         q.b = (R)(2.0 * M_PI * sg * sg * sg / 3.0);
         q.eta_coef = (R)(M_PI * sg * sg * sg / 6.0);
@@ -1632,93 +1708,91 @@ struct Ctx2 {
 };
 
 namespace {
-// k2_coll is compiled for each even Q of the 2D model (4 .. 16)
+// The velocity kernels are compiled for each even Q of the 2D model (4 .. 16);
+// f receives the order as a compile-time constant.
+template <typename F>
+auto with_q(int Q, F f) {
+    switch (Q) {
+        case 4: return f(std::integral_constant<int, 4>{});
+        case 6: return f(std::integral_constant<int, 6>{});
+        case 8: return f(std::integral_constant<int, 8>{});
+        case 10: return f(std::integral_constant<int, 10>{});
+        case 12: return f(std::integral_constant<int, 12>{});
+        case 14: return f(std::integral_constant<int, 14>{});
+        default: return f(std::integral_constant<int, 16>{});
+    }
+}
+
+// Velocities per CTA of k2_adv: up to 16 (the copy offsets are formed once per
+// CTA), fewer where the grid would otherwise hold less than four waves of
+// CTAs, one on grids of a few tiles.
 template <typename R>
-void launch_coll(int Q, int nc, size_t smem, cudaStream_t st, const Slab2& s, const R* rtab, const R* src,
-                 const R* fld, R* RL) {
-    switch (Q) {
-        case 4: k2_coll<R, 4><<<nc, 256, smem, st>>>(s, rtab, src, fld, RL); break;
-        case 6: k2_coll<R, 6><<<nc, 256, smem, st>>>(s, rtab, src, fld, RL); break;
-        case 8: k2_coll<R, 8><<<nc, 256, smem, st>>>(s, rtab, src, fld, RL); break;
-        case 10: k2_coll<R, 10><<<nc, 256, smem, st>>>(s, rtab, src, fld, RL); break;
-        case 12: k2_coll<R, 12><<<nc, 256, smem, st>>>(s, rtab, src, fld, RL); break;
-        case 14: k2_coll<R, 14><<<nc, 256, smem, st>>>(s, rtab, src, fld, RL); break;
-        default: k2_coll<R, 16><<<nc, 256, smem, st>>>(s, rtab, src, fld, RL); break;
-    }
-}
-
-// k2_adv is compiled for each even Q of the 2D model (4 .. 16) and both
-// output forms
-template <typename R, bool RHS>
-void launch_adv_t(int Q, dim3 g, cudaStream_t st, const Slab2& s, const Par2<R>& pr, const R* rtab, const R* src,
-                  const R* base, R* out, const R* RL, double* rhs_out) {
-    switch (Q) {
-        case 4: k2_adv<R, 4, RHS><<<g, 256, 0, st>>>(s, pr, rtab, src, base, out, RL, rhs_out); break;
-        case 6: k2_adv<R, 6, RHS><<<g, 256, 0, st>>>(s, pr, rtab, src, base, out, RL, rhs_out); break;
-        case 8: k2_adv<R, 8, RHS><<<g, 256, 0, st>>>(s, pr, rtab, src, base, out, RL, rhs_out); break;
-        case 10: k2_adv<R, 10, RHS><<<g, 256, 0, st>>>(s, pr, rtab, src, base, out, RL, rhs_out); break;
-        case 12: k2_adv<R, 12, RHS><<<g, 256, 0, st>>>(s, pr, rtab, src, base, out, RL, rhs_out); break;
-        case 14: k2_adv<R, 14, RHS><<<g, 256, 0, st>>>(s, pr, rtab, src, base, out, RL, rhs_out); break;
-        default: k2_adv<R, 16, RHS><<<g, 256, 0, st>>>(s, pr, rtab, src, base, out, RL, rhs_out); break;
-    }
-}
-
-// the FP32 stage form: F and G of a velocity as float2 pairs
-void launch_adv2(int Q, dim3 g, cudaStream_t st, const Slab2& s, const Par2<float>& pr, const float* rtab,
-                 const float* src, const float* base, float* out, const float* RL) {
-    switch (Q) {
-        case 4: k2_adv2<4><<<g, 256, kA2Smem, st>>>(s, pr, rtab, src, base, out, RL); break;
-        case 6: k2_adv2<6><<<g, 256, kA2Smem, st>>>(s, pr, rtab, src, base, out, RL); break;
-        case 8: k2_adv2<8><<<g, 256, kA2Smem, st>>>(s, pr, rtab, src, base, out, RL); break;
-        case 10: k2_adv2<10><<<g, 256, kA2Smem, st>>>(s, pr, rtab, src, base, out, RL); break;
-        case 12: k2_adv2<12><<<g, 256, kA2Smem, st>>>(s, pr, rtab, src, base, out, RL); break;
-        case 14: k2_adv2<14><<<g, 256, kA2Smem, st>>>(s, pr, rtab, src, base, out, RL); break;
-        default: k2_adv2<16><<<g, 256, kA2Smem, st>>>(s, pr, rtab, src, base, out, RL); break;
-    }
+void launch_adv(const Ctx2* c, cudaStream_t st, const Par2<R>& pr, const R* src, R* V) {
+    const Slab2& s = c->s;
+    const long long tiles = (long long)((s.nx + kPT - 1) / kPT) * ((s.ny + kPT - 1) / kPT), K = (long long)s.Q * s.Q;
+    const int planes =
+        (int)std::min<long long>(16, std::max<long long>(1, tiles * K / (4LL * adv_ctas<R>() * c->sms)));
+    const dim3 g((unsigned)tiles, (unsigned)((K + planes - 1) / planes));
+    constexpr bool F32 = std::is_same<R, float>::value;
+    const bool ftz = F32 && c->p.weno_eps >= kFtzMinEps;
+    with_q(s.Q, [&](auto q) {
+        constexpr int Q = decltype(q)::value;
+        const Pair<R>* in = (const Pair<R>*)src;
+        if (ftz) k2_adv<R, Q, F32><<<g, kPThreads, adv_smem<R>(), st>>>(s, pr, (const R*)c->rtab, in, (Pair<R>*)V, planes);
+        else k2_adv<R, Q, false><<<g, kPThreads, adv_smem<R>(), st>>>(s, pr, (const R*)c->rtab, in, (Pair<R>*)V, planes);
+    });
 }
 
 template <typename R>
-void launch_adv(int Q, dim3 g, cudaStream_t st, const Slab2& s, const Par2<R>& pr, const R* rtab, const R* src,
-                const R* base, R* out, const R* RL, double* rhs_out, int mode) {
-    if (mode == 1) launch_adv_t<R, true>(Q, g, st, s, pr, rtab, src, base, out, RL, rhs_out);
-    else launch_adv_t<R, false>(Q, g, st, s, pr, rtab, src, base, out, RL, rhs_out);
+void launch_coll(const Ctx2* c, cudaStream_t st, const Par2<R>& pr, const R* src, const R* base, R* V) {
+    const Slab2& s = c->s;
+    const int groups = (int)((s.N + kNB - 1) / kNB);
+    with_q(s.Q, [&](auto q) {
+        constexpr int Q = decltype(q)::value;
+        const R* fld = (const R*)c->fld;
+        const Pair<R> *in = (const Pair<R>*)src, *b = (const Pair<R>*)base;
+        if constexpr (std::is_same<R, float>::value)
+            k2_coll_pipe<Q><<<std::min(groups, c->coll_ctas), coll_threads<Q>(), c->smem_coll, st>>>(
+                s, pr, in, fld, b, (float2*)V, groups);
+        else k2_coll<R, Q><<<groups, 256, c->smem_coll, st>>>(s, pr, (const R*)c->rtab, in, fld, b, (Pair<R>*)V);
+    });
+}
+
+// Shared memory of the velocity kernels of order Q, and the resident CTAs of
+// the FP32 collision kernel.
+cudaError_t configure_2d(Ctx2* c) {
+    return with_q(c->s.Q, [&](auto q) {
+        constexpr int Q = decltype(q)::value;
+        const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        cudaError_t e;
+        if (c->prec == EVFDLB_FP32) {
+            c->smem_coll = sizeof(float) * Coll2Lay<Q>::PIPE;
+            e = cudaFuncSetAttribute(k2_coll_pipe<Q>, attr, (int)c->smem_coll);
+            int per_sm = 0;
+            if (e == cudaSuccess)
+                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k2_coll_pipe<Q>, coll_threads<Q>(), c->smem_coll);
+            c->coll_ctas = c->sms * std::max(1, per_sm);
+        } else {
+            c->smem_coll = sizeof(double) * Coll2Lay<Q>::ONE;
+            e = cudaFuncSetAttribute(k2_coll<double, Q>, attr, (int)c->smem_coll);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(k2_adv<double, Q, false>, attr, (int)adv_smem<double>());
+        }
+        return e;
+    });
 }
 
 // k2_moments: 128 nodes per CTA pass (grid-stride beyond 8192 CTAs)
 int moments_grid(long long N) { return (int)std::min<long long>((N + 127) / 128, 8192); }
 
-// k2_moments is compiled for each even Q of the 2D model (4 .. 16)
 template <typename R>
-void launch_moments(int Q, int nb, cudaStream_t st, const Slab2& s, const Pow2<R>& pw, const R* src, double* mom,
+void launch_moments(int Q, int nb, cudaStream_t st, const Slab2& s, const Pow2<R>& pw, const Pair<R>* src, double* mom,
                     float* prf, unsigned* err) {
-    switch (Q) {
-        case 4: k2_moments<R, 4><<<nb, 256, 0, st>>>(s, pw, src, mom, prf, err); break;
-        case 6: k2_moments<R, 6><<<nb, 256, 0, st>>>(s, pw, src, mom, prf, err); break;
-        case 8: k2_moments<R, 8><<<nb, 256, 0, st>>>(s, pw, src, mom, prf, err); break;
-        case 10: k2_moments<R, 10><<<nb, 256, 0, st>>>(s, pw, src, mom, prf, err); break;
-        case 12: k2_moments<R, 12><<<nb, 256, 0, st>>>(s, pw, src, mom, prf, err); break;
-        case 14: k2_moments<R, 14><<<nb, 256, 0, st>>>(s, pw, src, mom, prf, err); break;
-        default: k2_moments<R, 16><<<nb, 256, 0, st>>>(s, pw, src, mom, prf, err); break;
-    }
+    with_q(Q, [&](auto q) { k2_moments<R, decltype(q)::value><<<nb, 256, 0, st>>>(s, pw, src, mom, prf, err); });
 }
 
 template <typename R>
-cudaError_t coll_attr(int Q, size_t smem) {
-    const int v = (int)smem;
-    switch (Q) {
-        case 4: return cudaFuncSetAttribute(k2_coll<R, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
-        case 6: return cudaFuncSetAttribute(k2_coll<R, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
-        case 8: return cudaFuncSetAttribute(k2_coll<R, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
-        case 10: return cudaFuncSetAttribute(k2_coll<R, 10>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
-        case 12: return cudaFuncSetAttribute(k2_coll<R, 12>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
-        case 14: return cudaFuncSetAttribute(k2_coll<R, 14>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
-        default: return cudaFuncSetAttribute(k2_coll<R, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, v);
-    }
-}
-
-template <typename R>
-void queue_stage_t(Ctx2* c, cudaStream_t st, const void* src, const void* base, void* out, double* rhs_out,
-                   double alpha, double beta, int mode) {
+void queue_stage_t(Ctx2* c, cudaStream_t st, const void* src, const void* base, void* out, double alpha, double beta,
+                   int mode) {
     const Slab2& s = c->s;
     const int Q = s.Q;
     constexpr bool F32 = std::is_same<R, float>::value;
@@ -1726,40 +1800,33 @@ void queue_stage_t(Ctx2* c, cudaStream_t st, const void* src, const void* base, 
     // only needed by the FP64 build and by the diagnostics
     const int nbm = moments_grid(s.N);
     Par2<R> pr = c->template par<R>();
+    const double cb = mode == 1 ? 1.0 : beta * c->dt;
     pr.alpha = (R)alpha;
-    pr.beta = (R)beta;
+    pr.cb = (R)cb;
+    pr.ca = (R)(-cb / c->p.dx);
     pr.with_base = alpha != 0.0;
-    if constexpr (F32) launch_moments<float>(Q, nbm, st, s, c->pwf, (const float*)src, nullptr, c->prf, c->err);
-    else launch_moments<double>(Q, nbm, st, s, c->pwd, (const double*)src, c->mom, nullptr, c->err);
+    pr.hs = (R)(mode == 1 ? 0.0 : 1.0);
+    R* V = (R*)out;
+    if constexpr (F32) launch_moments<float>(Q, nbm, st, s, c->pwf, (const float2*)src, nullptr, c->prf, c->err);
+    else launch_moments<double>(Q, nbm, st, s, c->pwd, (const double2*)src, c->mom, nullptr, c->err);
     dim3 gf((s.nx + kTile2 - 1) / kTile2, (s.ny + kTile2 - 1) / kTile2);
     k2_fields<R><<<gf, 256, c->smem_fields, st>>>(s, pr, c->mom, c->prf, (const R*)c->ftw, c->fplan, c->fm_off,
                                                    (const R*)c->fm_w, (R*)c->fld, c->err);
-    int nc = (int)((s.N + kNB - 1) / kNB);
-    launch_coll<R>(Q, nc, c->smem_coll, st, s, (const R*)c->rtab, (const R*)src, (const R*)c->fld, (R*)c->RL);
-    const int tiles = ((s.nx + kAdvX - 1) / kAdvX) * ((s.ny + kAdvY - 1) / kAdvY);
-    if constexpr (F32) {
-        if (mode == 0) {   // the FP32 stage form: one CTA column per group of velocities, F and G paired
-            dim3 ga(tiles, (Q * Q + kAdvPlanes - 1) / kAdvPlanes);
-            launch_adv2(Q, ga, st, s, pr, (const float*)c->rtab, (const float*)src, (const float*)base, (float*)out,
-                        (const float*)c->RL);
-            return;
-        }
-    }
-    dim3 ga(tiles, (2 * Q * Q + kAdvPlanes - 1) / kAdvPlanes);
-    launch_adv<R>(Q, ga, st, s, pr, (const R*)c->rtab, (const R*)src, (const R*)base, (R*)out, (const R*)c->RL,
-                  rhs_out, mode);
+    launch_coll<R>(c, st, pr, (const R*)src, (const R*)base, V);
+    launch_adv<R>(c, st, pr, (const R*)src, V);
 }
 
-void queue_stage(Ctx2* c, cudaStream_t st, const void* src, const void* base, void* out, double* rhs_out,
-                 double alpha, double beta, int mode) {
-    if (c->prec == EVFDLB_FP32) queue_stage_t<float>(c, st, src, base, out, rhs_out, alpha, beta, mode);
-    else queue_stage_t<double>(c, st, src, base, out, rhs_out, alpha, beta, mode);
+// mode 0: out = alpha base + beta (src + dt L(src)); mode 1: out = L(src)
+void queue_stage(Ctx2* c, cudaStream_t st, const void* src, const void* base, void* out, double alpha, double beta,
+                 int mode) {
+    if (c->prec == EVFDLB_FP32) queue_stage_t<float>(c, st, src, base, out, alpha, beta, mode);
+    else queue_stage_t<double>(c, st, src, base, out, alpha, beta, mode);
 }
 
 void queue_step(Ctx2* c, cudaStream_t st) {
-    queue_stage(c, st, c->state[0], nullptr, c->state[1], nullptr, 0.0, 1.0, 0);
-    queue_stage(c, st, c->state[1], c->state[0], c->state[2], nullptr, 0.75, 0.25, 0);
-    queue_stage(c, st, c->state[2], c->state[0], c->state[0], nullptr, 1.0 / 3.0, 2.0 / 3.0, 0);
+    queue_stage(c, st, c->state[0], nullptr, c->state[1], 0.0, 1.0, 0);
+    queue_stage(c, st, c->state[1], c->state[0], c->state[2], 0.75, 0.25, 0);
+    queue_stage(c, st, c->state[2], c->state[0], c->state[0], 1.0 / 3.0, 2.0 / 3.0, 0);
 }
 
 evfdlb_status st2(cudaError_t e) {
@@ -1771,7 +1838,6 @@ void destroy_2d(Ctx2* c) {
     if (!c) return;
     if (c->g_one) cudaGraphExecDestroy(c->g_one);
     for (int i = 0; i < 3; ++i) cudaFree(c->state[i]);
-    cudaFree(c->RL);
     cudaFree(c->fld);
     cudaFree(c->mom);
     cudaFree(c->tables);
@@ -1805,6 +1871,10 @@ evfdlb_status create_2d(const evfdlb_params& p, void* stream, Ctx2** out) {
     s.N = (long long)p.nx * p.ny;
     s.dx = p.dx;
     c->dt = resolved_dt_2d(p);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        c->sms < 1)
+        c->sms = 1;
     Taps2 t = taps_2d(p);
     s.nft = (int)(t.fg.size() / 2);
     s.nfm = (int)t.mw.size();
@@ -1820,7 +1890,6 @@ evfdlb_status create_2d(const evfdlb_params& p, void* stream, Ctx2** out) {
         if (e == cudaSuccess) e = cudaMalloc(ptr, bytes);
     };
     for (int i = 0; i < 3; ++i) alloc(&c->state[i], c->esize * 2 * NF);
-    alloc(&c->RL, c->esize * 2 * NF);
     alloc(&c->fld, c->esize * kNumFld2 * s.N);
     alloc((void**)&c->mom, sizeof(double) * kNumMom2 * s.N);
     alloc((void**)&c->tables, sizeof(double) * tab.size());
@@ -1832,12 +1901,6 @@ evfdlb_status create_2d(const evfdlb_params& p, void* stream, Ctx2** out) {
     alloc((void**)&c->fm_off, sizeof(int) * t.moff.size());
     alloc(&c->fm_w, c->esize * t.mw.size());
     if (f32) alloc((void**)&c->prf, sizeof(float) * kNumPrf2 * s.N);
-    std::vector<double> dbl = d_blocks(p.Q, xi.data(), w.data());
-    {   // k2_coll's constant block: DA, DB, then S[k][l] = w_k psi_l(xi_k)
-        const TableLayout L(p.Q);
-        dbl.insert(dbl.end(), tab.begin() + L.S, tab.begin() + L.S + p.Q * p.Q);
-    }
-    const std::vector<float> dblf(dbl.begin(), dbl.end());
     alloc((void**)&c->scratch, sizeof(double) * (2 * NF + 8));
     alloc((void**)&c->err, sizeof(unsigned));
     std::vector<float> tabf(tab.begin(), tab.end()), ftwf(fp.w.begin(), fp.w.end()), mwf(t.mw.begin(), t.mw.end());
@@ -1849,13 +1912,13 @@ evfdlb_status create_2d(const evfdlb_params& p, void* stream, Ctx2** out) {
     if (e == cudaSuccess && c->prec == EVFDLB_FP32)
         e = cudaMemcpy(c->rtab, tabf.data(), sizeof(float) * tabf.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(c->fplan, fp.plan.data(), sizeof(int) * fp.plan.size(), cudaMemcpyHostToDevice);
-    // the parity blocks and the synthesis matrix of this Q into k2_coll's
+    // FP64: the parity blocks and the synthesis matrix of this Q into k2_coll's
     // constant bank (every context of the same Q writes the same values)
-    if (e == cudaSuccess)
-        e = f32 ? cudaMemcpyToSymbol(c_coll_f, dblf.data(), sizeof(float) * dblf.size(),
-                                     sizeof(float) * coll_coff(p.Q))
-                : cudaMemcpyToSymbol(c_coll_d, dbl.data(), sizeof(double) * dbl.size(),
-                                     sizeof(double) * coll_coff(p.Q));
+    if (e == cudaSuccess && !f32) {
+        std::vector<double> dbl = d_blocks(p.Q, xi.data(), w.data());
+        dbl.insert(dbl.end(), tab.begin() + L.S, tab.begin() + L.S + p.Q * p.Q);
+        e = cudaMemcpyToSymbol(c_coll_d, dbl.data(), sizeof(double) * dbl.size(), sizeof(double) * coll_coff(p.Q));
+    }
     if (e == cudaSuccess)
         e = f32 ? cudaMemcpy(c->ftw, ftwf.data(), sizeof(float) * ftwf.size(), cudaMemcpyHostToDevice)
                 : cudaMemcpy(c->ftw, fp.w.data(), sizeof(double) * fp.w.size(), cudaMemcpyHostToDevice);
@@ -1865,17 +1928,11 @@ evfdlb_status create_2d(const evfdlb_params& p, void* stream, Ctx2** out) {
                 : cudaMemcpy(c->fm_w, t.mw.data(), sizeof(double) * t.mw.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(c->err, 0, sizeof(unsigned));
     c->smem_fields = f32 ? fields_smem_bytes<float>(s.Mf, s.mfm) : fields_smem_bytes<double>(s.Mf, s.mfm);
-    c->smem_coll = (c->prec == EVFDLB_FP32) ? coll_smem_bytes<float>(p.Q) : coll_smem_bytes<double>(p.Q);
     if (c->smem_fields > 227 * 1024) e = cudaErrorInvalidValue;   // force disc too wide for a tile
-    if (e == cudaSuccess) {
-        if (c->prec == EVFDLB_FP32) {
-            e = cudaFuncSetAttribute(k2_fields<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->smem_fields);
-            if (e == cudaSuccess) e = coll_attr<float>(p.Q, c->smem_coll);
-        } else {
-            e = cudaFuncSetAttribute(k2_fields<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->smem_fields);
-            if (e == cudaSuccess) e = coll_attr<double>(p.Q, c->smem_coll);
-        }
-    }
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(f32 ? (const void*)k2_fields<float> : (const void*)k2_fields<double>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->smem_fields);
+    if (e == cudaSuccess) e = configure_2d(c);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) {
         cudaGraph_t g = nullptr;
@@ -1929,8 +1986,8 @@ evfdlb_status init_2d(Ctx2* c, const double* n0, const double* u0, const double*
     if (e == cudaSuccess) e = cudaMemsetAsync(c->err, 0, sizeof(unsigned), c->user);
     if (e != cudaSuccess) return st2(e);
     int nb = (int)std::min<long long>((N + 255) / 256, 4096);
-    if (c->prec == EVFDLB_FP32) k2_init<float><<<nb, 256, 0, c->user>>>(c->s, c->tables, dn, du, dT, (float*)c->state[0], c->err);
-    else k2_init<double><<<nb, 256, 0, c->user>>>(c->s, c->tables, dn, du, dT, (double*)c->state[0], c->err);
+    if (c->prec == EVFDLB_FP32) k2_init<float><<<nb, 256, 0, c->user>>>(c->s, c->tables, dn, du, dT, (float2*)c->state[0], c->err);
+    else k2_init<double><<<nb, 256, 0, c->user>>>(c->s, c->tables, dn, du, dT, (double2*)c->state[0], c->err);
     if ((e = cudaGetLastError()) != cudaSuccess) return st2(e);
     return check_2d(c);
 }
@@ -1943,30 +2000,39 @@ evfdlb_status step_async_2d(Ctx2* c, int64_t nsteps) {
     return EVFDLB_OK;
 }
 
-evfdlb_status get_state_2d(Ctx2* c, double* F, double* G, int on_device) {
+// The interleaved state `src` as F and G: device arrays are written by the
+// splitting kernel itself, host arrays go through the scratch block.
+cudaError_t split_2d(Ctx2* c, const void* src, double* F, double* G, int on_device) {
     const long long NF = dist_2d(c);
-    const double* src = (const double*)c->state[0];
-    cudaError_t e = cudaSuccess;
-    if (c->prec == EVFDLB_FP32) {
-        k2_convert<float, double><<<4096, 256, 0, c->user>>>((const float*)c->state[0], c->scratch, 2 * NF);
-        src = c->scratch;
-        e = cudaGetLastError();
-    }
-    cudaMemcpyKind kd = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(F, src, sizeof(double) * NF, kd, c->user);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(G, src + NF, sizeof(double) * NF, kd, c->user);
+    double *dF = on_device ? F : c->scratch, *dG = on_device ? G : c->scratch + NF;
+    if (c->prec == EVFDLB_FP32) k2_split<float><<<4096, 256, 0, c->user>>>((const float2*)src, dF, dG, NF);
+    else k2_split<double><<<4096, 256, 0, c->user>>>((const double2*)src, dF, dG, NF);
+    cudaError_t e = cudaGetLastError();
+    if (on_device) return e;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(F, dF, sizeof(double) * NF, cudaMemcpyDeviceToHost, c->user);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(G, dG, sizeof(double) * NF, cudaMemcpyDeviceToHost, c->user);
+    return e;
+}
+
+evfdlb_status get_state_2d(Ctx2* c, double* F, double* G, int on_device) {
+    cudaError_t e = split_2d(c, c->state[0], F, G, on_device);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->user);
     return st2(e);
 }
 
 evfdlb_status set_state_2d(Ctx2* c, const double* F, const double* G, int on_device) {
     const long long NF = dist_2d(c);
-    double* dst = (c->prec == EVFDLB_FP32) ? c->scratch : (double*)c->state[0];
-    cudaMemcpyKind kd = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    cudaError_t e = cudaMemcpyAsync(dst, F, sizeof(double) * NF, kd, c->user);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(dst + NF, G, sizeof(double) * NF, kd, c->user);
-    if (e == cudaSuccess && c->prec == EVFDLB_FP32) {
-        k2_convert<double, float><<<4096, 256, 0, c->user>>>(c->scratch, (float*)c->state[0], 2 * NF);
+    cudaError_t e = cudaSuccess;
+    const double *dF = F, *dG = G;
+    if (!on_device) {
+        e = cudaMemcpyAsync(c->scratch, F, sizeof(double) * NF, cudaMemcpyHostToDevice, c->user);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(c->scratch + NF, G, sizeof(double) * NF, cudaMemcpyHostToDevice, c->user);
+        dF = c->scratch;
+        dG = c->scratch + NF;
+    }
+    if (e == cudaSuccess) {
+        if (c->prec == EVFDLB_FP32) k2_join<float><<<4096, 256, 0, c->user>>>(dF, dG, (float2*)c->state[0], NF);
+        else k2_join<double><<<4096, 256, 0, c->user>>>(dF, dG, (double2*)c->state[0], NF);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(c->err, 0, sizeof(unsigned), c->user);
@@ -1975,12 +2041,10 @@ evfdlb_status set_state_2d(Ctx2* c, const double* F, const double* G, int on_dev
 }
 
 evfdlb_status rhs_2d(Ctx2* c, double* RF, double* RG, int on_device) {
-    const long long NF = dist_2d(c);
-    queue_stage(c, c->user, c->state[0], nullptr, nullptr, c->scratch, 0.0, 1.0, 1);
+    // into the first intermediate state, which holds nothing between steps
+    queue_stage(c, c->user, c->state[0], nullptr, c->state[1], 0.0, 1.0, 1);
     cudaError_t e = cudaGetLastError();
-    cudaMemcpyKind kd = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(RF, c->scratch, sizeof(double) * NF, kd, c->user);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(RG, c->scratch + NF, sizeof(double) * NF, kd, c->user);
+    if (e == cudaSuccess) e = split_2d(c, c->state[1], RF, RG, on_device);
     if (e != cudaSuccess) return st2(e);
     return check_2d(c);
 }
@@ -1990,9 +2054,9 @@ evfdlb_status moments_2d(Ctx2* c, double* n, double* u, double* T, double* q, do
     int nb = (int)std::min<long long>((N + 255) / 256, 4096);
     const int nbm = moments_grid(N);
     if (c->prec == EVFDLB_FP32)
-        launch_moments<float>(c->s.Q, nbm, c->user, c->s, c->pwf, (const float*)c->state[0], c->mom, nullptr, c->err);
+        launch_moments<float>(c->s.Q, nbm, c->user, c->s, c->pwf, (const float2*)c->state[0], c->mom, nullptr, c->err);
     else
-        launch_moments<double>(c->s.Q, nbm, c->user, c->s, c->pwd, (const double*)c->state[0], c->mom, nullptr, c->err);
+        launch_moments<double>(c->s.Q, nbm, c->user, c->s, c->pwd, (const double2*)c->state[0], c->mom, nullptr, c->err);
     double* b = c->scratch;   // n [N], u [2N], T [N], q [2N], totals [4]
     double* dn = n ? (on_device ? n : b) : nullptr;
     double* du = u ? (on_device ? u : b + N) : nullptr;
