@@ -1119,12 +1119,6 @@ k2_coll_pipe(Slab2 s, const Par2<float> pr, const float2* __restrict__ st, const
 // on aligned tiles alone) took 345 us and 241 instructions, and 376 us against
 // now 128 us on a 333x250 grid, whose rows are not 16-byte aligned.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float rcp_ftz(float x) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
 // The WENO-5 walk of Weno5Run on pairs.  With g_0 = 2 s_0 - d_1,
 // g_1 = 6 (s_1 + d_2), g_2 = 3 (d_2 - s_2) (60 times the candidate
 // corrections times their linear weights) the face is

@@ -441,36 +441,6 @@ __device__ void split_state_tile(const SlabDesc& sd, const WorkItem& it, const S
     }
 }
 
-// The state tile (+-3 nodes) and the parity-split interior columns
-// EO[((d * 2 + par) * H + j) * Z + t]: E_j = h_j + h_{Q-1-j}, O_j = h_j - h_{Q-1-j}
-// (the middle node of an odd Q: E = h, O = 0).  Each thread loads a node
-// pair (j, Q-1-j) of one column.
-template <typename R>
-__device__ void load_state_tile_eo(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, int Z,
-                                   const R* __restrict__ src, long long NF) {
-    const int Q = sd.Q, nx = sd.nx, bc = sd.bc, W = Z + 6, H = (Q + 1) / 2;
-    const int cols = it.nz + 6;
-#pragma unroll 4
-    for (int e = threadIdx.x; e < 2 * H * cols; e += blockDim.x) {
-        const int c = e % cols, r = e / cols;
-        const int j = r % H, d = r / H, jm = Q - 1 - j;
-        const int i = gidx(it.i0 - 3 + c, nx, bc);
-        const R* row = src + d * NF + sd.f_off + i;
-        const R v = row[(long long)j * nx];
-        s.F[(d * Q + j) * W + c] = v;
-        R vm = R(0);
-        if (jm != j) {
-            vm = row[(long long)jm * nx];
-            s.F[(d * Q + jm) * W + c] = vm;
-        }
-        if (c >= 3 && c < it.nz + 3) {
-            R* eo = s.EO + ((size_t)(2 * d) * H + j) * Z + (c - 3);
-            eo[0] = (jm != j) ? v + vm : v;
-            eo[(size_t)H * Z] = (jm != j) ? v - vm : R(0);
-        }
-    }
-}
-
 // sum_{|j| <= m} tap[j + m] x[j] in four interleaved partial sums: a quarter
 // of the dependent chain (an FP64 operation waits for the whole warp to pass
 // the FP64 pipe of its scheduler, tens of cycles on this part).
@@ -663,8 +633,8 @@ __device__ void node_fields(const SlabDesc& sd, const WorkItem& it, const Smem<R
 //      c2 = 3/5 K D T,        c3 = nu kq/5 + 3/10 K B T^2
 //   G: c0 = nu n T + 2/5 K T D,  c1 = 2/5 nu kq + K T^2 (A + 3/5 B),
 //      c2 = 3/5 K T^2 D,         c3 = nu kq T/5 + 3/10 K T^3 B
-// node_coefficients forms the constants (FP64, stored in R) and the moments
-// m_l (recurrence in R) per node; coefficients() then forms every c_l in
+// node_coefficients or node_roles form the constants per node, hermite_moments
+// the m_l (recurrence in R); coefficients() then forms every c_l in
 // parallel and adds the force term F1 sqrt(l) a_{l-1}
 // (d/dxi [omega psi_{l-1}] = -sqrt(l) omega psi_l).
 // ---------------------------------------------------------------------------
@@ -690,43 +660,24 @@ __device__ __forceinline__ void hermite_moments(int Q, const TableLayout& L, con
     }
 }
 
-// MM: also the Hermite moments m_l of the local Gaussian (else another
-// group of warps forms them, node_hermite_moments).
-template <typename R, bool MM = true>
-__device__ void node_coefficients(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, int Z,
-                                  const R* __restrict__ tab, int tid, int nth) {
-    const int Q = sd.Q;
-    TableLayout L(Q);
+// The FP32 state forms the constants on the FP32 pipe (an FP64 state: node_roles).
+__device__ inline void node_coefficients(const SlabDesc& sd, const WorkItem& it, const Smem<float>& s, int Z, int tid,
+                                         int nth) {
     for (int t = tid; t < it.nz; t += nth) {
         const double* sc = s.Sc;
-        double n = sc[SC_N * Z + t], u = sc[SC_U * Z + t], T = sc[SC_T * Z + t];
-        double nu = sc[SC_NU * Z + t], kq = sc[SC_KQ * Z + t], K = sc[SC_K * Z + t];
-        double A = sc[SC_A * Z + t], B = sc[SC_B * Z + t], D = sc[SC_D * Z + t];
-        R* cF = s.Cc + t;
-        R* cG = s.Cc + 4 * Z + t;
-        if constexpr (std::is_same<R, float>::value) {
-            // the FP32 variant forms the constants on the FP32 pipe
-            const float fn = d2f_bits(n), fT = d2f_bits(T), fnu = d2f_bits(nu), fkq = d2f_bits(kq);
-            const float fK = d2f_bits(K), fA = d2f_bits(A), fB = d2f_bits(B), fD = d2f_bits(D);
-            cF[0] = fnu * fn;
-            cF[Z] = fK * fA * fT;
-            cF[2 * Z] = 0.6f * fK * fD * fT;
-            cF[3 * Z] = 0.2f * fnu * fkq + 0.3f * fK * fB * fT * fT;
-            cG[0] = fnu * fn * fT + 0.4f * fK * fT * fD;
-            cG[Z] = 0.4f * fnu * fkq + fK * fT * fT * (fA + 0.6f * fB);
-            cG[2 * Z] = 0.6f * fK * fT * fT * fD;
-            cG[3 * Z] = 0.2f * fnu * fkq * fT + 0.3f * fK * fT * fT * fT * fB;
-        } else {
-            cF[0] = (R)(nu * n);
-            cF[Z] = (R)(K * A * T);
-            cF[2 * Z] = (R)(0.6 * K * D * T);
-            cF[3 * Z] = (R)(0.2 * nu * kq + 0.3 * K * B * T * T);
-            cG[0] = (R)(nu * n * T + 0.4 * K * T * D);
-            cG[Z] = (R)(0.4 * nu * kq + K * T * T * (A + 0.6 * B));
-            cG[2 * Z] = (R)(0.6 * K * T * T * D);
-            cG[3 * Z] = (R)(0.2 * nu * kq * T + 0.3 * K * T * T * T * B);
-        }
-        if constexpr (MM) hermite_moments<R>(Q, L, tab, u, T, s.Mm + t, Z);
+        auto f = [&](int which) { return d2f_bits(sc[which * Z + t]); };
+        const float fn = f(SC_N), fT = f(SC_T), fnu = f(SC_NU), fkq = f(SC_KQ);
+        const float fK = f(SC_K), fA = f(SC_A), fB = f(SC_B), fD = f(SC_D);
+        float* cF = s.Cc + t;
+        float* cG = s.Cc + 4 * Z + t;
+        cF[0] = fnu * fn;
+        cF[Z] = fK * fA * fT;
+        cF[2 * Z] = 0.6f * fK * fD * fT;
+        cF[3 * Z] = 0.2f * fnu * fkq + 0.3f * fK * fB * fT * fT;
+        cG[0] = fnu * fn * fT + 0.4f * fK * fT * fD;
+        cG[Z] = 0.4f * fnu * fkq + fK * fT * fT * (fA + 0.6f * fB);
+        cG[2 * Z] = 0.6f * fK * fT * fT * fD;
+        cG[3 * Z] = 0.2f * fnu * fkq * fT + 0.3f * fK * fT * fT * fT * fB;
     }
 }
 
@@ -739,6 +690,226 @@ __device__ void node_hermite_moments(const SlabDesc& sd, const WorkItem& it, con
     const int Q = sd.Q;
     TableLayout L(Q);
     for (int t = tid; t < it.nz; t += nth) hermite_moments<R>(Q, L, tab, s.U[t + 2], s.T[t + 2], s.Mm + t, Z);
+}
+
+// ---------------------------------------------------------------------------
+// The node work of an FP64 stage, by the first four warps of the CTA (one per
+// scheduler: an FP64 instruction occupies its scheduler's pipe for 64 cycles
+// whatever the active lanes, so the chain of one node is as long as its
+// instruction count and only other schedulers shorten it):
+//   warp 0  Fischer-Methfessel average and chi; X; transport; the
+//           coefficient constants c0 .. c3;
+//   warp 1  u, T, q from the raw sums; the gradients;
+//   warp 2  the Hermite moments of the local Gaussian;
+//   warp 3  the force sums.
+// The transport is written in x = b n chi throughout, with P = 1 + 4/5 x +
+// c16 x^2 the factor that mu chi and Pr share:
+//   nu = n sqrt(T) chi (1 + 2/5 x) / (mu0 P)  (times chi for the rate chi/tau),
+//   Pr = 2/3 (1 + 3/5 x) P / ((1 + 2/5 x) (1 + 6/5 x + c9 x^2)),
+// and q = S3/2 + G1 - u (3/2 S2 + G0 - u S1).  On tiles of a few nodes this
+// chain is the stage: about 100 FP64 instructions on its longest warp, where
+// one warp with everything took 260 (dx = 0.25, Q = 16) to 400: a stage of
+// 256 x 16 takes 12.5 us instead of 18.4, of 2000 x 16 (EV2) 15.9 instead of
+// 21.0, of 1024 x 24 16.6 instead of 22.5.
+// Every sum has a fixed order, so results do not depend on the tile.
+// ---------------------------------------------------------------------------
+// Raw sums for the roles: n on the density halo; S1, S2, G0 on +-2 nodes (in
+// the U, T and X arrays), S3 and G1 of the tile (in the KQ and A scalars).
+template <bool CG>
+__device__ void load_raw_sums(const SlabDesc& sd, const WorkItem& it, const Smem<double>& s, int Z,
+                              const double* __restrict__ mom, long long NN) {
+    const int M = sd.M, nx = sd.nx, bc = sd.bc;
+    const double* m = mom + sd.node_off;
+#pragma unroll 2
+    for (int t = threadIdx.x; t < it.nz + 2 * M; t += blockDim.x)
+        s.N[t] = gload<CG>(m + MOM_S0 * NN + gidx(it.i0 - M + t, nx, bc));
+    for (int t = (int)blockDim.x - 1 - (int)threadIdx.x; t < it.nz + 4; t += blockDim.x) {
+        const int i = gidx(it.i0 - 2 + t, nx, bc);
+        const bool tile = (t >= 2 && t < it.nz + 2);
+        const double s1 = gload<CG>(m + MOM_S1 * NN + i), s2 = gload<CG>(m + MOM_S2 * NN + i);
+        const double g0 = gload<CG>(m + MOM_G0 * NN + i);
+        const double s3 = tile ? gload<CG>(m + MOM_S3 * NN + i) : 0.0, g1 = tile ? gload<CG>(m + MOM_G1 * NN + i) : 0.0;
+        s.U[t] = s1;
+        s.T[t] = s2;
+        s.X[t] = g0;
+        if (tile) {
+            s.Sc[SC_KQ * Z + t - 2] = s3;
+            s.Sc[SC_A * Z + t - 2] = g1;
+        }
+    }
+}
+
+// sum_j tap[j] x[j], j < n, in C chains over j mod C joined pairwise, by lp
+// neighbouring lanes per sum (lp <= C a power of two; sub = the lane's index
+// among them): the same operations and order for every lp.
+template <int C, int PER>
+__device__ __forceinline__ double chain_sum_t(const double* __restrict__ tap, const double* x, int n, int sub) {
+    double a[PER];                                 // chains sub PER .. sub PER + PER - 1
+#pragma unroll
+    for (int c = 0; c < PER; ++c) a[c] = 0.0;
+    int j = sub * PER;
+    for (; j + PER <= n; j += C) {
+#pragma unroll
+        for (int c = 0; c < PER; ++c) a[c] = fma(tap[j + c], x[j + c], a[c]);
+    }
+#pragma unroll
+    for (int c = 0; c < PER; ++c)
+        if (j + c < n) a[c] = fma(tap[j + c], x[j + c], a[c]);
+#pragma unroll
+    for (int w = 1; w < PER; w *= 2)
+#pragma unroll
+        for (int c = 0; c < PER; c += 2 * w) a[c] += a[c + w];
+#pragma unroll
+    for (int w = 1; w < C / PER; w *= 2) a[0] += __shfl_xor_sync(0xffffffffu, a[0], w);
+    return a[0];
+}
+template <int C>
+__device__ __forceinline__ double chain_sum(const double* __restrict__ tap, const double* x, int n, int lp, int sub) {
+    if (lp == 1) return chain_sum_t<C, C>(tap, x, n, sub);
+    if (lp == 2) return chain_sum_t<C, C / 2>(tap, x, n, sub);
+    if (C == 4 || lp == 4) return chain_sum_t<C, C / 4>(tap, x, n, sub);
+    return chain_sum_t<C, (C >= 8 ? C / 8 : 1)>(tap, x, n, sub);
+}
+// lanes per sum for n sums on one warp
+__device__ __forceinline__ int lanes_per(int n, int most) {
+    int lp = 1;
+    while (lp < most && 2 * lp * n <= 32) lp *= 2;
+    return lp;
+}
+
+template <bool FO>
+__device__ void node_roles(const SlabDesc& sd, const WorkItem& it, const Smem<double>& s, int Z,
+                           const double* __restrict__ tab, long long NN, unsigned* err, double* fields_out) {
+    const int M = sd.M, nz = it.nz, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double* sc = s.Sc;
+    auto join3 = [] { asm volatile("bar.sync 1, 96;" ::: "memory"); };    // warps 0, 1, 2
+    auto join2 = [] { asm volatile("bar.sync 4, 64;" ::: "memory"); };    // warps 0, 1
+    auto field = [&](int f, int t, double v) {
+        if constexpr (FO) fields_out[f * NN + sd.node_off + it.i0 + t] = v;
+    };
+    auto node_ok = [&](int t) { return positive(s.N[t + M]) && positive(s.T[t + 2]); };
+    if (warp == 0) {
+        // Under the outflow rule a ghost node copies every field of the
+        // nearest interior node: the average is centred on the clamped node.
+        const int lp = lanes_per(nz + 4, 4), sub = lane % lp;
+        for (int t0 = 0; t0 < nz + 4; t0 += 32 / lp) {
+            const int t = min(t0 + lane / lp, nz + 3), pos = it.i0 - 2 + t;
+            const int shift = (sd.bc == EVFDLB_BC_OUTFLOW) ? gidx(pos, sd.nx, sd.bc) - pos : 0;
+            const double nb = chain_sum<4>(s.Mtap, s.N + (t - 2 + M + shift - sd.m), 2 * sd.m + 1, lp, sub);
+            const double eta = sd.eta_coef * nb, om = 1.0 - eta;
+            const double chi = div_nr(2.0 - eta, 2.0 * om * om * om);
+            if (sub == 0) {
+                s.Chi[t] = chi;
+                if (t >= 2 && t < nz + 2) field(4, t - 2, nb);
+            }
+        }
+        join3();
+        for (int t = lane; t < nz + 4; t += 32) {
+            const int pos = it.i0 - 2 + t;
+            const int shift = (sd.bc == EVFDLB_BC_OUTFLOW) ? gidx(pos, sd.nx, sd.bc) - pos : 0;
+            const double n = s.N[t - 2 + M + shift];
+            s.X[t] = n * n * s.Chi[t] * s.T[t];
+        }
+        join2();
+        for (int t = lane; t < nz; t += 32) {
+            const double n = s.N[t + M], T = s.T[t + 2], chi = s.Chi[t + 2], q = sc[SC_KQ * Z + t];
+            const double c16 = (4.0 / 25.0) * (1.0 + 12.0 / M_PI), c9 = (9.0 / 25.0) * (1.0 + 32.0 / (9.0 * M_PI));
+            const double x = sd.b * n * chi, a = fma(0.4, x, 1.0), P = fma(fma(c16, x, 0.8), x, 1.0), st = sqrt(T);
+            double nu = div_nr(n * st * chi * a, sd.mu0_coef * P);
+            if (sd.relax != EVFDLB_RELAX_INV_TAU) nu *= chi;
+            const double Pr = div_nr(fma(0.4, x, 2.0 / 3.0) * P, a * fma(fma(c9, x, 1.2), x, 1.0));
+            sc[SC_N * Z + t] = n;
+            sc[SC_T * Z + t] = T;
+            sc[SC_NU * Z + t] = nu;
+            sc[SC_KQ * Z + t] = (1.0 - Pr) * q;
+            sc[SC_K * Z + t] = -x * n;               // -b n^2 chi, the prefactor of J1
+            s.Scr[t] = nu;
+            if (!positive(n) || !positive(T)) atomicOr(err, (finite(n) && finite(T)) ? ERR_NEGATIVE : ERR_NONFINITE);
+            else if (!finite(nu) || !finite(q)) atomicOr(err, ERR_NONFINITE);
+            if constexpr (FO) {
+                const double mu = sd.mu0_coef * st * div_nr(P, chi);
+                field(0, t, n);
+                field(1, t, s.U[t + 2]);
+                field(2, t, T);
+                field(3, t, q);
+                field(5, t, chi);
+                field(7, t, mu);
+                field(8, t, div_nr(mu, n * T * a));
+                field(9, t, Pr);
+                field(10, t, nu);
+                field(14, t, s.X[t + 2]);
+                field(15, t, x);
+            }
+        }
+        join2();
+        // c0 .. c3 of both distributions (see node_coefficients)
+        for (int t = lane; t < nz; t += 32) {
+            const double n = sc[SC_N * Z + t], T = sc[SC_T * Z + t], nu = sc[SC_NU * Z + t];
+            const double kq = sc[SC_KQ * Z + t], K = sc[SC_K * Z + t];
+            const double A = sc[SC_A * Z + t], B = sc[SC_B * Z + t], D = sc[SC_D * Z + t];
+            const double KT = K * T, KT2 = KT * T, KTD = KT * D, nk = nu * kq;
+            const double f0 = nu * n, f2 = 0.6 * KTD, f3 = fma(0.3 * KT2, B, 0.2 * nk);
+            double* cF = s.Cc + t;
+            double* cG = s.Cc + 4 * Z + t;
+            cF[0] = f0;
+            cF[Z] = KT * A;
+            cF[2 * Z] = f2;
+            cF[3 * Z] = f3;
+            cG[0] = fma(f0, T, 0.4 * KTD);
+            cG[Z] = fma(KT2, fma(0.6, B, A), 0.4 * nk);
+            cG[2 * Z] = f2 * T;
+            cG[3 * Z] = f3 * T;
+        }
+    } else if (warp == 1) {
+        for (int t = lane; t < nz + 4; t += 32) {
+            const bool tile = (t >= 2 && t < nz + 2);
+            const int pos = it.i0 - 2 + t;
+            const int shift = (sd.bc == EVFDLB_BC_OUTFLOW) ? gidx(pos, sd.nx, sd.bc) - pos : 0;
+            const double n = s.N[t - 2 + M + shift], s1 = s.U[t], s2 = s.T[t], g0 = s.X[t];
+            const double inv_n = div_nr(1.0, n), u = s1 * inv_n;
+            s.U[t] = u;
+            // (3/2) n T = sum (xi-u)^2/2 F + sum G = S2/2 + G0 - n u^2/2
+            s.T[t] = (2.0 / 3.0) * fma(fma(0.5, s2, g0), inv_n, -0.5 * u * u);
+            if (tile) {
+                const double s3 = sc[SC_KQ * Z + t - 2], g1 = sc[SC_A * Z + t - 2];
+                sc[SC_KQ * Z + t - 2] = fma(-u, fma(-u, s1, fma(1.5, s2, g0)), fma(0.5, s3, g1));
+            }
+        }
+        join3();
+        const double inv12 = sd.inv_dx / 12.0;
+        // fourth-order central differences (Sec. III)
+        auto d4 = [&](const double* f) { return fma(8.0, f[1] - f[-1], f[-2] - f[2]) * inv12; };
+        for (int t = lane; t < nz; t += 32) {
+            sc[SC_D * Z + t] = d4(s.U + t + 2);
+            sc[SC_B * Z + t] = div_nr(d4(s.T + t + 2), s.T[t + 2]);
+        }
+        join2();
+        for (int t = lane; t < nz; t += 32) {
+            const double A = div_nr(d4(s.X + t + 2), s.X[t + 2]), B = sc[SC_B * Z + t];
+            sc[SC_A * Z + t] = A;
+            if (node_ok(t) && (!finite(A) || !finite(B))) atomicOr(err, ERR_NONFINITE);
+            field(11, t, A);
+            field(12, t, B);
+            field(13, t, sc[SC_D * Z + t]);
+        }
+        join2();
+    } else if (warp == 2) {
+        join3();
+        TableLayout L(sd.Q);
+        for (int t = lane; t < nz; t += 32) hermite_moments<double>(sd.Q, L, tab, s.U[t + 2], s.T[t + 2], s.Mm + t, Z);
+    } else {
+        // self-consistent force, Eq. (F1) (or the merged Eq. (F2) stencil)
+        const int lp = lanes_per(nz, 8), sub = lane % lp;
+        for (int t0 = 0; t0 < nz; t0 += 32 / lp) {
+            const int t = min(t0 + lane / lp, nz - 1);
+            const double f1 = chain_sum<8>(s.Ftap, s.N + t, 2 * M + 1, lp, sub);
+            if (sub == 0) {
+                s.Scr[Z + t] = f1;
+                if (!finite(f1)) atomicOr(err, ERR_NONFINITE);
+                field(6, t, f1);
+            }
+        }
+    }
 }
 
 // With DF the coefficients are stored as double-float pairs (float2) in the
@@ -773,6 +944,20 @@ __device__ void coefficients(const SlabDesc& sd, const WorkItem& it, const Smem<
     }
 }
 
+// Warp-sized groups of e = 0 .. n-1 from a shared counter (zeroed before), for
+// warps that arrive at different times: f(e) for every e, by one lane each.
+template <typename F>
+__device__ __forceinline__ void warp_pool(int* next, int n, F f) {
+    const int lane = threadIdx.x & 31;
+    for (;;) {
+        int g = 0;
+        if (lane == 0) g = atomicAdd(next, 1);
+        g = __shfl_sync(0xffffffffu, g, 0) * 32;
+        if (g >= n) return;
+        if (g + lane < n) f(g + lane);
+    }
+}
+
 // Analysis a_l = sum_j psi_l(xi_j) h_j, l <= Q-2 (the force needs
 // a_0 .. a_{Q-2}; the l = Q-1 term meets psi_Q(xi_k) = 0), two orders per
 // thread so that each state value loaded feeds two FMAs.
@@ -802,14 +987,16 @@ __device__ void analysis(const SlabDesc& sd, const WorkItem& it, const Smem<R>& 
 // Parity-split analysis: a_l = sum_{j<H} psi_l(xi_j) (E_j or O_j), l <= Q-2,
 // two orders of one parity (l, l+2) per thread sharing each E/O value loaded
 // (Pp holds the two table values side by side: one two-wide load).
+// Threads tid, tid + nth, ... (next null), or whole warps from the pool `next`.
 template <typename R>
-__device__ void analysis_eo(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, int Z, int tid, int nth) {
+__device__ void analysis_eo(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, int Z, int tid, int nth,
+                            int* next = nullptr) {
     using R2 = typename std::conditional<std::is_same<R, float>::value, float2, double2>::type;
     const int Q = sd.Q, nz = it.nz;
     const ParitySplit ps(Q);
     const int H = ps.H, G = ps.GE + ps.GO;
     const R2* Pp = reinterpret_cast<const R2*>(s.P);
-    for (int e = tid; e < 2 * G * nz; e += nth) {
+    auto task = [&](int e) {
         const int t = e % nz, r = e / nz;
         const int g = r % G, d = r / G;
         const int par = g < ps.GE ? 0 : 1;
@@ -825,7 +1012,10 @@ __device__ void analysis_eo(const SlabDesc& sd, const WorkItem& it, const Smem<R
         }
         s.A[((size_t)d * Q + l0) * Z + t] = a0;
         if (l0 + 2 <= Q - 2) s.A[((size_t)d * Q + l0 + 2) * Z + t] = a1;
-    }
+    };
+    if (next) warp_pool(next, 2 * G * nz, task);
+    else
+        for (int e = tid; e < 2 * G * nz; e += nth) task(e);
 }
 
 // Analysis in double-float: the state tile is split into pairs when it is
@@ -833,11 +1023,11 @@ __device__ void analysis_eo(const SlabDesc& sd, const WorkItem& it, const Smem<R
 // orders per thread (four independent accumulator chains, each pair loaded
 // feeding four terms), joined to FP64 for the coefficients.
 __device__ inline void analysis_df(const SlabDesc& sd, const WorkItem& it, const Smem<double>& s, const float2* Fd,
-                                   const float2* P, int Z, int tid, int nth) {
+                                   const float2* P, int Z, int* next) {
     const int Q = sd.Q, nz = it.nz;
     const int nq = Q / 4;                          // quads of orders covering l <= Q-2 (Q even)
     const int per_d = nq * nz;
-    for (int e = tid; e < 2 * per_d; e += nth) {
+    warp_pool(next, 2 * per_d, [&](int e) {
         int d = e / per_d, r = e % per_d;
         int l0 = 4 * (r / nz), t = r % nz;
         const int nl = min(4, Q - 1 - l0);         // orders l0 .. l0+nl-1 (<= Q-2)
@@ -859,7 +1049,7 @@ __device__ inline void analysis_df(const SlabDesc& sd, const WorkItem& it, const
         if (nl > 1) A[Z] = df_join(s1, e1);
         if (nl > 2) A[2 * Z] = df_join(s2, e2);
         if (nl > 3) A[3 * Z] = df_join(s3, e3);
-    }
+    });
 }
 
 // WENO-5 (Jiang & Shu) faces in difference form, along a run of faces.
@@ -967,13 +1157,29 @@ __device__ void faces(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, 
 }
 
 // ---------------------------------------------------------------------------
-// Double-float arithmetic for the FP64_DF faces: a value is an unevaluated
-// pair hi + lo of floats (about 48 significant bits).  Addition is Knuth's
-// TwoSum with the low parts folded in and one renormalisation (Dekker's
-// FastTwoSum); multiplication is the FMA TwoProduct with the cross terms;
-// the quotient takes the float reciprocal of the divisor's head and two
-// remainder corrections (each adds ~24 bits).  __fadd_rn / __fmul_rn keep
-// the compiler from contracting the error-free transformations.
+// WENO-5 faces of an FP64 state, split between the pipes.  The FP64 pipe of
+// this part takes a warp instruction per scheduler every 64 cycles, the FP32
+// pipe one per cycle.  With p = a_0 - a_1, q = a_2 - a_1 and the differences
+// dd_0 = t_1 - t_0, dd_1 = t_2 - t_1 (third differences of h) the face of
+// Weno5Run is
+//   v2 + (-2 d0 + 11 d1 + 24 d2 - 3 d3) / 60                 (linear weights)
+//      + (p (dd_1 - 6 dd_0) + q (2 dd_0 - 7 dd_1)) / (20 (a_0 + 6 a_1 + 3 a_2)),
+// an identity.  The first line and the e_r are FP64; the rest of the second,
+// which vanishes with the third differences, is double-float arithmetic on
+// the FP32 pipe (pairs hi + lo from the e_r and t_r; normalised products and
+// sums, about 2^-47 each).  17 FP64 operations a face, with its share of a
+// cell's, instead of 31.
+// The error of a face against extended precision is that of the FP64 form
+// or below on smooth profiles (its quotient is good to 2^-46 of the whole
+// difference; 100 000 samples of tanh profiles of every steepness), within
+// 4 % of it on grid-scale noise of 1 % of the value, 1.3 times at 3 %; one step
+// of noisy and liquid slabs, Q = 16 .. 32, against 80-bit arithmetic is equally
+// near in both forms (1.1e-16).  Stage of 4096 x 32: 50.6 -> 46.2 us, of
+// 65536 x 24 (tile 32): 520 -> 439 us.
+//
+// The e_r are scaled by a power of two to max(e_r) in [1, 2), so that a_r
+// stays in range whatever the size of the state or of eps; a face whose
+// max(e_r) leaves the float range takes the FP64 form.
 // ---------------------------------------------------------------------------
 struct dfl {
     float h, l;
@@ -982,15 +1188,171 @@ __device__ __forceinline__ dfl dfl_of(double x) {
     const float2 p = df_split(x);
     return {p.x, p.y};
 }
+__device__ __forceinline__ dfl dfl_norm(float h, float l) {
+    const float s = __fadd_rn(h, l);
+    return {s, __fsub_rn(l, __fsub_rn(s, h))};
+}
+// sums (Knuth's TwoSum, low parts folded in), not normalised
 __device__ __forceinline__ dfl dfl_add(dfl a, dfl b) {
+    const float s = __fadd_rn(a.h, b.h), bb = __fsub_rn(s, a.h);
+    const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, bb)), __fsub_rn(b.h, bb));
+    return {s, __fadd_rn(e, __fadd_rn(a.l, b.l))};
+}
+__device__ __forceinline__ dfl dfl_sub(dfl a, dfl b) {
+    const float s = __fsub_rn(a.h, b.h), bb = __fsub_rn(s, a.h);
+    const float e = __fsub_rn(__fsub_rn(a.h, __fsub_rn(s, bb)), __fadd_rn(b.h, bb));
+    return {s, __fadd_rn(e, __fsub_rn(a.l, b.l))};
+}
+__device__ __forceinline__ dfl dfl_norm(dfl a) { return dfl_norm(a.h, a.l); }
+// products (the FMA's TwoProduct and all cross terms), normalised
+__device__ __forceinline__ dfl dfl_mul(dfl a, dfl b) {
+    const float p = __fmul_rn(a.h, b.h);
+    return dfl_norm(p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.l, __fmaf_rn(a.h, b.h, -p)))));
+}
+__device__ __forceinline__ dfl dfl_sqr(dfl a) {
+    const float p = __fmul_rn(a.h, a.h);
+    return dfl_norm(p, __fmaf_rn(__fadd_rn(a.h, a.h), a.l, __fmaf_rn(a.l, a.l, __fmaf_rn(a.h, a.h, -p))));
+}
+// times a small integer, not normalised; times a power of two
+__device__ __forceinline__ dfl dfl_muli(dfl a, float b) {
+    const float p = __fmul_rn(a.h, b);
+    return {p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p))};
+}
+__device__ __forceinline__ dfl dfl_scale(dfl a, float b) { return {__fmul_rn(a.h, b), __fmul_rn(a.l, b)}; }
+__device__ __forceinline__ float rcp_ftz(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// The face of Weno5Run from its differences, in FP64 (the range fallback).
+static __device__ __noinline__ double weno5_face_f64(double v2, double d0, double d1, double d2, double d3, double eps) {
+    Weno5Run<double> w;
+    w.v2 = v2;
+    w.eps4 = 4.0 * eps;
+    w.d0 = d0;
+    w.d1 = d1;
+    w.d2 = d2;
+    w.d3 = d3;
+    w.u0 = w.tterm(d1 - d0);
+    w.u1 = w.tterm(d2 - d1);
+    w.u2 = w.tterm(d3 - d2);
+    return w.face();
+}
+
+// The run of Weno5Run on the split form.
+struct Weno5Split {
+    double v2, v3, v4, d0, d1, d2, d3, u0, u1, u2, eps4;   // u_r = 13/3 t_r^2 + 4 eps
+    dfl T2, dd0, dd1;                                      // T2: t_2 as a pair
+    __device__ __forceinline__ double tterm(double t) const { return fma((13.0 / 3.0) * t, t, eps4); }
+    __device__ __forceinline__ void start(double w0, double w1, double w2, double w3, double w4, double eps) {
+        eps4 = 4.0 * eps;
+        v2 = w2;
+        v3 = w3;
+        v4 = w4;
+        d0 = w1 - w0;
+        d1 = w2 - w1;
+        d2 = w3 - w2;
+        d3 = w4 - w3;
+        const double t0 = d1 - d0, t1 = d2 - d1, t2 = d3 - d2;
+        u0 = tterm(t0);
+        u1 = tterm(t1);
+        u2 = tterm(t2);
+        const dfl T0 = dfl_of(t0), T1 = dfl_of(t1);
+        T2 = dfl_of(t2);
+        dd0 = dfl_sub(T1, T0);
+        dd1 = dfl_sub(T2, T1);
+    }
+    __device__ __forceinline__ double face(double eps) const {
+        const double s0 = fma(3.0, d1, -d0), s1 = d1 + d2, s2 = fma(-3.0, d2, d3);
+        dfl e0 = dfl_of(fma(s0, s0, u0)), e1 = dfl_of(fma(s1, s1, u1)), e2 = dfl_of(fma(s2, s2, u2));
+        const float m = fmaxf(e0.h, fmaxf(e1.h, e2.h));
+        if (!(m > 1e-30f && m < 1e37f)) return weno5_face_f64(v2, d0, d1, d2, d3, eps);
+        const float sc = __int_as_float(0x7f000000 - (__float_as_int(m) & 0x7f800000));   // 2^-exponent(m)
+        e0 = dfl_scale(e0, sc);
+        e1 = dfl_scale(e1, sc);
+        e2 = dfl_scale(e2, sc);
+        const dfl E0 = dfl_sqr(e0), E1 = dfl_sqr(e1), E2 = dfl_sqr(e2);
+        const dfl a0 = dfl_mul(E1, E2), a1 = dfl_mul(E0, E2), a2 = dfl_mul(E0, E1);
+        const dfl p = dfl_norm(dfl_sub(a0, a1)), q = dfl_norm(dfl_sub(a2, a1));
+        const dfl A = dfl_norm(dfl_sub(dd1, dfl_muli(dd0, 6.f)));
+        const dfl B = dfl_norm(dfl_sub(dfl_scale(dd0, 2.f), dfl_muli(dd1, 7.f)));
+        const dfl num = dfl_norm(dfl_add(dfl_mul(p, A), dfl_mul(q, B)));
+        const dfl den = dfl_norm(dfl_add(a0, dfl_add(dfl_muli(a1, 6.f), dfl_muli(a2, 3.f))));
+        const float r = rcp_ftz(den.h);
+        const float q1 = __fmul_rn(num.h, r);
+        const float q2 = __fmul_rn(__fmaf_rn(-q1, den.l, __fadd_rn(__fmaf_rn(-q1, den.h, num.h), num.l)), r);
+        const double lin = fma(24.0 / 60.0, d2, fma(11.0 / 60.0, d1, fma(-3.0 / 60.0, d3, (-2.0 / 60.0) * d0)));
+        return v2 + fma(0.05, f2d_bits(q1) + f2d_bits(q2), lin);
+    }
+    __device__ __forceinline__ void shift(double w5) {
+        const double d4 = w5 - v4, t = d4 - d3;
+        d0 = d1;
+        d1 = d2;
+        d2 = d3;
+        d3 = d4;
+        u0 = u1;
+        u1 = u2;
+        u2 = tterm(t);
+        const dfl T = dfl_of(t);
+        dd0 = dd1;
+        dd1 = dfl_sub(T, T2);
+        T2 = T;
+        v2 = v3;
+        v3 = v4;
+        v4 = w5;
+    }
+};
+
+// faces() of an FP64 state: the same runs and walk, the split form, taken by
+// whole warps from the pool `next`.
+__device__ inline void faces_split(const SlabDesc& sd, const WorkItem& it, const Smem<double>& s, int Z,
+                                   const double* __restrict__ tab, int* next) {
+    const int Q = sd.Q, W = Z + 6, nf = it.nz + 1, rows = 2 * Q;
+    const int nruns = (nf + kRun - 1) / kRun;
+    TableLayout L(Q);
+    const double* xi = tab + sd.tab_off + L.xi;
+    warp_pool(next, rows * nruns, [&](int e) {
+        const int r = e % rows, run = e / rows;
+        const int k = r % Q;
+        const int fa = run * kRun, n = min(kRun, nf - fa), fl = fa + n - 1;
+        const bool pos = __double_as_longlong(xi[k]) >= 0 || !nonzero(xi[k]);
+        const int dir = pos ? 1 : -1, f0 = pos ? fa : fl;
+        const double* hb = s.F + (size_t)r * W + (pos ? fa : fl + 5);
+        double* out = s.Face + (size_t)r * (Z + 1);
+        Weno5Split w;
+        w.start(hb[0], hb[dir], hb[2 * dir], hb[3 * dir], hb[4 * dir], sd.weno_eps);
+#pragma unroll
+        for (int q = 0; q < kRun; ++q) {
+            if (q >= n) break;
+            out[f0 + dir * q] = w.face(sd.weno_eps);
+            if (q + 1 < n) w.shift(hb[dir * (q + 5)]);
+        }
+    });
+}
+
+// ---------------------------------------------------------------------------
+// Double-float arithmetic of the FP64_DF faces (every operation normalised): a
+// value is an unevaluated pair hi + lo of floats (about 48 significant bits).  Addition is Knuth's
+// TwoSum with the low parts folded in and one renormalisation (Dekker's
+// FastTwoSum); multiplication is the FMA TwoProduct with the cross terms;
+// the quotient takes the float reciprocal of the divisor's head and two
+// remainder corrections (each adds ~24 bits).  __fadd_rn / __fmul_rn keep
+// the compiler from contracting the error-free transformations.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ dfl dfn_of(double x) {
+    const float2 p = df_split(x);
+    return {p.x, p.y};
+}
+__device__ __forceinline__ dfl dfn_add(dfl a, dfl b) {
     const float s = __fadd_rn(a.h, b.h), bb = __fsub_rn(s, a.h);
     const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, bb)), __fsub_rn(b.h, bb));
     const float t = __fadd_rn(e, __fadd_rn(a.l, b.l));
     const float h = __fadd_rn(s, t);
     return {h, __fsub_rn(t, __fsub_rn(h, s))};
 }
-__device__ __forceinline__ dfl dfl_sub(dfl a, dfl b) { return dfl_add(a, {-b.h, -b.l}); }
-__device__ __forceinline__ dfl dfl_mul(dfl a, dfl b) {
+__device__ __forceinline__ dfl dfn_sub(dfl a, dfl b) { return dfn_add(a, {-b.h, -b.l}); }
+__device__ __forceinline__ dfl dfn_mul(dfl a, dfl b) {
     const float p = __fmul_rn(a.h, b.h);
     float e = fmaf(a.h, b.h, -p);
     e = fmaf(a.h, b.l, e);
@@ -999,26 +1361,26 @@ __device__ __forceinline__ dfl dfl_mul(dfl a, dfl b) {
     return {h, __fsub_rn(e, __fsub_rn(h, p))};
 }
 // times a float (exact small integers such as 3)
-__device__ __forceinline__ dfl dfl_mulf(dfl a, float b) {
+__device__ __forceinline__ dfl dfn_mulf(dfl a, float b) {
     const float p = __fmul_rn(a.h, b);
     float e = fmaf(a.h, b, -p);
     e = fmaf(a.l, b, e);
     const float h = __fadd_rn(p, e);
     return {h, __fsub_rn(e, __fsub_rn(h, p))};
 }
-__device__ __forceinline__ dfl dfl_div(dfl a, dfl b) {
+__device__ __forceinline__ dfl dfn_div(dfl a, dfl b) {
     const float r = __frcp_rn(b.h);
     const float q1 = __fmul_rn(a.h, r);
-    const dfl r1 = dfl_sub(a, dfl_mulf(b, q1));
+    const dfl r1 = dfn_sub(a, dfn_mulf(b, q1));
     const float q2 = __fmul_rn(r1.h, r);
-    const dfl r2 = dfl_sub(r1, dfl_mulf(b, q2));
+    const dfl r2 = dfn_sub(r1, dfn_mulf(b, q2));
     const float q3 = __fmul_rn(r2.h, r);
     const float s = __fadd_rn(q1, q2), bb = __fsub_rn(s, q1);
     const float e = __fadd_rn(__fsub_rn(q1, __fsub_rn(s, bb)), __fsub_rn(q2, bb));
-    return dfl_add({s, e}, {q3, 0.0f});
+    return dfn_add({s, e}, {q3, 0.0f});
 }
 // the constants of the difference-form WENO-5 face as pairs
-__device__ __forceinline__ dfl dfl_const(double x) {
+__device__ __forceinline__ dfl dfn_const(double x) {
     const float h = (float)x;
     return {h, (float)(x - (double)h)};
 }
@@ -1027,43 +1389,43 @@ __device__ __forceinline__ dfl dfl_const(double x) {
 struct Weno5RunDF {
     dfl v2, v3, v4, d0, d1, d2, d3, u0, u1, u2;
     dfl eps4, k133;
-    __device__ __forceinline__ dfl tterm(dfl t) const { return dfl_add(dfl_mul(dfl_mul(k133, t), t), eps4); }
+    __device__ __forceinline__ dfl tterm(dfl t) const { return dfn_add(dfn_mul(dfn_mul(k133, t), t), eps4); }
     // eps4 = 4 eps as a pair (formed once per thread by the caller)
     __device__ __forceinline__ void start(double w0, double w1, double w2, double w3, double w4, dfl e4) {
         eps4 = e4;
-        k133 = dfl_const(13.0 / 3.0);
-        const dfl a0 = dfl_of(w0), a1 = dfl_of(w1);
-        v2 = dfl_of(w2);
-        v3 = dfl_of(w3);
-        v4 = dfl_of(w4);
-        d0 = dfl_sub(a1, a0);
-        d1 = dfl_sub(v2, a1);
-        d2 = dfl_sub(v3, v2);
-        d3 = dfl_sub(v4, v3);
-        u0 = tterm(dfl_sub(d1, d0));
-        u1 = tterm(dfl_sub(d2, d1));
-        u2 = tterm(dfl_sub(d3, d2));
+        k133 = dfn_const(13.0 / 3.0);
+        const dfl a0 = dfn_of(w0), a1 = dfn_of(w1);
+        v2 = dfn_of(w2);
+        v3 = dfn_of(w3);
+        v4 = dfn_of(w4);
+        d0 = dfn_sub(a1, a0);
+        d1 = dfn_sub(v2, a1);
+        d2 = dfn_sub(v3, v2);
+        d3 = dfn_sub(v4, v3);
+        u0 = tterm(dfn_sub(d1, d0));
+        u1 = tterm(dfn_sub(d2, d1));
+        u2 = tterm(dfn_sub(d3, d2));
     }
     __device__ __forceinline__ double face() const {
-        const dfl s0 = dfl_sub(dfl_mulf(d1, 3.0f), d0), s1 = dfl_add(d1, d2), s2 = dfl_sub(d3, dfl_mulf(d2, 3.0f));
-        const dfl e0 = dfl_add(dfl_mul(s0, s0), u0), e1 = dfl_add(dfl_mul(s1, s1), u1), e2 = dfl_add(dfl_mul(s2, s2), u2);
-        const dfl E0 = dfl_mul(e0, e0), E1 = dfl_mul(e1, e1), E2 = dfl_mul(e2, e2);
-        const dfl a0 = dfl_mul(E1, E2), a1 = dfl_mul(E0, E2), a2 = dfl_mul(E0, E1);
-        const dfl c0 = dfl_sub(dfl_mul(dfl_const(5.0 / 60.0), d1), dfl_mul(dfl_const(2.0 / 60.0), d0));
-        const dfl c1 = dfl_add(dfl_mul(dfl_const(0.2), d2), dfl_mul(dfl_const(0.1), d1));
-        const dfl c2 = dfl_sub(dfl_mul(dfl_const(0.2), d2), dfl_mul(dfl_const(0.05), d3));
-        const dfl num = dfl_add(dfl_add(dfl_mul(a0, c0), dfl_mul(a1, c1)), dfl_mul(a2, c2));
-        const dfl den = dfl_add(dfl_add(dfl_mul(dfl_const(0.1), a0), dfl_mul(dfl_const(0.6), a1)),
-                                dfl_mul(dfl_const(0.3), a2));
-        const dfl f = dfl_add(v2, dfl_div(num, den));
+        const dfl s0 = dfn_sub(dfn_mulf(d1, 3.0f), d0), s1 = dfn_add(d1, d2), s2 = dfn_sub(d3, dfn_mulf(d2, 3.0f));
+        const dfl e0 = dfn_add(dfn_mul(s0, s0), u0), e1 = dfn_add(dfn_mul(s1, s1), u1), e2 = dfn_add(dfn_mul(s2, s2), u2);
+        const dfl E0 = dfn_mul(e0, e0), E1 = dfn_mul(e1, e1), E2 = dfn_mul(e2, e2);
+        const dfl a0 = dfn_mul(E1, E2), a1 = dfn_mul(E0, E2), a2 = dfn_mul(E0, E1);
+        const dfl c0 = dfn_sub(dfn_mul(dfn_const(5.0 / 60.0), d1), dfn_mul(dfn_const(2.0 / 60.0), d0));
+        const dfl c1 = dfn_add(dfn_mul(dfn_const(0.2), d2), dfn_mul(dfn_const(0.1), d1));
+        const dfl c2 = dfn_sub(dfn_mul(dfn_const(0.2), d2), dfn_mul(dfn_const(0.05), d3));
+        const dfl num = dfn_add(dfn_add(dfn_mul(a0, c0), dfn_mul(a1, c1)), dfn_mul(a2, c2));
+        const dfl den = dfn_add(dfn_add(dfn_mul(dfn_const(0.1), a0), dfn_mul(dfn_const(0.6), a1)),
+                                dfn_mul(dfn_const(0.3), a2));
+        const dfl f = dfn_add(v2, dfn_div(num, den));
         return f2d_bits(f.h) + f2d_bits(f.l);
     }
     __device__ __forceinline__ void shift(double w5) {
-        const dfl v5 = dfl_of(w5);
-        const dfl d4 = dfl_sub(v5, v4);
+        const dfl v5 = dfn_of(w5);
+        const dfl d4 = dfn_sub(v5, v4);
         u0 = u1;
         u1 = u2;
-        u2 = tterm(dfl_sub(d4, d3));
+        u2 = tterm(dfn_sub(d4, d3));
         d0 = d1;
         d1 = d2;
         d2 = d3;
@@ -1077,13 +1439,13 @@ struct Weno5RunDF {
 // faces() of the FP64_DF kernel: the same runs and walk, the face values in
 // double-float arithmetic on the FP32 pipe, stored as FP64.
 __device__ inline void faces_df(const SlabDesc& sd, const WorkItem& it, const Smem<double>& s, int Z,
-                                const double* __restrict__ tab, int tid, int nth) {
+                                const double* __restrict__ tab, int* next) {
     const int Q = sd.Q, W = Z + 6, nf = it.nz + 1, rows = 2 * Q;
     const int nruns = (nf + kRun - 1) / kRun;
     TableLayout L(Q);
     const double* xi = tab + sd.tab_off + L.xi;
-    const dfl eps4 = dfl_const(4.0 * sd.weno_eps);
-    for (int e = tid; e < rows * nruns; e += nth) {
+    const dfl eps4 = dfn_const(4.0 * sd.weno_eps);
+    warp_pool(next, rows * nruns, [&](int e) {
         const int r = e % rows, run = e / rows;
         const int k = r % Q;
         const int fa = run * kRun, n = min(kRun, nf - fa), fl = fa + n - 1;
@@ -1099,7 +1461,7 @@ __device__ inline void faces_df(const SlabDesc& sd, const WorkItem& it, const Sm
             out[f0 + dir * q] = w.face();
             if (q + 1 < n) w.shift(hb[dir * (q + 5)]);
         }
-    }
+    });
 }
 
 // Raw moment sums of one node from a column h[k * stride] (k < Q).  The

@@ -19,12 +19,13 @@ namespace evfdlb {
 constexpr int kQMax = 32;          // largest Gauss-Hermite order of a slab
 constexpr int kZMax = 64;          // largest node tile of one CTA
 constexpr int kThreads = 256;      // threads of the per-tile kernels
-// Threads of the RK-stage kernel (warp 0 forms the node work).  The FP64 pipe
-// of this part accepts one warp instruction per scheduler every 64 cycles
-// whatever the number of active lanes, so the FP64 kernels run 8 warps (two
-// worker warps beside the node warp per scheduler, and two CTAs of at most
-// 128 registers per SM when the work list spans several waves); the FP32
-// variant's per-velocity work is cheap and latency-bound, so it runs 16.
+// Threads of the RK-stage kernel.  The FP64 pipe of this part accepts one warp
+// instruction per scheduler every 64 cycles whatever the number of active
+// lanes, so the FP64 kernels run 8 warps (two per scheduler, of which four form
+// the node quantities first; two CTAs of at most 128 registers per SM when the
+// work list spans several waves); the FP32 variant's per-velocity work is
+// cheap and latency-bound, so it runs 16 (and FP64_DF where a CTA has its SM
+// to itself, see launch_stage_df).
 template <typename R, bool DF = false> struct StageThreads { static constexpr int value = 256; };
 template <> struct StageThreads<float, false> { static constexpr int value = 512; };
 constexpr int kNumMoments = 6;     // raw moment sums kept per node

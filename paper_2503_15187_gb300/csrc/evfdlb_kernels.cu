@@ -95,44 +95,71 @@ __device__ __forceinline__ void stage_body(const SlabDesc& sd, const WorkItem& i
     // the state tile by asynchronous copies, issued first, so that they are
     // in flight with the node inputs' loads and arithmetic
     if constexpr (!DF) issue_state_tile<R, CG>(sd, it, s, Z, src, NF);
-    load_node_inputs<R, !DF, CG, false>(sd, it, s, Z, rtab, mom_in, NN);
+    constexpr bool F64 = std::is_same<R, double>::value;
+    __shared__ int s_next[2];                    // pools of face runs and of analysis tasks
+    if constexpr (F64) {
+        if (threadIdx.x < 2) s_next[threadIdx.x] = 0;
+        load_raw_sums<CG>(sd, it, s, Z, mom_in, NN);
+    } else {
+        load_node_inputs<R, !DF, CG, false>(sd, it, s, Z, rtab, mom_in, NN);
+    }
     if constexpr (DF) load_state_tile<R>(sd, it, s, Z, src, NF, Fd);
     if constexpr (!DF && !CG) cp_async_wait_all();
     __syncthreads();
-    // The node warps form the node-level quantities of the tile (node fields,
-    // coefficient constants, Hermite moments of the local Gaussian) while the
-    // other warps do the velocity-space work that needs only the state tile
-    // (Hermite analysis, WENO-5 faces), so the serial node work overlaps it.
     // the tables of everything but the DF transforms
     const R* vtab = DF ? reinterpret_cast<const R*>(tables) : rtab;
     const R* rt = vtab + sd.tab_off;
     TableLayout L(Q);
-    // Node warps: one, or two when pass 1 (nz + 4 nodes) would take a
-    // second round on one warp; the passes are separated by a barrier of the
-    // node warps only (named barrier 1).
-    const int NW = (nz + 4 > 32) ? 2 : 1;
-    auto node_sync = [&]() {
-        if (NW == 1) __syncwarp();
-        else asm volatile("bar.sync 1, 64;" ::: "memory");
-    };
-    // FP32: the Eq. (F1) force sums need only the staged densities, so the
-    // worker warps (whose FP32 work finishes well before the node chain)
-    // form them first, a half-warp per node, and signal on named barrier 3
-    // without waiting; the node warps take them up before pass 2.  The last
-    // worker warp forms the Hermite moments of the local Gaussian meanwhile.
-    // FP64 keeps both in the node chain: there the worker warps are the
-    // longer side of the phase and the FP64 pipe the bound.
-    constexpr bool WF = std::is_same<R, float>::value && !DF;
-    if (threadIdx.x < 32 * NW) {
-        node_fields_pass1<R>(sd, it, s, s.Mtap, NN, fo, threadIdx.x, 32 * NW);
-        node_sync();
-        if constexpr (WF) asm volatile("bar.sync 3, %0;" ::"r"((int)blockDim.x) : "memory");
-        node_fields_pass2<R, WF>(sd, it, s, Z, s.Ftap, mom_in, NN, err, fo, threadIdx.x, 32 * NW);
-        node_sync();
-        node_coefficients<R, !WF>(sd, it, s, Z, rt, threadIdx.x, 32 * NW);
+    if constexpr (F64) {
+        // Warps 0-3 form the node quantities, the others split the state tile
+        // into parity parts; then every warp takes runs of WENO-5 faces, and
+        // groups of the Hermite analysis, as it arrives.
+        if (threadIdx.x < 128) {
+            node_roles<FO>(sd, it, s, Z, rt, NN, err, fo);
+            // the parity parts are there (barrier 8 + warp: this warp and the
+            // arrivals of the splitting warps)
+            if constexpr (!DF)
+                asm volatile("bar.sync %0, %1;" ::"r"(8 + (int)(threadIdx.x >> 5)), "r"((int)blockDim.x - 96) : "memory");
+        } else if constexpr (!DF) {
+            const int nth = blockDim.x - 128;
+            split_state_tile<R>(sd, it, s, Z, threadIdx.x - 128, nth);
+            __threadfence_block();
+#pragma unroll
+            for (int w = 0; w < 4; ++w) asm volatile("bar.arrive %0, %1;" ::"r"(8 + w), "r"(nth + 32) : "memory");
+            asm volatile("bar.sync 2, %0;" ::"r"(nth) : "memory");
+        }
+        if constexpr (DF) {
+            faces_df(sd, it, s, Z, tables, s_next);
+            analysis_df(sd, it, s, Fd, reinterpret_cast<const float2*>(s.P), Z, s_next + 1);
+        } else {
+            faces_split(sd, it, s, Z, vtab, s_next);
+            analysis_eo<R>(sd, it, s, Z, 0, 0, s_next + 1);
+        }
     } else {
-        const int tid = threadIdx.x - 32 * NW, nth = blockDim.x - 32 * NW;
-        if constexpr (WF) {
+        // The node warps form the node-level quantities of the tile (node
+        // fields, coefficient constants) while the other warps do the
+        // velocity-space work that needs only the state tile (Hermite analysis,
+        // WENO-5 faces), so the serial node work overlaps it.  One node warp,
+        // or two when pass 1 (nz + 4 nodes) would take a second round on one;
+        // the passes are separated by a barrier of the node warps only.
+        const int NW = (nz + 4 > 32) ? 2 : 1;
+        auto node_sync = [&]() {
+            if (NW == 1) __syncwarp();
+            else asm volatile("bar.sync 1, 64;" ::: "memory");
+        };
+        // The Eq. (F1) force sums need only the staged densities, so the
+        // worker warps (whose FP32 work finishes well before the node chain)
+        // form them first, a half-warp per node, and signal on named barrier
+        // 3 without waiting; the node warps take them up before pass 2.
+        if (threadIdx.x < 32 * NW) {
+            node_fields_pass1<R>(sd, it, s, s.Mtap, NN, fo, threadIdx.x, 32 * NW);
+            node_sync();
+            asm volatile("bar.sync 3, %0;" ::"r"((int)blockDim.x) : "memory");
+            node_fields_pass2<R, true>(sd, it, s, Z, s.Ftap, mom_in, NN, err, fo, threadIdx.x, 32 * NW);
+            node_sync();
+            node_coefficients(sd, it, s, Z, threadIdx.x, 32 * NW);
+        } else {
+            const int tid = threadIdx.x - 32 * NW, nth = blockDim.x - 32 * NW;
             // the Hermite moments of the local Gaussian (a serial recurrence
             // per node) need only u and T of the node inputs: the last worker
             // warp, whose share of the force sums (a half-warp per node from
@@ -142,18 +169,13 @@ __device__ __forceinline__ void stage_body(const SlabDesc& sd, const WorkItem& i
             tile_force_sums<R>(sd, it, s, Z, s.Ftap, tid, nth);
             __threadfence_block();
             asm volatile("bar.arrive 3, %0;" ::"r"((int)blockDim.x) : "memory");
-        }
-        if constexpr (DF) {
-            analysis_df(sd, it, s, Fd, reinterpret_cast<const float2*>(s.P), Z, tid, nth);
-        } else {
             // the worker warps split the tile into parity parts, then join on
             // named barrier 2 (the node warps go on meanwhile)
             split_state_tile<R>(sd, it, s, Z, tid, nth);
             asm volatile("bar.sync 2, %0;" ::"r"(nth) : "memory");
             analysis_eo<R>(sd, it, s, Z, tid, nth);
+            faces<R>(sd, it, s, Z, vtab, tid, nth);
         }
-        if constexpr (DF) faces_df(sd, it, s, Z, tables, tid, nth);
-        else faces<R>(sd, it, s, Z, vtab, tid, nth);
     }
     __syncthreads();
     coefficients<R, DF>(sd, it, s, Z, rt, threadIdx.x, blockDim.x);
@@ -356,7 +378,7 @@ __device__ __forceinline__ void stage_body(const SlabDesc& sd, const WorkItem& i
 }
 
 template <typename R, bool DF = false, int T = StageThreads<R, DF>::value>
-__global__ void __launch_bounds__(T, DF ? 3 : ((std::is_same<R, double>::value || T <= 256) ? 2 : 1))
+__global__ void __launch_bounds__(T, T > 256 ? 1 : (DF ? 3 : 2))
 stage_kernel(const SlabDesc* __restrict__ slabs, const WorkItem* __restrict__ items,
              const double* __restrict__ tables, const R* __restrict__ rtab,
              const double* __restrict__ taps, const R* __restrict__ rtaps,
@@ -755,8 +777,25 @@ size_t stage_smem_bytes_p(int prec, int Q, int Z, int M) {
 size_t stage_smem_bytes_df(int Q, int Z, int M) { return smem_bytes_t<double>(Q, Z, M); }
 
 cudaError_t configure_df(size_t smem_bytes) {
-    return cudaFuncSetAttribute(stage_kernel<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(stage_kernel<double, true, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem_bytes);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(stage_kernel<double, true, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem_bytes);
+}
+
+// SMs of the current device (cached per device).
+static int sm_count() {
+    static int cache[64] = {0};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) return 1;
+    if (!cache[dev]) {
+        int n = 0;
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        cache[dev] = n > 0 ? n : 1;
+    }
+    return cache[dev];
 }
 
 // FP64_DF stage: dftab holds the analysis and synthesis tables as pairs.
@@ -764,8 +803,13 @@ void launch_stage_df(int nitems, size_t smem, cudaStream_t st, const SlabDesc* s
                      const double* tables, const double* dftab, const double* taps, const double* src,
                      const double* base, double* out, double* rhs_out, const double* mom_in, double* mom_out,
                      long long NF, long long NN, double alpha, double beta, int mode, int Z, unsigned* err) {
-    launch_pdl(stage_kernel<double, true>, nitems, StageThreads<double, true>::value, smem, st, slabs, items, tables,
-               dftab, taps, taps, src, base, out, rhs_out, mom_in, mom_out, NF, NN, alpha, beta, mode, Z, err);
+    // 16 warps (one CTA per SM) where the work list fits one wave on the SMs,
+    // else 8 (up to three CTAs): the double-float runs of one CTA's 8 warps
+    // leave their pipe idle on latency (4096 x 32, 152 tiles: 40.9 -> 34.7 us a
+    // stage; 3001 x 24: 34.1 -> 22.8 us; two tiles per SM: 44.9 -> 47.7)
+    auto kernel = nitems <= sm_count() ? stage_kernel<double, true, 512> : stage_kernel<double, true, 256>;
+    launch_pdl(kernel, nitems, nitems <= sm_count() ? 512 : 256, smem, st, slabs, items, tables, dftab, taps, taps, src,
+               base, out, rhs_out, mom_in, mom_out, NF, NN, alpha, beta, mode, Z, err);
 }
 
 template <typename R>
@@ -807,20 +851,6 @@ cudaError_t ensure_stage_smem(size_t smem_bytes) {
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
-}
-
-// SMs of the current device (cached per device).
-static int sm_count() {
-    static int cache[64] = {0};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64) return 1;
-    if (!cache[dev]) {
-        int n = 0;
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        cache[dev] = n > 0 ? n : 1;
-    }
-    return cache[dev];
 }
 
 // The FP64 stage (8 warps; see StageThreads).
