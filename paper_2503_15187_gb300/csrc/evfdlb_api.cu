@@ -577,7 +577,7 @@ evfdlb_status evfdlb_create(const evfdlb_params* p, int32_t nbatch, const evfdlb
         d.node_off = NN;
         d.dx = q.dx;
         d.inv_dx = 1.0 / q.dx;
-        d.dt = resolved_dt(q);
+        d.dt = q.dt > 0 ? q.dt : q.cfl * q.dx / fabs(tables[d.tab_off + TableLayout(q.Q).xi + q.Q - 1]);
         d.weno_eps = q.weno_eps;
         d.b = 2.0 * M_PI * q.sigma * q.sigma * q.sigma / 3.0;
         d.eta_coef = M_PI * q.sigma * q.sigma * q.sigma / 6.0;

@@ -148,6 +148,5 @@ double ev2_kappa(const evfdlb_params& p);                        // Eq. (F2) kap
 double discrete_a(const evfdlb_params& p);
 double critical_T_of_a(double a, double sigma, double* n_c);
 bool coexistence_of(double a, double sigma, double T, double* nv, double* nl);
-double resolved_dt(const evfdlb_params& p);
 
 }  // namespace evfdlb

@@ -18,25 +18,30 @@ const long double kPiL = 3.141592653589793238462643383279502884L;
 const double kPi = 3.14159265358979323846;
 
 // Orthonormal probabilists' Hermite functions psi_l = He_l / sqrt(l!) at x,
-// l = 0..L, by psi_{l+1} = (x psi_l - sqrt(l) psi_{l-1}) / sqrt(l+1).
+// l = 0..L, by psi_{l+1} = (x psi_l - sqrt(l) psi_{l-1}) / sqrt(l+1);
+// r[l] = sqrt(l), l <= L.
 template <typename R>
-void psi_all(int L, R x, R* psi) {
+void psi_all(int L, R x, const R* r, R* psi) {
     psi[0] = 1;
     if (L >= 1) psi[1] = x;
-    for (int l = 1; l < L; ++l)
-        psi[l + 1] = (x * psi[l] - sqrtl((long double)l) * psi[l - 1]) / sqrtl((long double)(l + 1));
+    for (int l = 1; l < L; ++l) psi[l + 1] = (x * psi[l] - r[l] * psi[l - 1]) / r[l + 1];
+}
+
+template <typename R>
+void roots_of(int L, R* r) {
+    for (int l = 0; l <= L; ++l) r[l] = (R)sqrtl((long double)l);
 }
 
 // Number of eigenvalues below x of the Jacobi matrix of the probabilists'
 // Hermite recurrence (zero diagonal, off-diagonal sqrt(k)), by the Sturm
 // count of the LDL^T pivots.
-int sturm_count(int Q, long double x) {
+int sturm_count(int Q, double x) {
     int count = 0;
-    long double d = -x;
+    double d = -x;
     if (d < 0) ++count;
     for (int k = 1; k < Q; ++k) {
-        long double piv = (d == 0) ? 1e-300L : d;
-        d = -x - (long double)k / piv;
+        double piv = (d == 0) ? 1e-300 : d;
+        d = -x - (double)k / piv;
         if (d < 0) ++count;
     }
     return count;
@@ -46,37 +51,44 @@ int sturm_count(int Q, long double x) {
 // Roots of He_Q (the velocity nodes of the full-range Gauss-Hermite rule) by
 // bisection on the Sturm count, polished by Newton on psi_Q with
 // psi_Q' = sqrt(Q) psi_{Q-1}; weights w = 1 / (Q psi_{Q-1}(x)^2), which sum to 1.
+// Bisection and the first Newton steps run in FP64, the last ones in extended
+// precision, which is software on Arm hosts (2.7 ms for Q = 24 when all of it
+// was extended, now a tenth).  He_Q has the parity of Q: the positive half is
+// computed and mirrored, so the stored set is exactly symmetric
+// (xi_{Q-1-k} = -xi_k, w_{Q-1-k} = w_k, a zero node for odd Q), which the
+// parity-split transforms rely on.
 // Fixed-size storage (no heap), so that the allocation-free step can call it.
 bool velocity_set(int Q, double* xi, double* w) {
     if (Q < 1 || Q > kVelocitySetMax) return false;
-    long double psi[kVelocitySetMax + 1];
-    long double bound = sqrtl(4.0L * Q + 2.0L) + 1.0L;
-    for (int k = 0; k < Q; ++k) {
-        long double lo = -bound, hi = bound;   // k-th smallest: count(x) >= k+1
-        for (int it = 0; it < 200 && hi - lo > 1e-18L * (1 + fabsl(lo)); ++it) {
-            long double mid = 0.5L * (lo + hi);
+    long double psi[kVelocitySetMax + 1], r[kVelocitySetMax + 1];
+    double psd[kVelocitySetMax + 1], rd[kVelocitySetMax + 1];
+    roots_of<long double>(Q, r);
+    roots_of<double>(Q, rd);
+    const double bound = sqrt(4.0 * Q + 2.0) + 1.0;
+    for (int k = Q / 2; k < Q; ++k) {
+        double lo = -0.5, hi = bound;              // k-th smallest: count(x) >= k+1
+        for (int it = 0; it < 200 && hi - lo > 1e-9 * (1 + fabs(lo)); ++it) {
+            double mid = 0.5 * (lo + hi);
             if (sturm_count(Q, mid) >= k + 1) hi = mid; else lo = mid;
         }
-        long double x = 0.5L * (lo + hi);
-        for (int it = 0; it < 3; ++it) {
-            psi_all<long double>(Q, x, psi);
-            long double dpsi = sqrtl((long double)Q) * psi[Q - 1];
+        double xd = 0.5 * (lo + hi);
+        for (int it = 0; it < 2; ++it) {
+            psi_all<double>(Q, xd, rd, psd);
+            if (psd[Q - 1] == 0) break;
+            xd -= psd[Q] / (rd[Q] * psd[Q - 1]);
+        }
+        long double x = xd;
+        for (int it = 0; it < 2; ++it) {
+            psi_all<long double>(Q, x, r, psi);
+            long double dpsi = r[Q] * psi[Q - 1];
             if (dpsi == 0) break;
             x -= psi[Q] / dpsi;
         }
-        psi_all<long double>(Q, x, psi);
+        psi_all<long double>(Q, x, r, psi);
         xi[k] = (double)x;
         w[k] = (double)(1.0L / ((long double)Q * psi[Q - 1] * psi[Q - 1]));
-    }
-    // He_Q has the parity of Q: its roots are symmetric about 0.  Make the
-    // stored set exactly so (xi_{Q-1-k} = -xi_k, w_{Q-1-k} = w_k, a zero node
-    // for odd Q), which the parity-split transforms rely on.
-    for (int k = 0; k < Q / 2; ++k) {
-        const long double a = 0.5L * ((long double)xi[Q - 1 - k] - (long double)xi[k]);
-        const long double b = 0.5L * ((long double)w[Q - 1 - k] + (long double)w[k]);
-        xi[k] = (double)(-a);
-        xi[Q - 1 - k] = (double)a;
-        w[k] = w[Q - 1 - k] = (double)b;
+        xi[Q - 1 - k] = -xi[k];
+        w[Q - 1 - k] = w[k];
     }
     if (Q & 1) xi[Q / 2] = 0.0;
     return true;
@@ -85,11 +97,12 @@ bool velocity_set(int Q, double* xi, double* w) {
 // Fixed-size storage (no heap), like velocity_set.
 void build_tables(int Q, const double* xi, const double* w, double* out) {
     TableLayout L(Q);
-    long double psi[kVelocitySetMax + 1];
+    long double psi[kVelocitySetMax + 1], r[kVelocitySetMax + 1];
+    roots_of<long double>(Q, r);
     for (int k = 0; k < Q; ++k) {
         out[L.xi + k] = xi[k];
         out[L.w + k] = w[k];
-        psi_all<long double>(Q, (long double)xi[k], psi);
+        psi_all<long double>(Q, (long double)xi[k], r, psi);
         for (int l = 0; l < Q; ++l) {
             out[L.P + l * Q + k] = (double)psi[l];
             out[L.S + k * Q + l] = (double)((long double)w[k] * psi[l]);
@@ -269,13 +282,6 @@ double discrete_a(const evfdlb_params& p) {
     for (int j = -M; j <= M; ++j)
         acc += (long double)simpson(j, M, p.dx) * (j * p.dx) * g_kernel(j * p.dx, p.sigma, p.phi_a, p.gamma);
     return (double)(0.5L * acc);
-}
-
-double resolved_dt(const evfdlb_params& p) {
-    if (p.dt > 0) return p.dt;
-    double xi[kQMax], w[kQMax];
-    velocity_set(p.Q, xi, w);
-    return p.cfl * p.dx / fabs(xi[p.Q - 1]);
 }
 
 // ---------------------------------------------------------------------------
