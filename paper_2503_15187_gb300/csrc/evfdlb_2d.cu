@@ -390,24 +390,25 @@ __device__ __forceinline__ void prim2(const double* __restrict__ mom, long long 
 // staged density pair feeds 16 FMAs (8 rows x 2 components).  The per-warp
 // partial forces are summed in warp order (deterministic).
 // ---------------------------------------------------------------------------
-constexpr int kFWarps = 8;           // warps of k2_fields (256 threads)
 constexpr int kFRows = 8;            // rows of a force register block (= ring length)
-constexpr int kFPlanHead = 12;       // plan header: kFWarps + 1 prefix offsets, padded to 16 bytes
-static_assert(kTile2 == 16 && 2 * kFRows == kTile2 && kFWarps * 32 == 256, "force mapping: 16 x 2 lanes x 8 rows");
+constexpr int kFMaxWarps = 24;       // most warps of a CTA
+constexpr int kFPlanHead = 28;       // plan header: a prefix offset per warp and the end, padded to 16 bytes
+static_assert(kTile2 == 16 && 2 * kFRows == kTile2 && kFPlanHead > kFMaxWarps && kFPlanHead % 4 == 0,
+              "force mapping: 16 x 2 lanes x 8 rows");
 
 // pitch of the staged density row: >= W and = 2 (mod 4), so that rows 8
 // apart (the two row blocks of a warp) fall 16 banks apart
 __host__ __device__ inline int fields_pitch(int W) { return W + ((6 - W % 4) % 4); }
 
 template <typename R>
-__host__ __device__ inline size_t fields_smem_bytes(int Mf, int mfm) {
+__host__ __device__ inline size_t fields_smem_bytes(int Mf, int mfm, int nfm, int warps) {
     const int H = Mf > mfm + 2 ? Mf : mfm + 2, W = kTile2 + 2 * H, E = kTile2 + 4, Wr = fields_pitch(W);
-    const size_t nr = (size_t)(W + kFRows) * Wr, pf = 2 * (size_t)kFWarps * kTile2 * kTile2;
-    return sizeof(R) * ((nr > pf ? nr : pf) + 5 * (size_t)E * E);
+    const size_t nr = (size_t)(W + kFRows) * Wr, pf = 2 * (size_t)warps * kTile2 * kTile2;
+    return sizeof(R) * ((nr > pf ? nr : pf) + 5 * (size_t)E * E + nfm) + sizeof(int) * (size_t)nfm;
 }
 
-template <typename R>
-__global__ void __launch_bounds__(256)
+template <typename R, int NW>
+__global__ void __launch_bounds__(32 * NW)
 k2_fields(Slab2 s, const Par2<R> pr, const double* __restrict__ mom, const float* __restrict__ prf, const R* __restrict__ ftw,
           const int* __restrict__ fplan, const int* __restrict__ fm_off, const R* __restrict__ fm_w,
           R* __restrict__ fld, unsigned* err) {
@@ -417,7 +418,7 @@ k2_fields(Slab2 s, const Par2<R> pr, const double* __restrict__ mom, const float
     R* sm2 = reinterpret_cast<R*>(sm2raw);
     const int H = max(s.Mf, s.mfm + 2), W = kTile2 + 2 * H, E = kTile2 + 4, Wr = fields_pitch(W);
     R* Nr = sm2;                      // n on the tile + H halo, [W + 8][Wr]; rows W.. are zero
-    R* U = sm2 + max((W + kFRows) * Wr, 2 * kFWarps * kTile2 * kTile2);
+    R* U = sm2 + max((W + kFRows) * Wr, 2 * NW * kTile2 * kTile2);
     R* V = U + E * E;                 // ux, uy, T, X, chi on the tile + 2, [E][E] each
     R* Tt = V + E * E;
     R* Xt = Tt + E * E;
@@ -425,19 +426,34 @@ k2_fields(Slab2 s, const Par2<R> pr, const double* __restrict__ mom, const float
     const int nx = s.nx, ny = s.ny;
     const long long N = s.N;
     const int x0 = blockIdx.x * kTile2, y0 = blockIdx.y * kTile2;
-    for (int e = threadIdx.x; e < (W + kFRows) * W; e += blockDim.x) {
-        const int cy = e / W, cx = e % W;
-        R n = R(0);
-        if (cy < W) {
-            const long long i = (long long)wrapi(y0 - H + cy, ny) * nx + wrapi(x0 - H + cx, nx);
-            if constexpr (F32) n = prf[P2_N * N + i];
-            else n = mom[M2_S0 * N + i];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // a warp per row; one wrap is enough wherever the halo is narrower than the grid
+    auto wrap1 = [](int i, int n) {
+        i = i < 0 ? i + n : (i >= n ? i - n : i);
+        return (unsigned)i < (unsigned)n ? i : wrapi(i, n);
+    };
+    for (int cy = warp; cy < W + kFRows; cy += NW) {
+        const long long row = (long long)wrap1(y0 - H + cy, ny) * nx;
+        for (int cx = lane; cx < W; cx += 32) {
+            R n = R(0);
+            if (cy < W) {
+                const long long i = row + wrap1(x0 - H + cx, nx);
+                if constexpr (F32) n = prf[P2_N * N + i];
+                else n = mom[M2_S0 * N + i];
+            }
+            Nr[cy * Wr + cx] = n;
         }
-        Nr[cy * Wr + cx] = n;
+    }
+    // Fischer-Methfessel taps as offsets in the staged density
+    R* fw = Ct + E * E;
+    int* fo = reinterpret_cast<int*>(fw + s.nfm);
+    for (int t = threadIdx.x; t < s.nfm; t += 32 * NW) {
+        fw[t] = fm_w[t];
+        fo[t] = fm_off[2 * t + 1] * Wr + fm_off[2 * t];
     }
     for (int e = threadIdx.x; e < E * E; e += blockDim.x) {
         const int cy = e / E, cx = e % E;
-        const long long i = (long long)wrapi(y0 - 2 + cy, ny) * nx + wrapi(x0 - 2 + cx, nx);
+        const long long i = (long long)wrap1(y0 - 2 + cy, ny) * nx + wrap1(x0 - 2 + cx, nx);
         if constexpr (F32) {
             U[e] = prf[P2_UX * N + i];
             V[e] = prf[P2_UY * N + i];
@@ -456,7 +472,9 @@ k2_fields(Slab2 s, const Par2<R> pr, const double* __restrict__ mom, const float
         const int cy = e / E, cx = e % E;
         const int hy = cy - 2 + H, hx = cx - 2 + H;   // position in the halo array
         R nb = R(0);
-        for (int t = 0; t < s.nfm; ++t) nb = fma(fm_w[t], Nr[(hy + fm_off[2 * t + 1]) * Wr + hx + fm_off[2 * t]], nb);
+        const R* c = Nr + hy * Wr + hx;
+#pragma unroll 4
+        for (int t = 0; t < s.nfm; ++t) nb = fma(fw[t], c[fo[t]], nb);
         const R eta = pr.eta_coef * nb, om = R(1) - eta;
         const R chi = (R(2) - eta) / (R(2) * om * om * om);
         const R n = Nr[hy * Wr + hx];
@@ -464,7 +482,6 @@ k2_fields(Slab2 s, const Par2<R> pr, const double* __restrict__ mom, const float
         Xt[e] = n * n * chi * Tt[e];
     }
     // force over the disc
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int fxl = lane & 15, yb = lane >> 4;
     R ax[kFRows], ay[kFRows];
 #pragma unroll
@@ -500,25 +517,26 @@ k2_fields(Slab2 s, const Par2<R> pr, const double* __restrict__ mom, const float
             }
         }
     }
-    const int tx = threadIdx.x % kTile2, ty = threadIdx.x / kTile2;
+    constexpr int NN = kTile2 * kTile2;
+    const int node = threadIdx.x % NN, tx = node % kTile2, ty = node / kTile2;
     const R n = Nr[(ty + H) * Wr + tx + H];
     __syncthreads();                  // density reads done: its space takes the partial forces
-    R* Pf = sm2;                      // [kFWarps][2][256]
+    R* Pf = sm2;                      // [NW][2][NN]
 #pragma unroll
     for (int k = 0; k < kFRows; ++k) {
-        const int node = (yb * kFRows + k) * kTile2 + fxl;
-        Pf[(2 * warp) * 256 + node] = ax[k];
-        Pf[(2 * warp + 1) * 256 + node] = ay[k];
+        const int o = (yb * kFRows + k) * kTile2 + fxl;
+        Pf[(2 * warp) * NN + o] = ax[k];
+        Pf[(2 * warp + 1) * NN + o] = ay[k];
     }
     __syncthreads();
     R fx = R(0), fy = R(0);
 #pragma unroll
-    for (int w = 0; w < kFWarps; ++w) {
-        fx += Pf[(2 * w) * 256 + threadIdx.x];
-        fy += Pf[(2 * w + 1) * 256 + threadIdx.x];
+    for (int w = 0; w < NW; ++w) {
+        fx += Pf[(2 * w) * NN + node];
+        fy += Pf[(2 * w + 1) * NN + node];
     }
     const int x = x0 + tx, y = y0 + ty;
-    if (x >= nx || y >= ny) return;
+    if (threadIdx.x >= NN || x >= nx || y >= ny) return;
     const long long i = (long long)y * nx + x;
     const int c = (ty + 2) * E + (tx + 2);
     const R k12 = pr.k12;
@@ -1515,16 +1533,16 @@ Taps2 taps_2d(const evfdlb_params& p) {
 // Force plan of k2_fields: the disc's offset columns a = 0 .. Mf, each as a
 // run of `steps` weight pairs (a multiple of 8: offsets b = -w .. w, then
 // zeros), column 0 with halved g2y (its pass adds n(x) twice); the columns
-// are dealt to the kFWarps warps longest first, each to the least loaded
-// warp (deterministic).  Layout of `plan`: kFWarps + 1 prefix offsets
-// (padded to kFPlanHead ints), then per entry {a, weight offset, steps, w}.
+// are dealt to the warps longest first, each to the least loaded warp
+// (deterministic).  Layout of `plan`: warps + 1 prefix offsets (padded to
+// kFPlanHead ints), then per entry {a, weight offset, steps, w}.
 struct ForcePlan {
     std::vector<int> plan;
     std::vector<double> w;     // (g2x, g2y) pairs
     bool ok = true;
 };
 
-ForcePlan force_plan(const Taps2& t) {
+ForcePlan force_plan(const Taps2& t, int warps) {
     ForcePlan fp;
     const int Mf = t.Mf, D = 2 * Mf + 1;
     std::vector<double> gx((size_t)D * D, 0.0), gy((size_t)D * D, 0.0);
@@ -1562,23 +1580,23 @@ ForcePlan force_plan(const Taps2& t) {
     std::vector<int> order(cols.size());
     for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
     std::stable_sort(order.begin(), order.end(), [&](int p, int q) { return cols[p].steps > cols[q].steps; });
-    std::vector<std::vector<int>> bins(kFWarps);
-    std::vector<long long> load(kFWarps, 0);
+    std::vector<std::vector<int>> bins(warps);
+    std::vector<long long> load(warps, 0);
     for (int ci : order) {
         int best = 0;
-        for (int k = 1; k < kFWarps; ++k)
+        for (int k = 1; k < warps; ++k)
             if (load[k] < load[best]) best = k;
         bins[best].push_back(ci);
         load[best] += cols[ci].steps;
     }
     fp.plan.assign(kFPlanHead, 0);
     int n = 0;
-    for (int k = 0; k < kFWarps; ++k) {
+    for (int k = 0; k < warps; ++k) {
         fp.plan[k] = n;
         n += (int)bins[k].size();
     }
-    fp.plan[kFWarps] = n;
-    for (int k = 0; k < kFWarps; ++k)
+    fp.plan[warps] = n;
+    for (int k = 0; k < warps; ++k)
         for (int ci : bins[k]) {
             const Col& c = cols[ci];
             fp.plan.insert(fp.plan.end(), {c.a, c.off, c.steps, c.w});
@@ -1687,6 +1705,7 @@ struct Ctx2 {
     cudaGraphExec_t g_one = nullptr;
     size_t smem_fields = 0, smem_coll = 0;
     int coll_ctas = 1;           // resident CTAs of k2_coll_pipe
+    int field_warps = 8;         // warps per CTA of k2_fields
     // the model constants in precision R (the stage weights are the caller's)
     template <typename R>
     Par2<R> par() const {
@@ -1715,6 +1734,19 @@ auto with_q(int Q, F f) {
         case 14: return f(std::integral_constant<int, 14>{});
         default: return f(std::integral_constant<int, 16>{});
     }
+}
+
+// Warps per CTA of k2_fields: one CTA of 24 per SM where every tile has an SM to
+// itself (the force disc's columns then run side by side: 96x64 26.5 -> 17.4
+// us), 16 up to one and a half tiles per SM (200x200: 27.5 -> 24.2 us), else 8,
+// whose CTAs overlap each other's loads (384x384: 43.7 us against 46.9 and 57.1).
+int field_warps(const Ctx2* c) {
+    const long long tiles = (long long)((c->s.nx + kTile2 - 1) / kTile2) * ((c->s.ny + kTile2 - 1) / kTile2);
+    return tiles <= c->sms ? kFMaxWarps : (2 * tiles <= 3LL * c->sms ? 16 : 8);
+}
+template <typename R>
+auto fields_kernel_of(const Ctx2* c) {
+    return c->field_warps == 8 ? k2_fields<R, 8> : (c->field_warps == 16 ? k2_fields<R, 16> : k2_fields<R, kFMaxWarps>);
 }
 
 // Velocities per CTA of k2_adv: up to 16 (the copy offsets are formed once per
@@ -1804,8 +1836,8 @@ void queue_stage_t(Ctx2* c, cudaStream_t st, const void* src, const void* base, 
     if constexpr (F32) launch_moments<float>(Q, nbm, st, s, c->pwf, (const float2*)src, nullptr, c->prf, c->err);
     else launch_moments<double>(Q, nbm, st, s, c->pwd, (const double2*)src, c->mom, nullptr, c->err);
     dim3 gf((s.nx + kTile2 - 1) / kTile2, (s.ny + kTile2 - 1) / kTile2);
-    k2_fields<R><<<gf, 256, c->smem_fields, st>>>(s, pr, c->mom, c->prf, (const R*)c->ftw, c->fplan, c->fm_off,
-                                                   (const R*)c->fm_w, (R*)c->fld, c->err);
+    fields_kernel_of<R>(c)<<<gf, 32 * c->field_warps, c->smem_fields, st>>>(
+        s, pr, c->mom, c->prf, (const R*)c->ftw, c->fplan, c->fm_off, (const R*)c->fm_w, (R*)c->fld, c->err);
     launch_coll<R>(c, st, pr, (const R*)src, (const R*)base, V);
     launch_adv<R>(c, st, pr, (const R*)src, V);
 }
@@ -1887,7 +1919,8 @@ evfdlb_status create_2d(const evfdlb_params& p, void* stream, Ctx2** out) {
     alloc(&c->fld, c->esize * kNumFld2 * s.N);
     alloc((void**)&c->mom, sizeof(double) * kNumMom2 * s.N);
     alloc((void**)&c->tables, sizeof(double) * tab.size());
-    const ForcePlan fp = force_plan(t);
+    c->field_warps = field_warps(c);
+    const ForcePlan fp = force_plan(t, c->field_warps);
     if (!fp.ok) e = cudaErrorInvalidValue;      // the tap set lost its mirror symmetry
     const bool f32 = (c->prec == EVFDLB_FP32);
     alloc((void**)&c->fplan, sizeof(int) * fp.plan.size());
@@ -1921,11 +1954,14 @@ evfdlb_status create_2d(const evfdlb_params& p, void* stream, Ctx2** out) {
         e = f32 ? cudaMemcpy(c->fm_w, mwf.data(), sizeof(float) * mwf.size(), cudaMemcpyHostToDevice)
                 : cudaMemcpy(c->fm_w, t.mw.data(), sizeof(double) * t.mw.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(c->err, 0, sizeof(unsigned));
-    c->smem_fields = f32 ? fields_smem_bytes<float>(s.Mf, s.mfm) : fields_smem_bytes<double>(s.Mf, s.mfm);
+    c->smem_fields = f32 ? fields_smem_bytes<float>(s.Mf, s.mfm, s.nfm, c->field_warps)
+                         : fields_smem_bytes<double>(s.Mf, s.mfm, s.nfm, c->field_warps);
     if (c->smem_fields > 227 * 1024) e = cudaErrorInvalidValue;   // force disc too wide for a tile
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(f32 ? (const void*)k2_fields<float> : (const void*)k2_fields<double>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->smem_fields);
+        e = f32 ? cudaFuncSetAttribute(fields_kernel_of<float>(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)c->smem_fields)
+                : cudaFuncSetAttribute(fields_kernel_of<double>(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)c->smem_fields);
     if (e == cudaSuccess) e = configure_2d(c);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) {
