@@ -75,10 +75,11 @@ enum {
 };
 /* Precision.  FP64: every step in FP64.  FP32: FP32 state and per-velocity
  * work, FP64 chi / transport / gradients / conserved sums.  FP64_DF: FP64
- * state and FP64 arithmetic except the Hermite analysis and synthesis of the
- * stage, which run as double-float pairs (hi, lo floats, ~48 bits) on the
- * FP32 pipe with the compensated dot product Dot2 of Ogita, Rump & Oishi
- * (2005); the adjoint returns E_UNSUPPORTED for it. */
+ * state and FP64 arithmetic except the WENO-5 faces, which run as double-float
+ * pairs (hi, lo floats, ~47 bits) on the FP32 pipe, and the Hermite analysis
+ * and synthesis of the stage, which run as products of digit slices on the
+ * tensor cores (~56 bits; FP64 slabs with Q > 16 as well); the adjoint returns
+ * E_UNSUPPORTED for it. */
 enum { EVFDLB_FP64 = 0, EVFDLB_FP32 = 1, EVFDLB_FP64_DF = 2 };
 /* Force model (Sec. II.A).  EV1: the convolution of Eq. (F1), Simpson taps
  * over |z| <= r_cut.  EV2: its gradient expansion, Eq. (F2),

@@ -15,6 +15,7 @@
 
 namespace evfdlb {
 size_t stage_smem_bytes_p(int prec, int Q, int Z, int M);
+size_t stage_smem_cap_p(int prec, int Q, int M);
 cudaError_t configure_kernels_p(int prec, size_t smem_bytes);
 void launch_stage_p(int prec, int nitems, size_t smem, cudaStream_t st, const SlabDesc* slabs,
                     const WorkItem* items, const double* tables, const void* rtab, const double* taps,
@@ -32,12 +33,11 @@ void launch_init_p(int prec, int nitems, size_t smem, cudaStream_t st, const Sla
 void launch_sums_p(int prec, int nitems, cudaStream_t st, const SlabDesc* slabs, const WorkItem* items,
                    const double* tables, const void* rtab, const void* state, double* mom, long long NF,
                    long long NN, unsigned* err);
-size_t stage_smem_bytes_df(int Q, int Z, int M);
 cudaError_t configure_df(size_t smem_bytes);
 void launch_stage_df(int nitems, size_t smem, cudaStream_t st, const SlabDesc* slabs, const WorkItem* items,
-                     const double* tables, const double* dftab, const double* taps, const double* src,
-                     const double* base, double* out, double* rhs_out, const double* mom_in, double* mom_out,
-                     long long NF, long long NN, double alpha, double beta, int mode, int Z, unsigned* err);
+                     const double* tables, const double* taps, const double* src, const double* base, double* out,
+                     double* rhs_out, const double* mom_in, double* mom_out, long long NF, long long NN, double alpha,
+                     double beta, int mode, int Z, unsigned* err);
 void launch_iso_reset_p(int prec, int nitems, size_t smem, cudaStream_t st, const SlabDesc* slabs,
                         const WorkItem* items, const double* tables, const void* rtab, void* state, double* mom,
                         long long NF, long long NN, int Z);
@@ -137,8 +137,6 @@ struct evfdlb_ctx {
     int halo_G = 0;
     int halo_lo = 0, halo_hi = 0;   // ghost nodes below / above the interior (0: an outflow end)
     int rk_next = 0;
-    double* dftables = nullptr;  // analysis / synthesis tables as float pairs (FP64_DF)
-    size_t smem_df = 0;          // stage shared memory of the FP64_DF kernel
     // adjoint: checkpoints of the trajectory since the last init / set_state
     int ckpt_every = 0;          // 0: no tracking (no adjoint)
     int64_t steps = 0;           // steps since the trajectory origin
@@ -189,7 +187,6 @@ void free_ctx(evfdlb_ctx* c) {
         cudaFree(c->mom[i]);
     }
     if (c->rtables != c->tables) cudaFree(c->rtables);
-    cudaFree(c->dftables);
     if (c->rtaps != c->taps) cudaFree(c->rtaps);
     cudaFree(c->tables);
     cudaFree(c->taps);
@@ -221,7 +218,7 @@ void queue_stage(evfdlb_ctx* c, cudaStream_t st, const void* src, const void* ba
                  double* mo, double a, double b) {
     const int n = (int)c->items_h.size();
     if (c->df)
-        launch_stage_df(n, c->smem_df, st, c->slabs, c->items, c->tables, c->dftables, c->taps, (const double*)src,
+        launch_stage_df(n, c->smem, st, c->slabs, c->items, c->tables, c->taps, (const double*)src,
                         (const double*)base, (double*)out, nullptr, mi, mo, c->NF, c->NN, a, b, 0, c->Z, c->err);
     else
         launch_stage_p(c->prec, n, c->smem, st, c->slabs, c->items, c->tables, c->rtables, c->taps, c->rtaps, src,
@@ -281,8 +278,7 @@ void partition(evfdlb_ctx* c, int Z) {
         const int lo = c->halo_lo, hi = c->params[s].nx - c->halo_hi;
         for (int i0 = lo; i0 < hi; i0 += Z) c->items_h.push_back(WorkItem{s, i0, std::min(Z, hi - i0), 0});
     }
-    c->smem = stage_smem_bytes_p(c->prec, c->Qmax, Z, c->Mmax);
-    c->smem_df = stage_smem_bytes_df(c->Qmax, Z, c->Mmax);
+    c->smem = stage_smem_bytes_p(c->df ? EVFDLB_FP64_DF : c->prec, c->Qmax, Z, c->Mmax);
     if (c->items_cap == 0) c->items_cap = (size_t)c->NN;
     c->tiles_h.assign(c->nbatch, 0);
     for (const WorkItem& w : c->items_h) ++c->tiles_h[w.slab];
@@ -636,21 +632,9 @@ evfdlb_status evfdlb_create(const evfdlb_params* p, int32_t nbatch, const evfdlb
     if (e == cudaSuccess)
         e = cudaMemcpy(c->items, c->items_h.data(), sizeof(WorkItem) * c->items_h.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(c->err, 0, sizeof(unsigned));
-    if (e == cudaSuccess) e = configure_kernels_p(c->prec, stage_smem_bytes_p(c->prec, Qmax, kZMax, Mmax));
-    if (e == cudaSuccess && c->df) {
-        // analysis and synthesis tables as (hi, lo) float pairs in 8-byte slots
-        std::vector<double> dft(tables.size());
-        for (size_t i = 0; i < tables.size(); ++i) {
-            float pr[2];
-            pr[0] = (float)tables[i];
-            pr[1] = (float)(tables[i] - (double)pr[0]);
-            memcpy(&dft[i], pr, sizeof(pr));
-        }
-        alloc((void**)&c->dftables, sizeof(double) * dft.size());
-        if (e == cudaSuccess)
-            e = cudaMemcpy(c->dftables, dft.data(), sizeof(double) * dft.size(), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = configure_df(stage_smem_bytes_df(Qmax, kZMax, Mmax));
-    }
+    const size_t cap = stage_smem_cap_p(c->df ? EVFDLB_FP64_DF : c->prec, Qmax, Mmax);
+    if (e == cudaSuccess) e = configure_kernels_p(c->prec, cap);
+    if (e == cudaSuccess && c->df) e = configure_df(cap);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         evfdlb_status st = cuda_status(e);
@@ -825,8 +809,8 @@ evfdlb_status evfdlb_rhs(evfdlb_ctx* c, double* RF, double* RG, int32_t on_devic
     if (!c->have_state) return EVFDLB_E_STATE;
     if (c->halo) return EVFDLB_E_UNSUPPORTED;
     if (c->df)
-        launch_stage_df((int)c->items_h.size(), c->smem_df, c->user, c->slabs, c->items, c->tables, c->dftables,
-                        c->taps, (const double*)c->state[0], nullptr, nullptr, c->scratch, c->mom[0], nullptr, c->NF,
+        launch_stage_df((int)c->items_h.size(), c->smem, c->user, c->slabs, c->items, c->tables, c->taps,
+                        (const double*)c->state[0], nullptr, nullptr, c->scratch, c->mom[0], nullptr, c->NF,
                         c->NN, 0.0, 1.0, 1, c->Z, c->err);
     else
         launch_stage_p(c->prec, (int)c->items_h.size(), c->smem, c->user, c->slabs, c->items, c->tables,

@@ -8,6 +8,7 @@
 // public interface.
 #pragma once
 
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -63,7 +64,8 @@ struct Smem {
     R *Nr;              // n halo in R (the force convolution), aliases N for FP64
     R *Scr;             // nu and F1 in R, [2][Z]
     R *C;               // coefficients [2][Q][Z] (block of 4 H Z >= 2 Q Z values)
-    R *A;               // analysis [2][Q][Z]
+    R *A;               // analysis [2][Q][Z] (on the tensor cores: then the integer
+                        // parts of the synthesis, [2 d][H even, Q - H odd][Z])
     R *F;               // state tile with halo [2][Q][Z+6]
     R *Face;            // WENO face values [2][Q][Z+1]
     R *Cc;              // per-node coefficient constants c0..c3 [2][4][Z]
@@ -73,8 +75,11 @@ struct Smem {
     R *Vr;              //   and xi, xi^3 in R [2Q]
     R *EO;              // parity-split state tile [2][2][H][Z] (d, E/O), H = (Q+1)/2; it is
                         // read only before the coefficients are formed, so it shares
-                        // their block; the FP64_DF kernel keeps its float-pair state
-                        // tile there instead
+                        // their block
+    // set by stage_tables:
+    const R *Rec;       // recurrence constants rinv, rr, r1, r2, r3 [5Q]
+    const uint4 *Ma, *Ms;   // digit slices of the transforms on the tensor cores
+    int *Ti;            //   and their exponents sx [16], rk [16], gl [32]
     double *Mp64;       // FP32 state only: group terms of the FP64 moment sums [4][G][Z]
     R *Mp32;            //   and of the R ones [2][G][Z] (see pair_terms_f32)
 };
@@ -93,19 +98,55 @@ __host__ __device__ inline int pair_groups(int Q) { return ((Q + 1) / 2 + 1) / 2
 // two-wide (R2) loads.
 __host__ __device__ inline size_t qq_len(int Q) { return ((size_t)Q * Q + 1) & ~(size_t)1; }
 
+// Whether the transforms of an FP64 state run on the tensor cores (FP64_DF: all).
+template <typename R, bool DF = false>
+__host__ __device__ inline bool on_tensor_cores(int Q) {
+    return std::is_same<R, double>::value && (DF || Q >= kTsMinQ);
+}
+
+// Length of the table block (s.P and s.S, up to Q*Q entries each; with the
+// transforms on the tensor cores their exponents, the recurrence constants and the
+// scratch of tile_moment_sums, as long as the largest other Q's tables, so that
+// a batch's largest Q needs the most), even.
+template <typename R>
+__host__ __device__ inline size_t tab_len(int Q) {
+    return 2 * qq_len(on_tensor_cores<R>(Q) ? kTsMinQ - 1 : Q);
+}
+
+// Length of the block of the FP64 stage's recurrence constants: none where they fit
+// into the per-node scalars that its roles leave free (SC_U, SC_FORCE; the last
+// place there holds the pools) or, with the transforms on the tensor cores, into
+// the table block (counted all the same, as in tab_len).  FP32 reads them from
+// global memory.
+template <typename R>
+__host__ __device__ inline size_t rec_len(int Q, int Z) {
+    const int q = on_tensor_cores<R>(Q) ? kTsMinQ - 1 : Q;
+    return std::is_same<R, float>::value || 5 * q < 2 * Z ? 0 : 5 * (size_t)q;
+}
+
 template <typename R>
 __host__ __device__ inline size_t smem_bytes_t(int Q, int Z, int M) {
     // the FP64 block is padded to an even count (16-byte aligned R2 tables)
     size_t nd = (size_t)(Z + 2 * M) + 4 * (size_t)(Z + 4) + (size_t)kNumScalars * Z + (size_t)(2 * M + 1);
     nd = (nd + 1) & ~(size_t)1;
-    size_t nr = 2 * qq_len(Q) + (std::is_same<R, double>::value ? 0 : nr_len(Z, M)) + 2 * (size_t)Z +
+    size_t nr = tab_len<R>(Q) + (std::is_same<R, double>::value ? 0 : nr_len(Z, M)) + 2 * (size_t)Z +
                 4 * (size_t)((Q + 1) / 2) * Z + 2 * (size_t)Q * Z + 2 * (size_t)Q * (Z + 6) +
                 2 * (size_t)Q * (Z + 1) + 8 * (size_t)Z + ftap_len(M) + (size_t)Q * Z;
     // + the velocity powers (3Q doubles, 2Q R) and one R of padding before them
     size_t bytes = (nd + 3 * (size_t)Q) * sizeof(double) + (nr + 2 * (size_t)Q + 1) * sizeof(R);
+    bytes += rec_len<R>(Q, Z) * sizeof(R);
     // + the pair terms of the moment sums (FP32 state)
     if (std::is_same<R, float>::value) bytes += (size_t)pair_groups(Q) * Z * (4 * sizeof(double) + 2 * sizeof(R));
     return bytes;
+}
+
+// The digit slices of transforms on the tensor cores lie behind that.  A launch
+// whose shared memory does not hold them (a large tile beside thousands of force
+// taps) reads them from global memory instead.
+template <typename R, bool DF>
+__host__ __device__ inline size_t stage_full_bytes(int Q, int Z, int M) {
+    if (!on_tensor_cores<R, DF>(Q)) return smem_bytes_t<R>(Q, Z, M);
+    return ((smem_bytes_t<R>(Q, Z, M) + 15) & ~(size_t)15) + 2 * (size_t)kTsDoubles * sizeof(double);
 }
 
 template <typename R>
@@ -126,9 +167,9 @@ __device__ inline Smem<R> carve(double* base, int Q, int Z, int M) {
     s.S = s.P + qq_len(Q);
     if constexpr (std::is_same<R, double>::value) {
         s.Nr = s.N;
-        s.Scr = s.S + qq_len(Q);
+        s.Scr = s.P + tab_len<R>(Q);
     } else {
-        s.Nr = s.S + qq_len(Q);
+        s.Nr = s.P + tab_len<R>(Q);
         s.Scr = s.Nr + nr_len(Z, M);
     }
     s.C = s.Scr + 2 * Z;
@@ -149,7 +190,7 @@ __device__ inline Smem<R> carve(double* base, int Q, int Z, int M) {
     return s;
 }
 
-enum { SC_N = 0, SC_U, SC_T, SC_NU, SC_FORCE, SC_KQ, SC_K, SC_A, SC_B, SC_D };
+enum { SC_N = 0, SC_U, SC_FORCE, SC_T, SC_NU, SC_KQ, SC_K, SC_A, SC_B, SC_D };
 
 // IEEE tests by the bit pattern: integer operations, not the FP64 pipe
 // (whose compares sit on the node chain's critical path).
@@ -192,14 +233,8 @@ __device__ __forceinline__ T gload(const T* p) {
 }
 
 // ---------------------------------------------------------------------------
-// Double-float arithmetic for the FP64_DF variant: a value is an unevaluated
-// pair of floats (hi, lo) with x = hi + lo to about 48 significant bits.  Sums of products use the compensated dot product Dot2
-// of Ogita, Rump & Oishi ("Accurate sum and dot product", SIAM J. Sci.
-// Comput. 26, 2005): the error-free TwoProduct (by FMA) and TwoSum (Knuth)
-// of every term, errors collected in a second float; the cross terms
-// hi*lo of pair operands join the error float.  The result carries about
-// twice the float precision.  __fadd_rn / __fmul_rn keep the compiler from
-// contracting the error-free transformations into FMAs.
+// Double-float arithmetic: a value is an unevaluated pair of floats (hi, lo) with
+// x = hi + lo to about 48 significant bits.
 // ---------------------------------------------------------------------------
 // The split is exact bit surgery, no FP64 instruction: hi is x with its
 // significand cut to 24 bits (the top 23 stored bits), lo the remaining 29
@@ -226,7 +261,6 @@ __device__ __forceinline__ float2 df_split(double x) {
     }
     return make_float2(h, l);
 }
-__device__ __forceinline__ double df_join(float s, float e) { return (double)s + (double)e; }
 // double -> float by bit surgery (the head of df_split: the significand cut
 // to 24 bits, within one float ulp), no conversion instruction
 __device__ __forceinline__ float d2f_bits(double x) { return df_split(x).x; }
@@ -257,6 +291,11 @@ __device__ __forceinline__ double div_nr(double a, double b) {
     return fma(fma(-b, q, a), r, q);
 }
 
+// div_nr as one copy of its code: a warp that runs straight-line code once waits
+// for its instructions (9 of 10 stalls on the stage of 256 x 16 with every
+// quotient of the node roles inlined: 12.5 -> 11.6 us).
+static __device__ __noinline__ double div_call(double a, double b) { return div_nr(a, b); }
+
 // a / b to about 2^-46 relative: the float-seeded reciprocal of div_nr after
 // its Newton step, times a, without the residual correction (3 FP64
 // operations instead of 5).  For the WENO-5 face quotient: its error enters
@@ -271,57 +310,57 @@ __device__ __forceinline__ double div_face(double a, double b) {
     return a * r;
 }
 
-// (s, e) += a * b for pairs a, b.
-__device__ __forceinline__ void dot2_acc(float& s, float& e, float2 a, float2 b) {
-    const float p = __fmul_rn(a.x, b.x);
-    const float pe = fmaf(a.x, b.x, -p);            // exact: a.x b.x = p + pe
-    const float t = __fadd_rn(s, p);
-    const float z = __fsub_rn(t, s);
-    const float te = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z));   // exact: s + p = t + te
-    e = __fadd_rn(e, __fadd_rn(te, pe));
-    e = fmaf(a.x, b.y, e);
-    e = fmaf(a.y, b.x, e);
-    s = t;
-}
-
-
 // ---------------------------------------------------------------------------
 // Phase 0: stage the tables, the density halo, u/T near the tile and the
 // state tile (+-3 nodes for WENO-5) into shared memory.
 // ---------------------------------------------------------------------------
-// PARITY: the parity-split tables Pp and Sp go to s.P and s.S in place of
-// the full analysis and synthesis tables.
-// CG: the moment sums are read with L2-coherent loads (written earlier in
-// the same launch by other CTAs).
-// The velocity tables of the slab into shared memory: the parity-split
-// analysis pairs and synthesis rows (PARITY), else the full P and S.
-template <typename R, bool PARITY = false>
-__device__ void load_velocity_tables(const SlabDesc& sd, const Smem<R>& s, const R* __restrict__ rtab) {
+// The transform tables of the slab: the digit slices where the transforms run
+// on the tensor cores, else the parity-split analysis pairs and synthesis rows;
+// and the recurrence constants.
+template <typename R, bool DF>
+__device__ void stage_tables(const SlabDesc& sd, Smem<R>& s, int Z, double* smem, const R* __restrict__ rtab) {
     const int Q = sd.Q;
     TableLayout L(Q);
     const R* tab = rtab + sd.tab_off;
-    if constexpr (PARITY) {
+    const bool ts = on_tensor_cores<R, DF>(Q);
+    if constexpr (std::is_same<R, double>::value) {
+        double* rec = on_tensor_cores<R>(Q) ? s.P + kTsInts / 2
+                                            : (rec_len<R>(Q, Z) == 0 ? s.Sc + SC_U * Z : s.Vr + 2 * Q);
+        for (int t = threadIdx.x; t < 5 * Q; t += blockDim.x) rec[t] = tab[L.rinv + t];   // rinv .. r3 in a row
+        s.Rec = rec;
+        s.Ti = reinterpret_cast<int*>(s.P);
+    } else {
+        s.Rec = tab + L.rinv;
+    }
+    if (ts) {
+        if (threadIdx.x < kTsInts) s.Ti[threadIdx.x] = reinterpret_cast<const int*>(tab + L.Mi)[threadIdx.x];
+        s.Ma = reinterpret_cast<const uint4*>(tab + L.Ma);
+        s.Ms = reinterpret_cast<const uint4*>(tab + L.Ms);
+        unsigned dyn;
+        asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
+        if (stage_full_bytes<R, DF>(Q, Z, sd.M) <= dyn) {
+            uint4* x = reinterpret_cast<uint4*>(reinterpret_cast<char*>(smem) + ((smem_bytes_t<R>(Q, Z, sd.M) + 15) & ~(size_t)15));
+#pragma unroll 4
+            for (int t = threadIdx.x; t < kTsDoubles; t += blockDim.x) x[t] = s.Ma[t];   // Ma, Ms in a row
+            s.Ma = x;
+            s.Ms = x + kTsDoubles / 2;
+        }
+    }
+    if (!ts) {
         const ParitySplit ps(Q);
         const int la = ps.analysis_len(), ls = ps.synthesis_len();
 #pragma unroll 4
         for (int t = threadIdx.x; t < la; t += blockDim.x) s.P[t] = tab[L.Pp + t];
 #pragma unroll 4
         for (int t = threadIdx.x; t < ls; t += blockDim.x) s.S[t] = tab[L.Sp + t];
-    } else {
-        for (int t = threadIdx.x; t < Q * Q; t += blockDim.x) {
-            s.P[t] = tab[L.P + t];
-            s.S[t] = tab[L.S + t];
-        }
     }
 }
 
-// The velocity tables and the node inputs of the tile (TABLES false: the
-// node inputs only, the tables being staged already).
-template <typename R, bool PARITY = false, bool CG = false, bool TABLES = true>
+// The node inputs of the tile.
+template <typename R, bool CG = false>
 __device__ void load_node_inputs(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, int Z,
-                                 const R* __restrict__ rtab, const double* __restrict__ mom, long long NN) {
+                                 const double* __restrict__ mom, long long NN) {
     const int M = sd.M, nx = sd.nx, bc = sd.bc;
-    if constexpr (TABLES) load_velocity_tables<R, PARITY>(sd, s, rtab);
     const double* S0 = mom + MOM_S0 * NN + sd.node_off;
 #pragma unroll 2
     for (int t = threadIdx.x; t < it.nz + 2 * M; t += blockDim.x) {
@@ -352,23 +391,6 @@ __device__ void load_node_inputs(const SlabDesc& sd, const WorkItem& it, const S
         // fields read it from the KQ slot, which they then overwrite with (1 - Pr) q
         if (tile)
             s.Sc[SC_KQ * Z + (t - 2)] = 0.5 * (s3 - 3.0 * u * s2 + 3.0 * u * u * s1 - u * u * u * n) + g1 - u * g0;
-    }
-}
-
-// With Fd (FP64_DF), the tile's interior columns are also stored as
-// double-float pairs, Fd[(d Q + k) Z + t].
-template <typename R>
-__device__ void load_state_tile(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, int Z,
-                                const R* __restrict__ src, long long NF, float2* Fd = nullptr) {
-    const int Q = sd.Q, nx = sd.nx, bc = sd.bc, W = Z + 6;
-    const int cols = it.nz + 6;
-    for (int e = threadIdx.x; e < 2 * Q * cols; e += blockDim.x) {
-        int c = e % cols, r = e / cols;
-        int k = r % Q, d = r / Q;
-        int i = gidx(it.i0 - 3 + c, nx, bc);
-        R v = src[d * NF + sd.f_off + (long long)k * nx + i];
-        s.F[(d * Q + k) * W + c] = v;
-        if (Fd && c >= 3 && c < it.nz + 3) Fd[(size_t)r * Z + c - 3] = df_split((double)v);
     }
 }
 
@@ -641,8 +663,7 @@ __device__ void node_fields(const SlabDesc& sd, const WorkItem& it, const Smem<R
 // m_0 = 1, m_{l+1} = u m_l / sqrt(l+1) + (T-1) sqrt(l/(l+1)) m_{l-1}, to
 // mm[l stride] (u, T widened or narrowed to R as the node constants are)
 template <typename R>
-__device__ __forceinline__ void hermite_moments(int Q, const TableLayout& L, const R* __restrict__ tab, double u,
-                                                double T, R* mm, int stride) {
+__device__ __forceinline__ void hermite_moments(int Q, const R* rec, double u, double T, R* mm, int stride) {
     R ru, Tm1;
     if constexpr (std::is_same<R, float>::value) {
         ru = d2f_bits(u);
@@ -654,7 +675,7 @@ __device__ __forceinline__ void hermite_moments(int Q, const TableLayout& L, con
     R m0 = 1, m1 = 0;
     for (int l = 0; l < Q; ++l) {
         mm[l * stride] = m0;
-        R mn = fma(ru * tab[L.rinv + l], m0, Tm1 * tab[L.rr + l] * m1);
+        R mn = fma(ru * rec[l], m0, Tm1 * rec[Q + l] * m1);
         m1 = m0;
         m0 = mn;
     }
@@ -685,11 +706,9 @@ __device__ inline void node_coefficients(const SlabDesc& sd, const WorkItem& it,
 // nodes (the recurrence of node_coefficients) from the node inputs u, T of
 // load_node_inputs, by threads tid, tid + nth, ...
 template <typename R>
-__device__ void node_hermite_moments(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, int Z,
-                                     const R* __restrict__ tab, int tid, int nth) {
-    const int Q = sd.Q;
-    TableLayout L(Q);
-    for (int t = tid; t < it.nz; t += nth) hermite_moments<R>(Q, L, tab, s.U[t + 2], s.T[t + 2], s.Mm + t, Z);
+__device__ void node_hermite_moments(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, int Z, int tid,
+                                     int nth) {
+    for (int t = tid; t < it.nz; t += nth) hermite_moments<R>(sd.Q, s.Rec, s.U[t + 2], s.T[t + 2], s.Mm + t, Z);
 }
 
 // ---------------------------------------------------------------------------
@@ -778,8 +797,8 @@ __device__ __forceinline__ int lanes_per(int n, int most) {
 }
 
 template <bool FO>
-__device__ void node_roles(const SlabDesc& sd, const WorkItem& it, const Smem<double>& s, int Z,
-                           const double* __restrict__ tab, long long NN, unsigned* err, double* fields_out) {
+__device__ void node_roles(const SlabDesc& sd, const WorkItem& it, const Smem<double>& s, int Z, long long NN,
+                           unsigned* err, double* fields_out) {
     const int M = sd.M, nz = it.nz, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double* sc = s.Sc;
     auto join3 = [] { asm volatile("bar.sync 1, 96;" ::: "memory"); };    // warps 0, 1, 2
@@ -797,7 +816,7 @@ __device__ void node_roles(const SlabDesc& sd, const WorkItem& it, const Smem<do
             const int shift = (sd.bc == EVFDLB_BC_OUTFLOW) ? gidx(pos, sd.nx, sd.bc) - pos : 0;
             const double nb = chain_sum<4>(s.Mtap, s.N + (t - 2 + M + shift - sd.m), 2 * sd.m + 1, lp, sub);
             const double eta = sd.eta_coef * nb, om = 1.0 - eta;
-            const double chi = div_nr(2.0 - eta, 2.0 * om * om * om);
+            const double chi = div_call(2.0 - eta, 2.0 * om * om * om);
             if (sub == 0) {
                 s.Chi[t] = chi;
                 if (t >= 2 && t < nz + 2) field(4, t - 2, nb);
@@ -815,9 +834,9 @@ __device__ void node_roles(const SlabDesc& sd, const WorkItem& it, const Smem<do
             const double n = s.N[t + M], T = s.T[t + 2], chi = s.Chi[t + 2], q = sc[SC_KQ * Z + t];
             const double c16 = (4.0 / 25.0) * (1.0 + 12.0 / M_PI), c9 = (9.0 / 25.0) * (1.0 + 32.0 / (9.0 * M_PI));
             const double x = sd.b * n * chi, a = fma(0.4, x, 1.0), P = fma(fma(c16, x, 0.8), x, 1.0), st = sqrt(T);
-            double nu = div_nr(n * st * chi * a, sd.mu0_coef * P);
+            double nu = div_call(n * st * chi * a, sd.mu0_coef * P);
             if (sd.relax != EVFDLB_RELAX_INV_TAU) nu *= chi;
-            const double Pr = div_nr(fma(0.4, x, 2.0 / 3.0) * P, a * fma(fma(c9, x, 1.2), x, 1.0));
+            const double Pr = div_call(fma(0.4, x, 2.0 / 3.0) * P, a * fma(fma(c9, x, 1.2), x, 1.0));
             sc[SC_N * Z + t] = n;
             sc[SC_T * Z + t] = T;
             sc[SC_NU * Z + t] = nu;
@@ -827,14 +846,14 @@ __device__ void node_roles(const SlabDesc& sd, const WorkItem& it, const Smem<do
             if (!positive(n) || !positive(T)) atomicOr(err, (finite(n) && finite(T)) ? ERR_NEGATIVE : ERR_NONFINITE);
             else if (!finite(nu) || !finite(q)) atomicOr(err, ERR_NONFINITE);
             if constexpr (FO) {
-                const double mu = sd.mu0_coef * st * div_nr(P, chi);
+                const double mu = sd.mu0_coef * st * div_call(P, chi);
                 field(0, t, n);
                 field(1, t, s.U[t + 2]);
                 field(2, t, T);
                 field(3, t, q);
                 field(5, t, chi);
                 field(7, t, mu);
-                field(8, t, div_nr(mu, n * T * a));
+                field(8, t, div_call(mu, n * T * a));
                 field(9, t, Pr);
                 field(10, t, nu);
                 field(14, t, s.X[t + 2]);
@@ -866,7 +885,7 @@ __device__ void node_roles(const SlabDesc& sd, const WorkItem& it, const Smem<do
             const int pos = it.i0 - 2 + t;
             const int shift = (sd.bc == EVFDLB_BC_OUTFLOW) ? gidx(pos, sd.nx, sd.bc) - pos : 0;
             const double n = s.N[t - 2 + M + shift], s1 = s.U[t], s2 = s.T[t], g0 = s.X[t];
-            const double inv_n = div_nr(1.0, n), u = s1 * inv_n;
+            const double inv_n = div_call(1.0, n), u = s1 * inv_n;
             s.U[t] = u;
             // (3/2) n T = sum (xi-u)^2/2 F + sum G = S2/2 + G0 - n u^2/2
             s.T[t] = (2.0 / 3.0) * fma(fma(0.5, s2, g0), inv_n, -0.5 * u * u);
@@ -881,11 +900,11 @@ __device__ void node_roles(const SlabDesc& sd, const WorkItem& it, const Smem<do
         auto d4 = [&](const double* f) { return fma(8.0, f[1] - f[-1], f[-2] - f[2]) * inv12; };
         for (int t = lane; t < nz; t += 32) {
             sc[SC_D * Z + t] = d4(s.U + t + 2);
-            sc[SC_B * Z + t] = div_nr(d4(s.T + t + 2), s.T[t + 2]);
+            sc[SC_B * Z + t] = div_call(d4(s.T + t + 2), s.T[t + 2]);
         }
         join2();
         for (int t = lane; t < nz; t += 32) {
-            const double A = div_nr(d4(s.X + t + 2), s.X[t + 2]), B = sc[SC_B * Z + t];
+            const double A = div_call(d4(s.X + t + 2), s.X[t + 2]), B = sc[SC_B * Z + t];
             sc[SC_A * Z + t] = A;
             if (node_ok(t) && (!finite(A) || !finite(B))) atomicOr(err, ERR_NONFINITE);
             field(11, t, A);
@@ -895,8 +914,7 @@ __device__ void node_roles(const SlabDesc& sd, const WorkItem& it, const Smem<do
         join2();
     } else if (warp == 2) {
         join3();
-        TableLayout L(sd.Q);
-        for (int t = lane; t < nz; t += 32) hermite_moments<double>(sd.Q, L, tab, s.U[t + 2], s.T[t + 2], s.Mm + t, Z);
+        for (int t = lane; t < nz; t += 32) hermite_moments<double>(sd.Q, s.Rec, s.U[t + 2], s.T[t + 2], s.Mm + t, Z);
     } else {
         // self-consistent force, Eq. (F1) (or the merged Eq. (F2) stencil)
         const int lp = lanes_per(nz, 8), sub = lane % lp;
@@ -912,13 +930,11 @@ __device__ void node_roles(const SlabDesc& sd, const WorkItem& it, const Smem<do
     }
 }
 
-// With DF the coefficients are stored as double-float pairs (float2) in the
-// same block, for the double-float synthesis.
-template <typename R, bool DF = false>
-__device__ void coefficients(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, int Z,
-                             const R* __restrict__ tab, int tid, int nth) {
+template <typename R>
+__device__ void coefficients(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, int Z, int tid,
+                             int nth) {
     const int Q = sd.Q, nz = it.nz;
-    TableLayout L(Q);
+    const R *r1 = s.Rec + 2 * Q, *r2 = s.Rec + 3 * Q, *r3 = s.Rec + 4 * Q;
     // one (l, node) per item, both distributions: the scaled moments
     // sqrt(l(l-1)..) m_{l-j} and the force factor F1 sqrt(l) are shared
     for (int e = tid; e < Q * nz; e += nth) {
@@ -926,10 +942,10 @@ __device__ void coefficients(const SlabDesc& sd, const WorkItem& it, const Smem<
         const R* mm = s.Mm + t;
         // the sqrt factors vanish where the moment index would be negative
         const R m0 = mm[l * Z];
-        const R M1 = tab[L.r1 + l] * mm[max(l - 1, 0) * Z];
-        const R M2 = tab[L.r2 + l] * mm[max(l - 2, 0) * Z];
-        const R M3 = tab[L.r3 + l] * mm[max(l - 3, 0) * Z];
-        const R f = s.Scr[Z + t] * tab[L.r1 + l];
+        const R M1 = r1[l] * mm[max(l - 1, 0) * Z];
+        const R M2 = r2[l] * mm[max(l - 2, 0) * Z];
+        const R M3 = r3[l] * mm[max(l - 3, 0) * Z];
+        const R f = s.Scr[Z + t] * r1[l];
 #pragma unroll
         for (int d = 0; d < 2; ++d) {
             const R* cc = s.Cc + d * 4 * Z + t;
@@ -938,8 +954,7 @@ __device__ void coefficients(const SlabDesc& sd, const WorkItem& it, const Smem<
             c = fma(cc[2 * Z], M2, c);
             c = fma(cc[3 * Z], M3, c);
             if (l >= 1) c = fma(f, s.A[((size_t)d * Q + l - 1) * Z + t], c);
-            if constexpr (DF) reinterpret_cast<float2*>(s.C)[((size_t)d * Q + l) * Z + t] = df_split((double)c);
-            else s.C[((size_t)d * Q + l) * Z + t] = c;
+            s.C[((size_t)d * Q + l) * Z + t] = c;
         }
     }
 }
@@ -958,31 +973,228 @@ __device__ __forceinline__ void warp_pool(int* next, int n, F f) {
     }
 }
 
-// Analysis a_l = sum_j psi_l(xi_j) h_j, l <= Q-2 (the force needs
-// a_0 .. a_{Q-2}; the l = Q-1 term meets psi_Q(xi_k) = 0), two orders per
-// thread so that each state value loaded feeds two FMAs.
-template <typename R>
-__device__ void analysis(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, int Z, int tid, int nth) {
-    const int Q = sd.Q, W = Z + 6, nz = it.nz;
-    const int np = Q / 2;                          // pairs (l, l+1) covering l <= Q-2
-    const int per_d = np * nz;
-    for (int e = tid; e < 2 * per_d; e += nth) {
-        int d = e / per_d, r = e % per_d;
-        int l0 = 2 * (r / nz), t = r % nz;
-        const bool two = (l0 + 1 <= Q - 2);
-        const R* P0 = s.P + l0 * Q;
-        const R* P1 = s.P + (two ? l0 + 1 : l0) * Q;
-        const R* h = s.F + (size_t)d * Q * W + (t + 3);
-        R a0 = 0, a1 = 0;
-        for (int j = 0; j < Q; ++j) {
-            R hv = h[j * W];
-            a0 = fma(P0[j], hv, a0);
-            a1 = fma(P1[j], hv, a1);
-        }
-        s.A[((size_t)d * Q + l0) * Z + t] = a0;
-        if (two) s.A[((size_t)d * Q + l0 + 1) * Z + t] = a1;
+// ---------------------------------------------------------------------------
+// The Hermite transforms of an FP64 stage on the tensor cores, in fixed point
+// (see kTsSlices): one warp forms both parities of one distribution for eight
+// nodes.  A lane holds the values of rows 2 (lane % 4) + {0, 1, 8, 9} of node
+// lane / 4 (the fragment of mma.m16n8k16's B operand), turns them into
+// integers on the node's own exponent, cuts their digits, and 21 products per
+// parity of digit slices accumulate exactly; the six accumulators join in
+// 64-bit integers, which become doubles by bit operations.  Nothing runs on the
+// FP64 pipe, which bounds the stage and spent a third of it on the sums.  The
+// result carries about 2^-56 of the largest value times the largest entry, below
+// the rounding of an FP64 sum of up to 16 terms (2^-53 each): a step's error
+// against 80-bit arithmetic is that of the plain sums or less.  Columns
+// (nodes) are independent, so results do not depend on the tile.  Stage of
+// 4096 x 32: 44.6 -> 33.8 us, of 65536 x 24 (tile 32): 438 -> 328 us.
+//
+// A warp's work is a chain of integer operations (about 900 instructions a
+// parity, mostly the digits and the joins; the products take 180 cycles), so the
+// phase is bound by latency: values and results go through it four at a time.
+// FP64_DF with Q <= 16 has both parities in one block (even orders in rows and
+// columns 0-7, odd in 8-15).
+// ---------------------------------------------------------------------------
+// sign, exponent field (with `shift` added; 0 for zero and subnormal values)
+// and 53-bit significand of x
+struct FixIn {
+    unsigned hi, lo;
+    int e;
+};
+__device__ __forceinline__ FixIn fix_in(double x, int shift) {
+    FixIn f;
+    f.hi = (unsigned)__double2hiint(x);
+    f.lo = (unsigned)__double2loint(x);
+    const int e = (int)((f.hi >> 20) & 0x7ffu);
+    f.e = e == 0 ? -100000 : (e == 2047 ? 100000 : e + shift);
+    return f;
+}
+// x 2^(lead + 1075 - emax), rounded (emax >= the exponent of x; zero if none)
+__device__ __forceinline__ long long fix_value(const FixIn& f, int emax, int lead) {
+    // one bit more than wanted, then rounded by it
+    const unsigned sh = (unsigned)min(emax - f.e, 63);
+    const unsigned long long m = (((unsigned long long)((f.hi & 0xfffffu) | 0x100000u) << 32) | f.lo) << (lead + 1);
+    const long long v = (long long)(((m >> sh) + 1) >> 1);
+    return (int)f.hi < 0 ? -v : v;
+}
+// digit slices of two values |v| < 2^59 as FP16 pairs, most significant first
+__device__ __forceinline__ void fix_slices(long long va, long long vb, unsigned (&out)[kTsSlices]) {
+    // + 512 in every digit makes them the unsigned 10-bit fields u of the sum
+    // (the top one up to 1024); 0x6400 + u is the FP16 number 1024 + u
+    constexpr unsigned long long bias = 512ull * (1ull + (1ull << 10) + (1ull << 20) + (1ull << 30) + (1ull << 40) + (1ull << 50));
+    const unsigned long long a = (unsigned long long)va + bias, b = (unsigned long long)vb + bias;
+    const __half2 off = __half2half2(__short_as_half((short)0x6600));           // 1536 = 1024 + 512
+#pragma unroll
+    for (int i = 0; i < kTsSlices; ++i) {
+        const int pos = 10 * (kTsSlices - 1 - i);
+        unsigned ua = (unsigned)(a >> pos), ub = (unsigned)(b >> pos);
+        if (i > 0) ua &= 1023u, ub &= 1023u;
+        const unsigned w = 0x64006400u + (ua | (ub << 16));
+        const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&w), off);
+        out[i] = *reinterpret_cast<const unsigned*>(&h);
     }
 }
+// acc[s] += the slice products of weight s: table slices A (global fragment
+// order in shared memory) times value slices (b0: rows k, k+1; b1: k+8, k+9)
+__device__ __forceinline__ void fix_products(const uint4* A, const unsigned (&b0)[kTsSlices],
+                                             const unsigned (&b1)[kTsSlices], float (&acc)[kTsSlices][4]) {
+#pragma unroll
+    for (int s = 0; s < kTsSlices; ++s)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[s][c] = 0.f;
+#pragma unroll
+    for (int i = 0; i < kTsSlices; ++i) {
+        const uint4 a = A[i * 32 + (threadIdx.x & 31)];
+#pragma unroll
+        for (int k = 0; i + k < kTsSlices; ++k) {
+            float(&c)[4] = acc[i + k];
+            asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3},{%4,%5,%6,%7},{%8,%9},{%0,%1,%2,%3};"
+                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0[k]), "r"(b1[k]));
+        }
+    }
+}
+// the sum of the accumulators of element c, in units of 2^3
+__device__ __forceinline__ long long fix_join(const float (&acc)[kTsSlices][4], int c) {
+    auto g = [&](int s) {
+        return ((long long)__float2int_rn(acc[s][c]) << 20) + ((long long)__float2int_rn(acc[s + 1][c]) << 10) +
+               __float2int_rn(acc[s + 2][c]);
+    };
+    return (g(0) << 18) + ((g(3) + 2048) >> 12);
+}
+// Four values of a lane's node through one 16 x 16 block of the table: results
+// for rows lane / 4 (+ 8) of nodes 2 (lane % 4) (+ 1) in the order of the
+// accumulator fragment.  One copy of the code serves every task: straight-line
+// code that a CTA runs once waits for its instructions (half of all stalls of
+// the stage of 4096 x 32 with the tasks inlined, 9 of 10 on 256 x 16).
+struct Fix4 {
+    long long v[4];
+};
+static __device__ __noinline__ Fix4 fix_transform(const uint4* A, Fix4 x) {
+    unsigned b0[kTsSlices], b1[kTsSlices];
+    fix_slices(x.v[0], x.v[1], b0);
+    fix_slices(x.v[2], x.v[3], b1);
+    float acc[kTsSlices][4];
+    fix_products(A, b0, b1, acc);
+    Fix4 o;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) o.v[c] = fix_join(acc, c);
+    return o;
+}
+// v 2^q as a double, rounded to nearest (ties away; zero below the normal
+// range), |v| < 2^62; NaN when `bad`
+__device__ __forceinline__ double fix_out(long long v, int q, bool bad) {
+    const unsigned long long a = (unsigned long long)(v < 0 ? -v : v);
+    const int lz = __clzll((long long)a);
+    const int e = 62 - lz + q + 1023;                          // exponent field - 1: the leading bit adds one
+    // the significand with its leading bit at 52, rounded; a carry out of it
+    // goes into the exponent as it should
+    unsigned long long r = ((unsigned long long)e << 52) + (((a << (lz - 1)) + 0x200ull) >> 10);
+    if (a == 0 || e < 0) r = 0;
+    if (e >= 2046) r = 0x7ff0000000000000ull;
+    if (v < 0) r |= 0x8000000000000000ull;
+    if (bad) r = 0x7ff8000000000000ull;
+    return __longlong_as_double((long long)r);
+}
+
+// the largest of a value over the four lanes of a node
+__device__ __forceinline__ int quad_max(int e) {
+    e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
+    return max(e, __shfl_xor_sync(0xffffffffu, e, 2));
+}
+
+// Task g of the analysis, a_l = sum_{j<H} psi_l(xi_j) (E_j or O_j), l <= Q-2, E_j
+// = h_j + h_{Q-1-j}, O_j = h_j - h_{Q-1-j} (the middle velocity of an odd Q: h, 0),
+// formed as integers: distribution g % 2, nodes 8 (g / 2) .. + 7, parities p0 .. p1 - 1.
+template <bool DF>
+__device__ __forceinline__ void analysis_task(const SlabDesc& sd, const WorkItem& it, const Smem<double>& s, int Z,
+                                              int g, int p0, int p1) {
+    const int Q = sd.Q, H = (Q + 1) / 2, W = Z + 6, nz = it.nz, lane = threadIdx.x & 31;
+    const int d = g & 1, t0 = (g >> 1) * 8, t = min(t0 + lane / 4, nz - 1), k0 = 2 * (lane % 4);
+    const double* h = s.F + (size_t)d * Q * W + t + 3;
+    FixIn x[4], y[4];
+    int emax = -100000;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const int j = k0 + (c & 1) + 8 * (c >> 1), jm = Q - 1 - j;
+        const bool in = j < H;
+        const int sx = in ? s.Ti[j] : 0;
+        x[c] = fix_in(in ? h[j * W] : 0.0, -sx);
+        y[c] = fix_in(in && jm != j ? h[jm * W] : 0.0, -sx);
+        emax = max(emax, max(x[c].e, y[c].e));
+    }
+    emax = quad_max(emax);
+    const bool bad = emax > 50000;
+    long long E[4], O[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const int j = k0 + (c & 1) + 8 * (c >> 1);
+        const long long a = bad ? 0 : fix_value(x[c], emax, 5);
+        const long long b = bad ? 0 : fix_value(y[c], emax, 5);
+        E[c] = a + b;
+        O[c] = 2 * j == Q - 1 ? 0 : a - b;
+    }
+    const int q = emax - 1077;
+    const bool folded = DF && Q <= 16;
+    double* A = s.A + (size_t)d * Q * Z;
+    for (int par = p0; par < p1; ++par) {
+        Fix4 v;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v.v[c] = par == 0 ? E[c] : O[c];
+        if (folded) v.v[2] = O[0], v.v[3] = O[1];
+        const Fix4 o = fix_transform(s.Ma + par * kTsSlices * 32, v);
+        // element c: row lane / 4 (+ 8), node t0 + 2 (lane % 4) (+ 1), whose
+        // exponent the lanes of that node hold
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int col = k0 + (c & 1), src = col * 4;
+            const int qc = __shfl_sync(0xffffffffu, q, src), fl = __shfl_sync(0xffffffffu, (int)bad, src);
+            const int l = folded ? 2 * (lane / 4) + (c >> 1) : 2 * (lane / 4 + 8 * (c >> 1)) + par;
+            if (l <= Q - 2 && t0 + col < nz) A[l * Z + t0 + col] = fix_out(o.v[c], qc, fl != 0);
+        }
+    }
+}
+
+// Task g of the synthesis: the sum of S_kl c_l over the orders of parity g % 2
+// for k < H, distribution (g / 2) % 2, nodes 8 (g / 4) .. + 7, as integers of the
+// unit 2^(qn - 1078 + rk_k), qn the exponent of the node's largest coefficient
+// (of both parities, so that the two sums share a unit; kTsBad marks a
+// non-finite one); E + O is the synthesis at k, E - O at Q-1-k.
+constexpr int kTsBad = 1 << 20;
+template <bool DF>
+__device__ __forceinline__ void synthesis_task(const SlabDesc& sd, const WorkItem& it, const Smem<double>& s, int Z,
+                                               long long* part, int* qn, int g) {
+    const int Q = sd.Q, H = (Q + 1) / 2, nz = it.nz, lane = threadIdx.x & 31;
+    const bool folded = DF && Q <= 16;
+    const int par = folded ? 0 : g & 1;
+    if (!folded) g >>= 1;
+    const int d = g & 1, t0 = (g >> 1) * 8, t = min(t0 + lane / 4, nz - 1), k0 = 2 * (lane % 4);
+    const int* gl = s.Ti + 32;
+    const double* c0 = s.C + (size_t)d * Q * Z + t;
+    FixIn x[4];
+    int emax = -100000;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const int m = k0 + (c & 1);
+        const int l = folded ? 2 * m + (c >> 1) : 2 * (m + 8 * (c >> 1)) + par, lo = folded ? l : l ^ 1;
+        x[c] = fix_in(l < Q ? c0[l * Z] : 0.0, l < Q ? gl[l] : 0);
+        emax = max(emax, max(x[c].e, fix_in(lo < Q ? c0[lo * Z] : 0.0, lo < Q ? gl[lo] : 0).e));
+    }
+    emax = quad_max(emax);
+    const bool bad = emax > 50000;
+    Fix4 v;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v.v[c] = bad ? 0 : fix_value(x[c], emax, 6);
+    const Fix4 r = fix_transform(s.Ms + par * kTsSlices * 32, v);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const int tt = t0 + k0 + (c & 1), k = folded ? lane / 4 : lane / 4 + 8 * (c >> 1);
+        const int po = folded ? c >> 1 : par;
+        // (the odd part of an odd Q's middle velocity is zero)
+        if (k < (po ? Q - H : H) && tt < nz) part[((size_t)d * Q + po * H + k) * Z + tt] = r.v[c];
+    }
+    if (par == 0 && (lane & 3) == 0 && t0 + lane / 4 < nz) qn[d * Z + t] = bad ? kTsBad : emax;
+}
+__host__ __device__ inline int transform_tasks(int nz) { return 2 * ((nz + 7) / 8); }
 
 // Parity-split analysis: a_l = sum_{j<H} psi_l(xi_j) (E_j or O_j), l <= Q-2,
 // two orders of one parity (l, l+2) per thread sharing each E/O value loaded
@@ -1016,40 +1228,6 @@ __device__ void analysis_eo(const SlabDesc& sd, const WorkItem& it, const Smem<R
     if (next) warp_pool(next, 2 * G * nz, task);
     else
         for (int e = tid; e < 2 * G * nz; e += nth) task(e);
-}
-
-// Analysis in double-float: the state tile is split into pairs when it is
-// staged (Fd[(d Q + j) Z + t]); a_l = sum_j psi_l(xi_j) h_j by Dot2, four
-// orders per thread (four independent accumulator chains, each pair loaded
-// feeding four terms), joined to FP64 for the coefficients.
-__device__ inline void analysis_df(const SlabDesc& sd, const WorkItem& it, const Smem<double>& s, const float2* Fd,
-                                   const float2* P, int Z, int* next) {
-    const int Q = sd.Q, nz = it.nz;
-    const int nq = Q / 4;                          // quads of orders covering l <= Q-2 (Q even)
-    const int per_d = nq * nz;
-    warp_pool(next, 2 * per_d, [&](int e) {
-        int d = e / per_d, r = e % per_d;
-        int l0 = 4 * (r / nz), t = r % nz;
-        const int nl = min(4, Q - 1 - l0);         // orders l0 .. l0+nl-1 (<= Q-2)
-        const float2* P0 = P + l0 * Q;
-        const float2* P1 = P + min(l0 + 1, Q - 1) * Q;
-        const float2* P2 = P + min(l0 + 2, Q - 1) * Q;
-        const float2* P3 = P + min(l0 + 3, Q - 1) * Q;
-        const float2* h = Fd + (size_t)d * Q * Z + t;
-        float s0 = 0.f, e0 = 0.f, s1 = 0.f, e1 = 0.f, s2 = 0.f, e2 = 0.f, s3 = 0.f, e3 = 0.f;
-        for (int j = 0; j < Q; ++j) {
-            const float2 hv = h[j * Z];
-            dot2_acc(s0, e0, P0[j], hv);
-            dot2_acc(s1, e1, P1[j], hv);
-            dot2_acc(s2, e2, P2[j], hv);
-            dot2_acc(s3, e3, P3[j], hv);
-        }
-        double* A = s.A + ((size_t)d * Q + l0) * Z + t;
-        A[0] = df_join(s0, e0);
-        if (nl > 1) A[Z] = df_join(s1, e1);
-        if (nl > 2) A[2 * Z] = df_join(s2, e2);
-        if (nl > 3) A[3 * Z] = df_join(s3, e3);
-    });
 }
 
 // WENO-5 (Jiang & Shu) faces in difference form, along a run of faces.
@@ -1129,12 +1307,10 @@ struct Weno5Run {
 // by xi_k = 0 in the flux difference.
 constexpr int kRun = 4;
 template <typename R>
-__device__ void faces(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, int Z,
-                      const R* __restrict__ rtab, int tid, int nth) {
+__device__ void faces(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, int Z, int tid, int nth) {
     const int Q = sd.Q, W = Z + 6, nf = it.nz + 1, rows = 2 * Q;
     const int nruns = (nf + kRun - 1) / kRun;
-    TableLayout L(Q);
-    const R* xi = rtab + sd.tab_off + L.xi;
+    const R* xi = s.Vr;
     const R eps = slab_weno_eps<R>(sd);
     for (int e = tid; e < rows * nruns; e += nth) {
         const int r = e % rows, run = e / rows;
@@ -1306,12 +1482,10 @@ struct Weno5Split {
 
 // faces() of an FP64 state: the same runs and walk, the split form, taken by
 // whole warps from the pool `next`.
-__device__ inline void faces_split(const SlabDesc& sd, const WorkItem& it, const Smem<double>& s, int Z,
-                                   const double* __restrict__ tab, int* next) {
+__device__ inline void faces_split(const SlabDesc& sd, const WorkItem& it, const Smem<double>& s, int Z, int* next) {
     const int Q = sd.Q, W = Z + 6, nf = it.nz + 1, rows = 2 * Q;
     const int nruns = (nf + kRun - 1) / kRun;
-    TableLayout L(Q);
-    const double* xi = tab + sd.tab_off + L.xi;
+    const double* xi = s.Vp;
     warp_pool(next, rows * nruns, [&](int e) {
         const int r = e % rows, run = e / rows;
         const int k = r % Q;
@@ -1322,11 +1496,11 @@ __device__ inline void faces_split(const SlabDesc& sd, const WorkItem& it, const
         double* out = s.Face + (size_t)r * (Z + 1);
         Weno5Split w;
         w.start(hb[0], hb[dir], hb[2 * dir], hb[3 * dir], hb[4 * dir], sd.weno_eps);
-#pragma unroll
-        for (int q = 0; q < kRun; ++q) {
-            if (q >= n) break;
+#pragma unroll 1
+        for (int q = 0;; ++q) {
             out[f0 + dir * q] = w.face(sd.weno_eps);
-            if (q + 1 < n) w.shift(hb[dir * (q + 5)]);
+            if (q + 1 >= n) break;
+            w.shift(hb[dir * (q + 5)]);
         }
     });
 }
@@ -1438,12 +1612,10 @@ struct Weno5RunDF {
 
 // faces() of the FP64_DF kernel: the same runs and walk, the face values in
 // double-float arithmetic on the FP32 pipe, stored as FP64.
-__device__ inline void faces_df(const SlabDesc& sd, const WorkItem& it, const Smem<double>& s, int Z,
-                                const double* __restrict__ tab, int* next) {
+__device__ inline void faces_df(const SlabDesc& sd, const WorkItem& it, const Smem<double>& s, int Z, int* next) {
     const int Q = sd.Q, W = Z + 6, nf = it.nz + 1, rows = 2 * Q;
     const int nruns = (nf + kRun - 1) / kRun;
-    TableLayout L(Q);
-    const double* xi = tab + sd.tab_off + L.xi;
+    const double* xi = s.Vp;
     const dfl eps4 = dfn_const(4.0 * sd.weno_eps);
     warp_pool(next, rows * nruns, [&](int e) {
         const int r = e % rows, run = e / rows;
@@ -1455,11 +1627,11 @@ __device__ inline void faces_df(const SlabDesc& sd, const WorkItem& it, const Sm
         double* out = s.Face + (size_t)r * (Z + 1);
         Weno5RunDF w;
         w.start(hb[0], hb[dir], hb[2 * dir], hb[3 * dir], hb[4 * dir], eps4);
-#pragma unroll
-        for (int q = 0; q < kRun; ++q) {
-            if (q >= n) break;
+#pragma unroll 1
+        for (int q = 0;; ++q) {
             out[f0 + dir * q] = w.face();
-            if (q + 1 < n) w.shift(hb[dir * (q + 5)]);
+            if (q + 1 >= n) break;
+            w.shift(hb[dir * (q + 5)]);
         }
     });
 }
@@ -1613,6 +1785,28 @@ template <typename R>
 __device__ void tile_moment_sums_staged(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, int Z,
                                         const double* xp, const R* xr, double* __restrict__ mom_out, long long NN) {
     const int Q = sd.Q, W = Z + 6, nz = it.nz;
+    if constexpr (std::is_same<R, double>::value) {
+        // small tiles: the four chains of a sum (moment_sum) on four lanes,
+        // joined by shuffles in the same order
+        if (nz <= 8 && blockDim.x >= 32 * kNumMoments) {
+            const int which = threadIdx.x >> 5, t = (threadIdx.x & 31) >> 2, c = threadIdx.x & 3;
+            if (which < kNumMoments) {
+                const int d = which >= MOM_G0 ? 1 : 0, p = (which >= MOM_G0) ? which - MOM_G0 : which;
+                const double* h = s.F + (size_t)d * Q * W + min(t, nz - 1) + 3;
+                const double* w = xp + (p > 0 ? p - 1 : 0) * Q;
+                double a = 0.0;
+                auto acc = [&](int k) { a = p == 0 ? a + h[k * W] : fma(w[k], h[k * W], a); };
+                const int Q4 = Q & ~3;
+                for (int k = c; k < Q4; k += 4) acc(k);
+                if (c == 0)
+                    for (int k = Q4; k < Q; ++k) acc(k);
+                a += __shfl_xor_sync(0xffffffffu, a, 1);
+                a += __shfl_xor_sync(0xffffffffu, a, 2);
+                if (c == 0 && t < nz) mom_out[which * NN + sd.node_off + it.i0 + t] = a;
+            }
+            return;
+        }
+    }
     if (nz <= 32 && blockDim.x >= 32 * kNumMoments) {
         const int which = threadIdx.x >> 5, t = threadIdx.x & 31;
         if (which < kNumMoments && t < nz) {

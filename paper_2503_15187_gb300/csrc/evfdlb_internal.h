@@ -60,9 +60,39 @@ struct ParitySplit {
     EVF_HD int synthesis_len() const { return H * QE; }             // Sp
 };
 
+// The FP64 transforms on the tensor cores: an entry or a state value, scaled by
+// a power of two, is a fixed-point number of kTsSlices signed digits of
+// kTsBits bits; a digit is an exact FP16 value, and the products of two digits
+// summed over up to 16 terms (and up to four digit pairs of the same weight)
+// are integers below 2^24, exact in the FP32 accumulators of mma.m16n8k16.  The
+// digit pairs of weight s = i + k < kTsSlices are kept (weights 4 and 5, five and
+// six pairs, could only ever be off by a unit below the result's last place).
+//   analysis   a_l = sum_{j<H} psi_l(xi_j) (E_j or O_j): entries psi_l(xi_j) 2^sx_j,
+//              values h_j 2^-sx_j, 2^sx_j about sqrt(w_j) (then the entries are an
+//              orthogonal matrix's, and the values of one magnitude);
+//   synthesis  E_k, O_k = sum over even, odd l of S_kl c_l: entries
+//              S_kl 2^(-gl_l - rk_k), values c_l 2^gl_l, the result times 2^rk_k; 2^gl_l
+//              follows the decay of a Maxwellian's coefficients, so that the
+//              entries of the outer velocities, which act on high orders,
+//              use the digits too.
+// Layout per transform and parity: [slice][lane][4] 32-bit registers of the
+// matrix fragment, rows = orders of the parity (analysis) or k < H, columns =
+// j < H or orders of the parity, zero-padded to 16 x 16; Q <= 16: the two
+// parities' 8 x 8 blocks on the diagonal of one.
+constexpr int kTsSlices = 6, kTsBits = 10;
+constexpr int kTsDoubles = 2 * kTsSlices * 32 * 4 / 2;   // one transform, both parities
+// Orders of an FP64 slab from which they run there (by Q alone, so that a slab's
+// results depend neither on its tile nor on the slabs beside it): up to 16 the
+// sums have at most eight terms and half of each 16 x 16 block would be zeros
+// (stage of 2000 x 16: 15.3 us plain, 17.0 on the tensor cores, even with both
+// parities in one block; 1024 x 24: 14.9 / 15.1; 3001 x 24: 27.9 / 26.4; 32768 x 18:
+// 172 / 146; 4096 x 32: 44.6 / 33.8).
+constexpr int kTsMinQ = 17;
+constexpr int kTsInts = 64;                              // sx [16], rk [16], gl [32]
+
 // Offsets inside the table block of one velocity order Q (doubles).
 struct TableLayout {
-    int xi, w, P, S, rinv, rr, r1, r2, r3, Pp, Sp, total;
+    int xi, w, P, S, rinv, rr, r1, r2, r3, Pp, Sp, Ma, Ms, Mi, total;
     EVF_HD explicit TableLayout(int Q) {
         const ParitySplit ps(Q);
         xi = 0;
@@ -81,7 +111,13 @@ struct TableLayout {
         // parity-split synthesis rows Sp[k][l] = S[k][l], k < H, rows padded to
         // an even length QE with zeros (orders l, l+1 in one two-wide load)
         Sp = Pp + ps.analysis_len();
-        total = Sp + ps.synthesis_len();
+        // digit slices of the transforms for the tensor cores (see kTsSlices), 16-byte
+        // aligned in a block that starts aligned: analysis, synthesis, and the
+        // exponents as kTsInts integers
+        Ma = (Sp + ps.synthesis_len() + 1) & ~1;
+        Ms = Ma + kTsDoubles;
+        Mi = Ms + kTsDoubles;
+        total = Mi + kTsInts / 2;
     }
 };
 

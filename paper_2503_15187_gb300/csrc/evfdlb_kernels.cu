@@ -50,11 +50,8 @@ namespace evfdlb {
 // ---------------------------------------------------------------------------
 
 // mode 0: out = alpha base + beta (src + dt R);  mode 1: rhs_out = R (FP64).
-// DF (R = double only): the FP64_DF variant -- rtab holds the analysis and
-// synthesis tables as double-float pairs, every other table value comes from
-// the FP64 `tables`; the Hermite analysis and synthesis run as Dot2 sums of
-// pairs on the FP32 pipe (state tile split into pairs once per stage in a
-// block after the Hermite moments), everything else as in the FP64 kernel.
+// DF (R = double only): the FP64_DF variant -- WENO-5 faces wholly in double-float
+// and the Hermite transforms on the tensor cores at every Q, else the FP64 kernel.
 //
 // The body runs one work item (slab tile) with the CTA's threads; CG: the
 // stage input, base and moment sums are read with L2-coherent loads (the
@@ -73,54 +70,52 @@ __device__ __forceinline__ void stage_body(const SlabDesc& sd, const WorkItem& i
     Smem<R> s = carve<R>(smem, Q, Z, sd.M);
     double* const fo = FO ? fields_out : nullptr;
 
-    // FP64 / FP32: parity-split tables and state tile (half the transform
-    // products); FP64_DF: the full tables as float pairs and the state tile
-    // split into float pairs in the EO block.
     // The inputs that no stage writes come first (velocity tables, force and
     // Fischer-Methfessel taps, velocity powers): in a programmatic launch
     // they are staged while the previous stage still runs, and
     // griddepcontrol.wait then holds back the reads of its state and moment
     // sums until that stage has completed (a no-op in a plain launch).
-    float2* Fd = DF ? reinterpret_cast<float2*>(s.EO) : nullptr;
-    load_velocity_tables<R, !DF>(sd, s, rtab);
+    constexpr bool F64 = std::is_same<R, double>::value;
+    stage_tables<R, DF>(sd, s, Z, smem, rtab);
+    const bool ts = on_tensor_cores<R, DF>(Q);
     for (int j = threadIdx.x; j < 2 * sd.M + 1; j += blockDim.x) s.Ftap[j] = rtaps[sd.tap_off + j];
     for (int j = threadIdx.x; j < 2 * sd.m + 1; j += blockDim.x) s.Mtap[j] = taps[sd.tap_off + 2 * sd.M + 1 + j];
     // velocity powers of the closing moment sums, formed once per CTA
     {
-        const R* vt = DF ? reinterpret_cast<const R*>(tables) : rtab;
         const int xo = sd.tab_off + TableLayout(Q).xi;
-        velocity_powers<R>(Q, tables + xo, vt + xo, s.Vp, s.Vr, threadIdx.x, blockDim.x);
+        velocity_powers<R>(Q, tables + xo, rtab + xo, s.Vp, s.Vr, threadIdx.x, blockDim.x);
     }
     if constexpr (!CG) asm volatile("griddepcontrol.wait;" ::: "memory");
     // the state tile by asynchronous copies, issued first, so that they are
     // in flight with the node inputs' loads and arithmetic
-    if constexpr (!DF) issue_state_tile<R, CG>(sd, it, s, Z, src, NF);
-    constexpr bool F64 = std::is_same<R, double>::value;
-    __shared__ int s_next[2];                    // pools of face runs and of analysis tasks
+    issue_state_tile<R, CG>(sd, it, s, Z, src, NF);
+    // pools of face runs and of analysis tasks (in a place the FP64 roles leave free)
+    int* s_next = reinterpret_cast<int*>(s.Sc + (SC_FORCE + 1) * Z - 1);
     if constexpr (F64) {
         if (threadIdx.x < 2) s_next[threadIdx.x] = 0;
         load_raw_sums<CG>(sd, it, s, Z, mom_in, NN);
     } else {
-        load_node_inputs<R, !DF, CG, false>(sd, it, s, Z, rtab, mom_in, NN);
+        load_node_inputs<R, CG>(sd, it, s, Z, mom_in, NN);
     }
-    if constexpr (DF) load_state_tile<R>(sd, it, s, Z, src, NF, Fd);
-    if constexpr (!DF && !CG) cp_async_wait_all();
+    if constexpr (!CG) cp_async_wait_all();
     __syncthreads();
-    // the tables of everything but the DF transforms
-    const R* vtab = DF ? reinterpret_cast<const R*>(tables) : rtab;
-    const R* rt = vtab + sd.tab_off;
-    TableLayout L(Q);
     if constexpr (F64) {
-        // Warps 0-3 form the node quantities, the others split the state tile
-        // into parity parts; then every warp takes runs of WENO-5 faces, and
-        // groups of the Hermite analysis, as it arrives.
+        // Warps 0-3 form the node quantities; every warp takes runs of WENO-5 faces
+        // and the Hermite analysis from pools as it arrives.  With the transforms on
+        // the tensor cores the analysis (tasks of eight nodes, a parity each on
+        // small tiles) comes first: it keeps off the FP64 pipe, which the node work
+        // needs alone (a chain of FP64 instructions slows down with every other warp
+        // that issues them) -- but where the other warps hold all runs of faces in one
+        // round, these, the longer tasks, come first (1024 x 24: 16.6 -> 15.2 us).  On the
+        // plain path (see kTsMinQ) the warps from 4 on first split the state tile
+        // into parity parts, and the faces come before the analysis.
         if (threadIdx.x < 128) {
-            node_roles<FO>(sd, it, s, Z, rt, NN, err, fo);
+            node_roles<FO>(sd, it, s, Z, NN, err, fo);
             // the parity parts are there (barrier 8 + warp: this warp and the
             // arrivals of the splitting warps)
-            if constexpr (!DF)
+            if (!ts)
                 asm volatile("bar.sync %0, %1;" ::"r"(8 + (int)(threadIdx.x >> 5)), "r"((int)blockDim.x - 96) : "memory");
-        } else if constexpr (!DF) {
+        } else if (!ts) {
             const int nth = blockDim.x - 128;
             split_state_tile<R>(sd, it, s, Z, threadIdx.x - 128, nth);
             __threadfence_block();
@@ -128,13 +123,29 @@ __device__ __forceinline__ void stage_body(const SlabDesc& sd, const WorkItem& i
             for (int w = 0; w < 4; ++w) asm volatile("bar.arrive %0, %1;" ::"r"(8 + w), "r"(nth + 32) : "memory");
             asm volatile("bar.sync 2, %0;" ::"r"(nth) : "memory");
         }
-        if constexpr (DF) {
-            faces_df(sd, it, s, Z, tables, s_next);
-            analysis_df(sd, it, s, Fd, reinterpret_cast<const float2*>(s.P), Z, s_next + 1);
-        } else {
-            faces_split(sd, it, s, Z, vtab, s_next);
-            analysis_eo<R>(sd, it, s, Z, 0, 0, s_next + 1);
+        auto all_faces = [&] {
+            if constexpr (DF) faces_df(sd, it, s, Z, s_next);
+            else faces_split(sd, it, s, Z, s_next);
+        };
+        const int face_warps = (2 * Q * ((nz + kRun) / kRun) + 31) / 32;
+        const bool faces_first = !ts || face_warps <= (int)(blockDim.x >> 5) - 4;
+        for (int phase = 0; phase < 2; ++phase) {
+            if ((phase == 0) == faces_first) {
+                all_faces();
+            } else if (ts) {
+                const int parities = Q <= 16 ? 1 : 2, halves = transform_tasks(nz) < 8 ? parities : 1;
+                for (;;) {
+                    int g = 0;
+                    if ((threadIdx.x & 31) == 0) g = atomicAdd(s_next + 1, 1);
+                    g = __shfl_sync(0xffffffffu, g, 0);
+                    if (g >= halves * transform_tasks(nz)) break;
+                    if (halves == 2) analysis_task<DF>(sd, it, s, Z, g >> 1, g & 1, (g & 1) + 1);
+                    else analysis_task<DF>(sd, it, s, Z, g, 0, parities);
+                }
+            }
         }
+        if constexpr (!DF)
+            if (!ts) analysis_eo<R>(sd, it, s, Z, 0, 0, s_next + 1);
     } else {
         // The node warps form the node-level quantities of the tile (node
         // fields, coefficient constants) while the other warps do the
@@ -165,7 +176,7 @@ __device__ __forceinline__ void stage_body(const SlabDesc& sd, const WorkItem& i
             // warp, whose share of the force sums (a half-warp per node from
             // the first worker) is empty on tiles of up to nth/16 - 2 nodes,
             // forms them first, beside the other workers' force sums
-            if (tid >= nth - 32) node_hermite_moments<R>(sd, it, s, Z, rt, tid - (nth - 32), 32);
+            if (tid >= nth - 32) node_hermite_moments<R>(sd, it, s, Z, tid - (nth - 32), 32);
             tile_force_sums<R>(sd, it, s, Z, s.Ftap, tid, nth);
             __threadfence_block();
             asm volatile("bar.arrive 3, %0;" ::"r"((int)blockDim.x) : "memory");
@@ -174,18 +185,20 @@ __device__ __forceinline__ void stage_body(const SlabDesc& sd, const WorkItem& i
             split_state_tile<R>(sd, it, s, Z, tid, nth);
             asm volatile("bar.sync 2, %0;" ::"r"(nth) : "memory");
             analysis_eo<R>(sd, it, s, Z, tid, nth);
-            faces<R>(sd, it, s, Z, vtab, tid, nth);
+            faces<R>(sd, it, s, Z, tid, nth);
         }
     }
     __syncthreads();
-    coefficients<R, DF>(sd, it, s, Z, rt, threadIdx.x, blockDim.x);
+    coefficients<R>(sd, it, s, Z, threadIdx.x, blockDim.x);
     __syncthreads();
     // the next stage (a programmatic launch) may now be scheduled beside
     // this CTA and stage its constant inputs
     if constexpr (!CG) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     // Phase 5: synthesis, advection, relaxation and the RK stage.
-    const R* xi = rt + L.xi;
+    const R* xi;                                 // the velocities, staged
+    if constexpr (F64) xi = s.Vp;
+    else xi = s.Vr;
     const R dt = slab_dt<R>(sd), inv_dx = slab_inv_dx<R>(sd), ralpha = alpha, rbeta = beta;
     const bool rhs_form = (mode == 1), with_base = nonzero(alpha);
     // The stage out = alpha base + beta (h + dt R) with
@@ -202,7 +215,7 @@ __device__ __forceinline__ void stage_body(const SlabDesc& sd, const WorkItem& i
     // The FP32 state's moment sums take their pair terms from the values
     // written here (PT); the other forms sum the new tile after the
     // synthesis, so emit stores it back into s.F.
-    constexpr bool PT = std::is_same<R, float>::value && !DF;
+    constexpr bool PT = std::is_same<R, float>::value;
     auto emit = [&](int d, int t, int k, R syn, R ch, R cx, R bv) -> R {
         R* hp = s.F + (size_t)(d * Q + k) * W + t + 3;
         const R h = *hp;
@@ -221,32 +234,52 @@ __device__ __forceinline__ void stage_body(const SlabDesc& sd, const WorkItem& i
         if constexpr (!PT) *hp = o;
         return o;
     };
-    if constexpr (DF) {
-        // four velocities per thread (four independent Dot2 chains hide the
-        // FP32 latency)
-        constexpr int VK = 4;
-        const int nkg = (Q + VK - 1) / VK;
-        for (int e = threadIdx.x; e < 2 * nkg * nz; e += blockDim.x) {
-            int t = e % nz, r = e / nz;
-            int k0 = VK * (r % nkg), d = r / nkg;
-            const int nk = min(VK, Q - k0);
-            const float2* Sd = reinterpret_cast<const float2*>(s.S);
-            const float2* c = reinterpret_cast<const float2*>(s.C) + (size_t)d * Q * Z + t;
-            float a[VK], b[VK];
-#pragma unroll
-            for (int q = 0; q < VK; ++q) a[q] = b[q] = 0.f;
-            for (int l = 0; l < Q; ++l) {
-                const float2 cl = c[l * Z];
-#pragma unroll
-                for (int q = 0; q < VK; ++q) dot2_acc(a[q], b[q], Sd[min(k0 + q, Q - 1) * Q + l], cl);
-            }
-            const R ch = fma(-cs, s.Scr[t], rbeta);
-#pragma unroll
-            for (int q = 0; q < VK; ++q)
-                if (q < nk)
-                    emit(d, t, k0 + q, df_join(a[q], b[q]), ch, csx * xi[k0 + q],
-                         (with_base && !rhs_form) ? gload<CG>(base + gidx_of(d, t, k0 + q)) : R(0));
+    if (ts) {
+      if constexpr (F64) {
+        // the transform's tasks by whole warps, to the (now free) analysis
+        // block; the per-node and per-velocity factors of the stage beside it
+        const int nwarps = blockDim.x >> 5, nth = blockDim.x;
+        long long* part = reinterpret_cast<long long*>(s.A);
+        double* chn = s.Sc + SC_U * Z;           // ch per node
+        double* cxk = s.Mm;                      // cx per velocity
+        int* qn = reinterpret_cast<int*>(s.Cc);  // exponents of the synthesis [2][Z]
+        for (int e = threadIdx.x; e < nz + (Q + 1) / 2; e += nth) {
+            if (e < nz) chn[e] = fma(-cs, s.Scr[e], rbeta);
+            else cxk[e - nz] = csx * xi[e - nz];
         }
+        for (int g = threadIdx.x >> 5; g < (Q <= 16 ? 1 : 2) * transform_tasks(nz); g += nwarps)
+            synthesis_task<DF>(sd, it, s, Z, part, qn, g);
+        __syncthreads();
+        const bool lb = with_base && !rhs_form;
+        // one velocity pair (k, Q-1-k) of a node per item: two independent
+        // chains a thread; the next item's base values in flight
+        const int H = (Q + 1) / 2, dr = nth / nz, dtt = nth - dr * nz;     // (row, node) step of a thread
+        int r = threadIdx.x / nz, t = threadIdx.x - r * nz;
+        double b0 = 0, b1 = 0;
+        auto load_base = [&] {
+            if (!lb || r >= 2 * H) return;
+            const int d = r >= H ? 1 : 0, k = r - d * H;
+            b0 = gload<CG>(base + gidx_of(d, t, k));
+            b1 = gload<CG>(base + gidx_of(d, t, Q - 1 - k));
+        };
+        load_base();
+        while (r < 2 * H) {
+            const int d = r >= H ? 1 : 0, k = r - d * H, tt = t;
+            const double a0 = b0, a1 = b1;
+            r += dr, t += dtt;
+            if (t >= nz) t -= nz, ++r;
+            load_base();
+            const bool pair = Q - 1 - k != k;
+            const long long* p = part + ((size_t)d * Q + k) * Z + tt;
+            const long long E = p[0], O = pair ? p[(size_t)H * Z] : 0;
+            const int qe = qn[d * Z + tt];
+            const int q = qe - 1078 + s.Ti[16 + k];
+            const double ch = chn[tt], cx = cxk[k];
+            const double v0 = fix_out(E + O, q, qe == kTsBad), v1 = fix_out(E - O, q, qe == kTsBad);
+            emit(d, tt, k, v0, ch, cx, a0);
+            if (pair) emit(d, tt, Q - 1 - k, v1, ch, -cx, a1);
+        }
+      }
     } else if constexpr (PT) {
         // FP32, parity split: the velocity pairs (k, Q-1-k) of group g
         // (k = 2g, 2g+1) for one node per task, so that each coefficient
@@ -296,7 +329,7 @@ __device__ __forceinline__ void stage_body(const SlabDesc& sd, const WorkItem& i
             }
             if (!rhs_form) pair_terms_f32(d, g, two, t, Q, Z, a0, m0, a1, m1, s.Vp, s.Vr, s.Mp64, s.Mp32);
         }
-    } else {
+    } else if constexpr (!DF) {
         // parity split: one velocity pair (k, Q-1-k) per task; even orders
         // build E, odd orders O (one two-wide table load per two orders); the
         // synthesis is E + O at k and E - O at Q-1-k
@@ -648,7 +681,7 @@ fields_kernel(const SlabDesc* __restrict__ slabs, const WorkItem* __restrict__ i
     const WorkItem it = items[blockIdx.x];
     const SlabDesc sd = slabs[it.slab];
     Smem<R> s = carve<R>(smem, sd.Q, Z, sd.M);
-    load_node_inputs<R>(sd, it, s, Z, rtab, mom, NN);
+    load_node_inputs<R>(sd, it, s, Z, mom, NN);
     __syncthreads();
     node_fields<R>(sd, it, s, Z, taps, rtaps, mom, NN, err, fields);
 }
@@ -766,15 +799,29 @@ __global__ void convert_kernel(const A* __restrict__ in, B* __restrict__ out, lo
 // instantiation: EVFDLB_FP64 (R = double) or EVFDLB_FP32 (R = float); the R
 // tables and taps are the FP64 ones for FP64 and float copies for FP32.
 // ---------------------------------------------------------------------------
-size_t stage_smem_bytes(int Q, int Z, int M) { return smem_bytes_t<double>(Q, Z, M); }
+// Dynamic shared memory of the stage: with its tables where a CTA can hold them
+// (see stage_full_bytes).
+constexpr size_t kStageSmemLimit = 227 * 1024 - 64;   // less the kernels' static variables
+template <typename R, bool DF>
+static size_t stage_bytes(int Q, int Z, int M) {
+    const size_t full = stage_full_bytes<R, DF>(Q, Z, M);
+    return full <= kStageSmemLimit ? full : smem_bytes_t<R>(Q, Z, M);
+}
+size_t stage_smem_bytes(int Q, int Z, int M) { return stage_bytes<double, false>(Q, Z, M); }
 
 size_t stage_smem_bytes_p(int prec, int Q, int Z, int M) {
-    return prec == EVFDLB_FP32 ? smem_bytes_t<float>(Q, Z, M) : smem_bytes_t<double>(Q, Z, M);
+    if (prec == EVFDLB_FP64_DF) return stage_bytes<double, true>(Q, Z, M);
+    return prec == EVFDLB_FP32 ? stage_bytes<float, false>(Q, Z, M) : stage_bytes<double, false>(Q, Z, M);
 }
-
-// The FP64_DF stage keeps its split state tile (2 Q Z float pairs) in the EO
-// block (4 H Z >= 2 Q Z doubles).
-size_t stage_smem_bytes_df(int Q, int Z, int M) { return smem_bytes_t<double>(Q, Z, M); }
+// What covers every tile of up to kZMax nodes: the smaller ones may hold their
+// tables where the largest does not.
+size_t stage_smem_cap_p(int prec, int Q, int M) {
+    const size_t most = stage_smem_bytes_p(prec, Q, kZMax, M);
+    const size_t full = prec == EVFDLB_FP64_DF ? stage_full_bytes<double, true>(Q, kZMax, M)
+                        : prec == EVFDLB_FP32  ? stage_full_bytes<float, false>(Q, kZMax, M)
+                                               : stage_full_bytes<double, false>(Q, kZMax, M);
+    return full <= kStageSmemLimit ? full : std::max(most, kStageSmemLimit);
+}
 
 cudaError_t configure_df(size_t smem_bytes) {
     cudaError_t e = cudaFuncSetAttribute(stage_kernel<double, true, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -798,17 +845,18 @@ static int sm_count() {
     return cache[dev];
 }
 
-// FP64_DF stage: dftab holds the analysis and synthesis tables as pairs.
+// FP64_DF stage (the FP64 stage with its faces in double-float).
 void launch_stage_df(int nitems, size_t smem, cudaStream_t st, const SlabDesc* slabs, const WorkItem* items,
-                     const double* tables, const double* dftab, const double* taps, const double* src,
-                     const double* base, double* out, double* rhs_out, const double* mom_in, double* mom_out,
-                     long long NF, long long NN, double alpha, double beta, int mode, int Z, unsigned* err) {
+                     const double* tables, const double* taps, const double* src, const double* base, double* out,
+                     double* rhs_out, const double* mom_in, double* mom_out, long long NF, long long NN, double alpha,
+                     double beta, int mode, int Z, unsigned* err) {
     // 16 warps (one CTA per SM) where the work list fits one wave on the SMs,
     // else 8 (up to three CTAs): the double-float runs of one CTA's 8 warps
     // leave their pipe idle on latency (4096 x 32, 152 tiles: 40.9 -> 34.7 us a
-    // stage; 3001 x 24: 34.1 -> 22.8 us; two tiles per SM: 44.9 -> 47.7)
+    // stage; 3001 x 24: 34.1 -> 22.8 us; two tiles per SM: 44.9 -> 47.7; these with the
+    // transforms still in double-float, 4096 x 32 now 27.4 us)
     auto kernel = nitems <= sm_count() ? stage_kernel<double, true, 512> : stage_kernel<double, true, 256>;
-    launch_pdl(kernel, nitems, nitems <= sm_count() ? 512 : 256, smem, st, slabs, items, tables, dftab, taps, taps, src,
+    launch_pdl(kernel, nitems, nitems <= sm_count() ? 512 : 256, smem, st, slabs, items, tables, tables, taps, taps, src,
                base, out, rhs_out, mom_in, mom_out, NF, NN, alpha, beta, mode, Z, err);
 }
 

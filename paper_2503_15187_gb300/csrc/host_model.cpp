@@ -6,6 +6,9 @@
 // Paper: Busuioc & Sofonea, arXiv:2503.15187.  Equations cited by label.
 #include <math.h>
 
+#include <stdint.h>
+#include <string.h>
+
 #include <algorithm>
 #include <vector>
 
@@ -94,6 +97,40 @@ bool velocity_set(int Q, double* xi, double* w) {
     return true;
 }
 
+namespace {
+// FP16 bits of an integer |v| <= 1024 (exact)
+uint16_t half_of_int(int v) {
+    if (v == 0) return 0;
+    const uint16_t sign = v < 0 ? 0x8000 : 0;
+    unsigned a = (unsigned)(v < 0 ? -v : v);
+    int e = 0;
+    while ((a >> e) > 1) ++e;
+    return (uint16_t)(sign | ((e + 15) << 10) | ((a << (10 - e)) & 0x3ff));
+}
+
+// The digit slices of a 16 x 16 block T, |T| <= 1 (see kTsSlices), in the
+// fragment order of mma.m16n8k16's row-major A operand.
+void slice_block(const long double (*T)[16], uint32_t* out) {
+    static_assert(kTsBits == 10, "digit extraction");
+    for (int lane = 0; lane < 32; ++lane)
+        for (int reg = 0; reg < 4; ++reg) {
+            const int row = lane / 4 + 8 * (reg & 1), col = (lane % 4) * 2 + 8 * (reg >> 1);
+            int64_t v[2];
+            for (int c = 0; c < 2; ++c)
+                v[c] = T[row][col + c] == 0 ? 0 : llroundl(ldexpl(T[row][col + c], kTsBits * kTsSlices - 1));
+            for (int i = kTsSlices - 1; i >= 0; --i) {           // digits in [-512, 511], the first in [-512, 512]
+                uint32_t word = 0;
+                for (int c = 0; c < 2; ++c) {
+                    int64_t d = i ? ((v[c] + 512) & 1023) - 512 : v[c];
+                    v[c] = (v[c] - d) / 1024;
+                    word |= (uint32_t)half_of_int((int)d) << (16 * c);
+                }
+                out[(i * 32 + lane) * 4 + reg] = word;
+            }
+        }
+}
+}  // namespace
+
 // Fixed-size storage (no heap), like velocity_set.
 void build_tables(int Q, const double* xi, const double* w, double* out) {
     TableLayout L(Q);
@@ -119,6 +156,45 @@ void build_tables(int Q, const double* xi, const double* w, double* out) {
     }
     for (int k = 0; k < ps.H; ++k)
         for (int l = 0; l < ps.QE; ++l) out[L.Sp + k * ps.QE + l] = (l < Q) ? out[L.S + k * Q + l] : 0.0;
+    // digit slices of the tensor-core transforms (see kTsSlices)
+    if (L.Ma > L.Sp + ps.synthesis_len()) out[L.Ma - 1] = 0.0;
+    int32_t ints[kTsInts] = {0};
+    int32_t *sx = ints, *rk = ints + 16, *gl = ints + 32;
+    for (int l = 0; l < Q && l < 32; ++l) gl[l] = (int)(0.45 * l);
+    long double T[16][16];
+    const int H = ps.H < 16 ? ps.H : 16;
+    long double all[16][33];
+    for (int j = 0; j < H; ++j) {
+        psi_all<long double>(Q, (long double)xi[j], r, all[j]);
+        sx[j] = (int)lround(0.5 * log2(w[j])) - 1;               // |psi_l(xi_j)| 2^sx <= 2^-0.5
+        double most = 0;
+        for (int l = 0; l < Q; ++l) most = std::max(most, fabs(ldexp(w[j] * (double)all[j][l], -gl[l])));
+        rk[j] = ilogb(most) + 2;                                 // entries below 1 (after every rounding)
+    }
+    const bool folded = Q <= 16;                                 // both parities in one block
+    for (int transform = 0; transform < 2; ++transform)
+        for (int par = 0; par < 2; ++par) {
+            if (par == 0 || !folded)
+                for (int a = 0; a < 16; ++a)
+                    for (int b = 0; b < 16; ++b) T[a][b] = 0;
+            const int at = folded ? 8 * par : 0;
+            for (int j = 0; j < H; ++j)
+                for (int m = 0; 2 * m + par < Q; ++m) {
+                    const int l = 2 * m + par;
+                    if (transform == 0) {
+                        if (l <= Q - 2) T[at + m][at + j] = ldexpl(all[j][l], sx[j]);
+                    } else {
+                        T[at + j][at + m] = ldexpl((long double)w[j] * all[j][l], -gl[l] - rk[j]);
+                    }
+                }
+            if (folded && par == 0) continue;
+            uint32_t slices[kTsSlices * 32 * 4];
+            slice_block(T, slices);
+            char* at_block = (char*)(out + (transform ? L.Ms : L.Ma));
+            memcpy(at_block + (folded ? 0 : par) * sizeof(slices), slices, sizeof(slices));
+            if (folded) memset(at_block + sizeof(slices), 0, sizeof(slices));
+        }
+    memcpy(out + L.Mi, ints, sizeof(ints));
     for (int l = 0; l < Q; ++l) {
         long double ll = l;
         out[L.rinv + l] = (double)(1.0L / sqrtl(ll + 1));
