@@ -268,6 +268,40 @@ void queue_step(evfdlb_ctx* c, cudaStream_t st) {
                            c->NN, c->Z);
 }
 
+// The node tile of a new context: one tile an SM, of up to kZMax nodes, unless
+// smaller tiles fill the SMs better.  That is estimated: a CTA of Z nodes alone on
+// its SM takes about Z + h units (h: its share of work that does not grow with
+// the tile); a second one adds half of that, as one CTA leaves half of the SM to
+// others; the tiles go round in waves of r CTAs an SM, r by registers and shared
+// memory, and the last wave has what is left.  Measured over Q = 8 .. 32, 3001 ..
+// 65536 nodes and seven batches, a stage at the estimate's choice takes, against
+// one tile an SM: FP64 never longer, 12000 x 32 133 -> 89 us, 8192 x 24 54 -> 45,
+// 65536 x 24 393 -> 363, 24 slabs of 200 x 16 42 -> 30; FP32 12000 x 32 48 -> 22,
+// 65536 x 32 167 -> 111 (at most 2 % longer: 256 of 333 x 24).  An FP32 stage of up to
+// 32 nodes an SM waits on latency at any tile, and FP64_DF has a form of its own for
+// one tile an SM (see launch_stage_df): both keep that; more FP64_DF tiles than SMs
+// share them three at a time up to 32 nodes (65536 x 32: 395 -> 319 us; Q = 8, with
+// room for larger ones, 129 against 124 at 64).
+int default_tile(const evfdlb_ctx* c, int sms) {
+    const int one = (int)std::min<long long>(std::max<long long>((c->NN + sms - 1) / sms, 1), kZMax);
+    if (c->df) return c->NN <= (long long)kZMax * sms || c->Qmax <= 8 ? one : 32;
+    if (c->prec == EVFDLB_FP32 && one <= 32) return one;
+    std::map<int, long long> lens;              // interior nodes -> slabs
+    for (const evfdlb_params& q : c->params) ++lens[q.nx - c->halo_lo - c->halo_hi];
+    const double h = c->prec == EVFDLB_FP32 ? 24 : 12;
+    int best = 1;
+    double least = 0;
+    for (int Z = 1; Z <= kZMax; ++Z) {
+        long long tiles = 0;
+        for (const auto& l : lens) tiles += l.second * ((l.first + Z - 1) / Z);
+        const long long r = 228 * 1024 / (stage_smem_bytes_p(c->prec, c->Qmax, Z, c->Mmax) + 1024) >= 2 ? 2 : 1;
+        auto time = [&](long long k) { return k == 0 ? 0.0 : (Z + h) * (k == 1 ? 1.0 : 1.55); };
+        const double t = (double)(tiles / (r * sms)) * time(r) + time((tiles % (r * sms) + sms - 1) / sms);
+        if (Z == 1 || t <= least) best = Z, least = t;
+    }
+    return best;
+}
+
 // Splits every slab into node tiles of Z nodes (the last tile of a slab may
 // be shorter); the device work list is sized for the finest split (Z = 1).
 void partition(evfdlb_ctx* c, int Z) {
@@ -593,9 +627,7 @@ evfdlb_status evfdlb_create(const evfdlb_params* p, int32_t nbatch, const evfdlb
     c->Qmax = Qmax;
     c->Mmax = Mmax;
     c->mmax = mmax;
-    // node tile: one wave of CTAs over the SMs when possible
-    long long z = (NN + sms - 1) / sms;
-    partition(c, (int)std::min<long long>(std::max<long long>(z, 1), kZMax));
+    partition(c, default_tile(c, sms));
 
     cudaError_t e = cudaSuccess;
     auto alloc = [&](void** ptr, size_t bytes) {
