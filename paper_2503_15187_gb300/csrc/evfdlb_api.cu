@@ -21,7 +21,7 @@ void launch_stage_p(int prec, int nitems, size_t smem, cudaStream_t st, const Sl
                     const WorkItem* items, const double* tables, const void* rtab, const double* taps,
                     const void* rtaps, const void* src, const void* base, void* out, double* rhs_out,
                     const double* mom_in, double* mom_out, long long NF, long long NN, double alpha, double beta,
-                    int mode, int Z, unsigned* err);
+                    int mode, int Z, int Q, unsigned* err);
 void launch_stage_fields(int nitems, size_t smem, cudaStream_t st, const SlabDesc* slabs, const WorkItem* items,
                          const double* tables, const double* taps, const double* src, const double* base,
                          double* out, const double* mom_in, double* mom_out, double* fields_out, long long NF,
@@ -222,7 +222,7 @@ void queue_stage(evfdlb_ctx* c, cudaStream_t st, const void* src, const void* ba
                         (const double*)base, (double*)out, nullptr, mi, mo, c->NF, c->NN, a, b, 0, c->Z, c->err);
     else
         launch_stage_p(c->prec, n, c->smem, st, c->slabs, c->items, c->tables, c->rtables, c->taps, c->rtaps, src,
-                       base, out, nullptr, mi, mo, c->NF, c->NN, a, b, 0, c->Z, c->err);
+                       base, out, nullptr, mi, mo, c->NF, c->NN, a, b, 0, c->Z, c->Qmax, c->err);
 }
 
 // Queues nsteps steps of every slab as one persistent launch (after zeroing
@@ -847,7 +847,7 @@ evfdlb_status evfdlb_rhs(evfdlb_ctx* c, double* RF, double* RG, int32_t on_devic
     else
         launch_stage_p(c->prec, (int)c->items_h.size(), c->smem, c->user, c->slabs, c->items, c->tables,
                        c->rtables, c->taps, c->rtaps, c->state[0], nullptr, nullptr, c->scratch, c->mom[0], nullptr,
-                       c->NF, c->NN, 0.0, 1.0, 1, c->Z, c->err);
+                       c->NF, c->NN, 0.0, 1.0, 1, c->Z, c->Qmax, c->err);
     TRY_CUDA(cudaGetLastError());
     size_t bytes = sizeof(double) * c->NF;
     evfdlb_status s;

@@ -23,7 +23,8 @@ constexpr int kThreads = 256;      // threads of the per-tile kernels
 // instruction per scheduler every 64 cycles whatever the number of active
 // lanes, so the FP64 kernels run 8 warps (two per scheduler, of which four form
 // the node quantities first; two CTAs of at most 128 registers per SM when the
-// work list spans several waves); the FP32 variant's per-velocity work is
+// work list spans several waves; 16 for larger tiles that have their SMs to
+// themselves, see launch_stage_fp64); the FP32 variant's per-velocity work is
 // cheap and latency-bound, so it runs 16 (and FP64_DF where a CTA has its SM
 // to itself, see launch_stage_df).
 template <typename R, bool DF = false> struct StageThreads { static constexpr int value = 256; };

@@ -864,11 +864,9 @@ template <typename R>
 static cudaError_t configure_t(size_t smem_bytes) {
     cudaError_t e = cudaFuncSetAttribute(stage_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
     if (e != cudaSuccess) return e;
-    if (std::is_same<R, float>::value) {
-        e = cudaFuncSetAttribute(stage_kernel<float, false, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem_bytes);
-        if (e != cudaSuccess) return e;
-    }
+    e = cudaFuncSetAttribute(stage_kernel<R, false, (StageThreads<R>::value == 512 ? 256 : 512)>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(init_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(iso_reset_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
@@ -889,7 +887,8 @@ cudaError_t configure_kernels(size_t smem_bytes) { return configure_t<double>(sm
 // Raises (never lowers) the dynamic shared-memory limit of the FP64 stage and
 // isothermal-reset kernels on the current device to at least smem_bytes.
 cudaError_t ensure_stage_smem(size_t smem_bytes) {
-    const void* fns[2] = {(const void*)stage_kernel<double>, (const void*)iso_reset_kernel<double>};
+    const void* fns[3] = {(const void*)stage_kernel<double>, (const void*)stage_kernel<double, false, 512>,
+                          (const void*)iso_reset_kernel<double>};
     for (const void* f : fns) {
         cudaFuncAttributes a;
         cudaError_t e = cudaFuncGetAttributes(&a, f);
@@ -901,21 +900,30 @@ cudaError_t ensure_stage_smem(size_t smem_bytes) {
     return cudaSuccess;
 }
 
-// The FP64 stage (8 warps; see StageThreads).
+// The FP64 stage: 8 warps (see StageThreads), or 16 (one CTA an SM) where the work
+// list fits one wave on the SMs, the transforms run on the tensor cores and a
+// tile is more than ten nodes.  Then the faces and the transforms, which wait on
+// latency rather than on the FP64 pipe, have tasks for all of them (4096 x 32, 27
+// nodes a tile: 33.9 -> 32.5 us; 3001 x 24, 20: 26.8 -> 23.6; 2000 x 17, 14: 19.3 ->
+// 18.2).  Smaller tiles have not, and the node roles' chains slow down beside more
+// warps (1200 x 24, 8: 16.3 -> 16.6; 256 x 32, 2: 15.8 -> 16.5); plain sums are bound
+// by the FP64 pipe (4096 x 16: 22.7 -> 23.1; 256 x 16: 11.6 -> 12.5).
 static void launch_stage_fp64(int nitems, size_t smem, cudaStream_t st, const SlabDesc* slabs,
                               const WorkItem* items, const double* tables, const double* rtab, const double* taps,
                               const double* rtaps, const double* src, const double* base, double* out,
                               double* rhs_out, const double* mom_in, double* mom_out, long long NF, long long NN,
-                              double alpha, double beta, int mode, int Z, unsigned* err) {
-    launch_pdl(stage_kernel<double>, nitems, StageThreads<double>::value, smem, st, slabs, items, tables, rtab, taps,
-               rtaps, src, base, out, rhs_out, mom_in, mom_out, NF, NN, alpha, beta, mode, Z, err);
+                              double alpha, double beta, int mode, int Z, int Q, unsigned* err) {
+    const bool wide = nitems <= sm_count() && Q >= kTsMinQ && Z > 10;
+    auto kernel = wide ? stage_kernel<double, false, 512> : stage_kernel<double, false, 256>;
+    launch_pdl(kernel, nitems, wide ? 512 : 256, smem, st, slabs, items, tables, rtab, taps, rtaps, src, base, out,
+               rhs_out, mom_in, mom_out, NF, NN, alpha, beta, mode, Z, err);
 }
 
 void launch_stage_p(int prec, int nitems, size_t smem, cudaStream_t st, const SlabDesc* slabs,
                     const WorkItem* items, const double* tables, const void* rtab, const double* taps,
                     const void* rtaps, const void* src, const void* base, void* out, double* rhs_out,
                     const double* mom_in, double* mom_out, long long NF, long long NN, double alpha, double beta,
-                    int mode, int Z, unsigned* err) {
+                    int mode, int Z, int Q, unsigned* err) {
     if (prec == EVFDLB_FP32) {
         // the 16-warp form (one CTA per SM) where the work list fits one wave
         // on the SMs, else the 8-warp form (two CTAs per SM), which finishes
@@ -931,7 +939,7 @@ void launch_stage_p(int prec, int nitems, size_t smem, cudaStream_t st, const Sl
     } else
         launch_stage_fp64(nitems, smem, st, slabs, items, tables, (const double*)rtab, taps, (const double*)rtaps,
                           (const double*)src, (const double*)base, (double*)out, rhs_out, mom_in, mom_out, NF, NN,
-                          alpha, beta, mode, Z, err);
+                          alpha, beta, mode, Z, Q, err);
 }
 
 // FP64 stage that also stores the node fields of its input state (the
@@ -949,9 +957,9 @@ void launch_stage_fields(int nitems, size_t smem, cudaStream_t st, const SlabDes
 void launch_stage(int nitems, size_t smem, cudaStream_t st, const SlabDesc* slabs, const WorkItem* items,
                   const double* tables, const double* taps, const double* src, const double* base,
                   double* out, const double* mom_in, double* mom_out, long long NF, long long NN,
-                  double alpha, double beta, int mode, int Z, unsigned* err) {
+                  double alpha, double beta, int mode, int Z, int Q, unsigned* err) {
     launch_stage_fp64(nitems, smem, st, slabs, items, tables, tables, taps, taps, src, base, out, out, mom_in, mom_out,
-                      NF, NN, alpha, beta, mode, Z, err);
+                      NF, NN, alpha, beta, mode, Z, Q, err);
 }
 
 void launch_init_p(int prec, int nitems, size_t smem, cudaStream_t st, const SlabDesc* slabs,

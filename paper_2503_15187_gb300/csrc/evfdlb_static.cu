@@ -31,7 +31,7 @@ cudaError_t ensure_stage_smem(size_t smem_bytes);
 void launch_stage(int nitems, size_t smem, cudaStream_t st, const SlabDesc* slabs, const WorkItem* items,
                   const double* tables, const double* taps, const double* src, const double* base,
                   double* out, const double* mom_in, double* mom_out, long long NF, long long NN,
-                  double alpha, double beta, int mode, int Z, unsigned* err);
+                  double alpha, double beta, int mode, int Z, int Q, unsigned* err);
 void launch_iso_reset_p(int prec, int nitems, size_t smem, cudaStream_t st, const SlabDesc* slabs,
                         const WorkItem* items, const double* tables, const void* rtab, void* state, double* mom,
                         long long NF, long long NN, int Z);
@@ -167,11 +167,11 @@ extern "C" evfdlb_status evfdlb_step_static(const evfdlb_params* p, double* stat
     launch_sums(nitems, st, desc, items, tables, state, mom[0], NF, NN, err);
     for (int64_t s = 0; s < nsteps; ++s) {
         launch_stage(nitems, smem, st, desc, items, tables, taps, state, nullptr, u1, mom[0], mom[1], NF, NN,
-                     0.0, 1.0, 0, Z, err);
+                     0.0, 1.0, 0, Z, p->Q, err);
         launch_stage(nitems, smem, st, desc, items, tables, taps, u1, state, u2, mom[1], mom[2], NF, NN, 0.75,
-                     0.25, 0, Z, err);
+                     0.25, 0, Z, p->Q, err);
         launch_stage(nitems, smem, st, desc, items, tables, taps, u2, state, state, mom[2], mom[0], NF, NN,
-                     1.0 / 3.0, 2.0 / 3.0, 0, Z, err);
+                     1.0 / 3.0, 2.0 / 3.0, 0, Z, p->Q, err);
         if (p->T_iso > 0.0)
             launch_iso_reset_p(EVFDLB_FP64, nitems, smem, st, desc, items, tables, tables, state, mom[0], NF, NN, Z);
     }
