@@ -117,7 +117,7 @@ class ClockSampler:
 
 TILE = 0   # --tile: fixed node tile for every leg (0: the autotuner's choice per leg)
 # 2D step: bytes of state the kernels move per node-velocity-step (FP32)
-IMPL_BYTES_2D = 168
+IMPL_BYTES_2D = 160
 # DRAM bytes (read + write) of one stage_kernel<double> launch (its one-wave
 # 12-warp form) of this workload at the one-wave 27-node tile, from
 # `ncu --set full` of the current kernel (4.51 MB read, 0 written: the outputs
@@ -271,7 +271,8 @@ def run_ours(args, rank, world):
                      "peak_nominal_note": "152 SMs x 2 FP64 FMA/clk x 2070 MHz",
                      "flops_per_launch": flops,
                      "flops_note": "2 (68 + 4Q) per node-velocity (WENO-5 face ~60, analysis 2Q, synthesis 2Q, "
-                                   "collision and RK 8; two distributions)",
+                                   "collision and RK 8; two distributions); the transforms run on the tensor "
+                                   "cores and part of the faces on the FP32 pipe",
                      "flops_per_launch_detailed": flops_detail,
                      "frac_detailed": flops_detail / (launch_ms * 1e-3) / 1e9 / peak,
                      "launch_ms": launch_ms, "stage_ms": stage_ms,
@@ -371,9 +372,9 @@ def ev2_variant(args, ev, p, T, n0, stream, flush, barrier, maxred, world, n64):
 
 def df_variant(args, ev, p, T, n0, stream, flush, barrier, maxred, world, n64):
     """The FP64_DF variant on the same slab and timing protocol: FP64 state and
-    arithmetic except the stage's Hermite analysis and synthesis, which run as
-    double-float (Dot2) sums on the FP32 pipe.  Its density after the same
-    number of steps is compared with the FP64 run."""
+    arithmetic except the stage's WENO-5 faces (double-float, FP32 pipe) and its
+    Hermite transforms (digit products, tensor cores).  Its density after the
+    same number of steps is compared with the FP64 run."""
     import dataclasses
     import numpy as np
     import torch
@@ -397,7 +398,7 @@ def df_variant(args, ev, p, T, n0, stream, flush, barrier, maxred, world, n64):
     tile = sim.tile_nodes()
     sim.close()
     return {"value": NZ * Q * args.steps * world / (ms * 1e-3) / 1e9, "unit": UNIT,
-            "dtype": "f64 (Hermite transforms and WENO-5 faces as double-float pairs on the FP32 pipe)",
+            "dtype": "f64 (WENO-5 faces as double-float pairs on the FP32 pipe, Hermite transforms as digit products on the tensor cores)",
             "ms_per_step": ms / args.steps,
             "max_rel_diff_n_vs_fp64": float(np.abs(nd - n64).max() / np.abs(n64).max()),
             "gpu_launches": 3 * args.steps, "tile_nodes": tile}
