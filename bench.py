@@ -118,11 +118,11 @@ class ClockSampler:
 TILE = 0   # --tile: fixed node tile for every leg (0: the autotuner's choice per leg)
 # 2D step: bytes of state the kernels move per node-velocity-step (FP32)
 IMPL_BYTES_2D = 160
-# DRAM bytes (read + write) of one stage_kernel<double> launch (its one-wave
-# 12-warp form) of this workload at the one-wave 27-node tile, from
-# `ncu --set full` of the current kernel (4.51 MB read, 0 written: the outputs
-# stay in the 129 MB L2); to be re-measured whenever the stage kernel changes.
-STAGE_TRAFFIC_BYTES = 4516352   # dram read + write of one stage_kernel<double> launch, tile 27 (ncu)
+# DRAM bytes (read + write) of one stage_kernel<double> launch of this workload
+# at the one-wave 27-node tile, from ncu of the current kernel (2.46 MB read,
+# 0 written: the outputs stay in the 129 MB L2); to be re-measured whenever the
+# stage kernel changes.
+STAGE_TRAFFIC_BYTES = 2460000   # dram read + write of one stage_kernel<double> launch, tile 27 (ncu)
 
 
 def tuned_tile(p, n0, T, stream):
