@@ -1353,9 +1353,15 @@ __device__ void faces(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, 
 // near in both forms (1.1e-16).  Stage of 4096 x 32: 50.6 -> 46.2 us, of
 // 65536 x 24 (tile 32): 520 -> 439 us.
 //
-// The e_r are scaled by a power of two to max(e_r) in [1, 2), so that a_r
-// stays in range whatever the size of the state or of eps; a face whose
-// max(e_r) leaves the float range takes the FP64 form.
+// The e_r are scaled by a power of two to max(e_r) in [1, 2), so that the a_r
+// do not overflow whatever the size of the state or of eps.  The divisor is of
+// the square of the second largest e_r: beside a jump two of them may stay at
+// 4 eps, and where they are small against the third their products leave the
+// range in which a pair holds both its halves (from 2^-36 of the largest on the
+// quotient loses digits, from 2^-75 on it is 0/0).  A face whose second largest e_r
+// is not above kSplitRatio of the largest, or whose largest leaves the float range,
+// takes the FP64 form; at the default eps = 1e-6 that begins at differences of
+// about 20 between neighbouring nodes, which a slab of sigma = 1 does not hold.
 // ---------------------------------------------------------------------------
 struct dfl {
     float h, l;
@@ -1401,6 +1407,8 @@ __device__ __forceinline__ float rcp_ftz(float x) {
     return r;
 }
 
+constexpr float kSplitRatio = 2.33e-10f;   // 2^-32
+
 // The face of Weno5Run from its differences, in FP64 (the range fallback).
 static __device__ __noinline__ double weno5_face_f64(double v2, double d0, double d1, double d2, double d3, double eps) {
     Weno5Run<double> w;
@@ -1443,7 +1451,8 @@ struct Weno5Split {
         const double s0 = fma(3.0, d1, -d0), s1 = d1 + d2, s2 = fma(-3.0, d2, d3);
         dfl e0 = dfl_of(fma(s0, s0, u0)), e1 = dfl_of(fma(s1, s1, u1)), e2 = dfl_of(fma(s2, s2, u2));
         const float m = fmaxf(e0.h, fmaxf(e1.h, e2.h));
-        if (!(m > 1e-30f && m < 1e37f)) return weno5_face_f64(v2, d0, d1, d2, d3, eps);
+        const float mid = fmaxf(fminf(e0.h, e1.h), fminf(fmaxf(e0.h, e1.h), e2.h));
+        if (!(m > 1e-30f && m < 1e37f && mid > kSplitRatio * m)) return weno5_face_f64(v2, d0, d1, d2, d3, eps);
         const float sc = __int_as_float(0x7f000000 - (__float_as_int(m) & 0x7f800000));   // 2^-exponent(m)
         e0 = dfl_scale(e0, sc);
         e1 = dfl_scale(e1, sc);
