@@ -1358,10 +1358,15 @@ __device__ void faces(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, 
 // the square of the second largest e_r: beside a jump two of them may stay at
 // 4 eps, and where they are small against the third their products leave the
 // range in which a pair holds both its halves (from 2^-36 of the largest on the
-// quotient loses digits, from 2^-75 on it is 0/0).  A face whose second largest e_r
-// is not above kSplitRatio of the largest, or whose largest leaves the float range,
-// takes the FP64 form; at the default eps = 1e-6 that begins at differences of
-// about 20 between neighbouring nodes, which a slab of sigma = 1 does not hold.
+// quotient loses digits, from 2^-75 on it is 0/0).  The pairs are cut before they
+// are scaled, and a value below 2^-74 keeps its upper half alone: with eps and
+// differences that small the weights would have 24 bits (faces of grid-scale noise
+// of 1e-12 with eps = 1e-32: 6e-8 of it instead of 2e-14).  So a face takes the
+// FP64 form unless its second largest e_r is above kSplitRatio of the largest and
+// above kSplitLeast (a third one below 2^-74 then weighs less than 2^-14 of
+// that, squared), and the largest is in the float range; at the default eps =
+// 1e-6 that begins at differences of about 20 between neighbouring nodes, which
+// a slab of sigma = 1 does not hold.
 // ---------------------------------------------------------------------------
 struct dfl {
     float h, l;
@@ -1408,6 +1413,7 @@ __device__ __forceinline__ float rcp_ftz(float x) {
 }
 
 constexpr float kSplitRatio = 2.33e-10f;   // 2^-32
+constexpr float kSplitLeast = 1e-18f;
 
 // The face of Weno5Run from its differences, in FP64 (the range fallback).
 static __device__ __noinline__ double weno5_face_f64(double v2, double d0, double d1, double d2, double d3, double eps) {
@@ -1452,7 +1458,7 @@ struct Weno5Split {
         dfl e0 = dfl_of(fma(s0, s0, u0)), e1 = dfl_of(fma(s1, s1, u1)), e2 = dfl_of(fma(s2, s2, u2));
         const float m = fmaxf(e0.h, fmaxf(e1.h, e2.h));
         const float mid = fmaxf(fminf(e0.h, e1.h), fminf(fmaxf(e0.h, e1.h), e2.h));
-        if (!(m > 1e-30f && m < 1e37f && mid > kSplitRatio * m)) return weno5_face_f64(v2, d0, d1, d2, d3, eps);
+        if (!(m < 1e37f && mid > kSplitRatio * m && mid > kSplitLeast)) return weno5_face_f64(v2, d0, d1, d2, d3, eps);
         const float sc = __int_as_float(0x7f000000 - (__float_as_int(m) & 0x7f800000));   // 2^-exponent(m)
         e0 = dfl_scale(e0, sc);
         e1 = dfl_scale(e1, sc);

@@ -29,6 +29,8 @@ def profile(kind, nx):
     z = np.arange(nx) / nx
     if kind == "smooth":
         return 0.3 * (1 + 0.4 * np.sin(2 * np.pi * z) ** 3)
+    if kind == "rough":                     # grid-scale noise
+        return 0.3 * (1 + 0.3 * np.random.default_rng(nx).uniform(-1, 1, nx))
     n = np.full(nx, 0.1)
     if kind == "hat":                       # flat, up by a jump, flat, down again
         n[nx // 4:nx // 2] = 0.4
@@ -72,3 +74,12 @@ def test_small_unit_of_length(kind, sigma):
     """The same slab with lengths in a larger unit: densities of 4e7 and 2e10
     at the default regulariser."""
     check(60, 16, sigma, 1.0, 1e-6, kind, ev.FP64)
+
+
+@pytest.mark.parametrize("scale", [1e-6, 1e-9, 1e-12])
+@pytest.mark.parametrize("eps", EPS)
+@pytest.mark.parametrize("kind", ["smooth", "rough"])
+def test_small_differences(eps, scale, kind):
+    """Rare gases: differences far below 1, with a regulariser above or below
+    their squares."""
+    check(60, 16, 1.0, scale, eps, kind, ev.FP64)
