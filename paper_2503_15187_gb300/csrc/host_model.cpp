@@ -160,7 +160,7 @@ void build_tables(int Q, const double* xi, const double* w, double* out) {
     if (L.Ma > L.Sp + ps.synthesis_len()) out[L.Ma - 1] = 0.0;
     int32_t ints[kTsInts] = {0};
     int32_t *sx = ints, *rk = ints + 16, *gl = ints + 32;
-    for (int l = 0; l < Q && l < 32; ++l) gl[l] = (int)(0.45 * l);
+    for (int l = 0; l < Q && l < 32; ++l) gl[l] = l / 10;
     long double T[16][16];
     const int H = ps.H < 16 ? ps.H : 16;
     long double all[16][33];
