@@ -1789,19 +1789,18 @@ void launch_coll(const Ctx2* c, cudaStream_t st, const Par2<R>& pr, const R* src
 cudaError_t configure_2d(Ctx2* c) {
     return with_q(c->s.Q, [&](auto q) {
         constexpr int Q = decltype(q)::value;
-        const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
         cudaError_t e;
         if (c->prec == EVFDLB_FP32) {
             c->smem_coll = sizeof(float) * Coll2Lay<Q>::PIPE;
-            e = cudaFuncSetAttribute(k2_coll_pipe<Q>, attr, (int)c->smem_coll);
+            e = raise_smem_limit((const void*)k2_coll_pipe<Q>, c->smem_coll);
             int per_sm = 0;
             if (e == cudaSuccess)
                 e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k2_coll_pipe<Q>, coll_threads<Q>(), c->smem_coll);
             c->coll_ctas = c->sms * std::max(1, per_sm);
         } else {
             c->smem_coll = sizeof(double) * Coll2Lay<Q>::ONE;
-            e = cudaFuncSetAttribute(k2_coll<double, Q>, attr, (int)c->smem_coll);
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(k2_adv<double, Q, false>, attr, (int)adv_smem<double>());
+            e = raise_smem_limit((const void*)k2_coll<double, Q>, c->smem_coll);
+            if (e == cudaSuccess) e = raise_smem_limit((const void*)k2_adv<double, Q, false>, adv_smem<double>());
         }
         return e;
     });
@@ -1958,10 +1957,8 @@ evfdlb_status create_2d(const evfdlb_params& p, void* stream, Ctx2** out) {
                          : fields_smem_bytes<double>(s.Mf, s.mfm, s.nfm, c->field_warps);
     if (c->smem_fields > 227 * 1024) e = cudaErrorInvalidValue;   // force disc too wide for a tile
     if (e == cudaSuccess)
-        e = f32 ? cudaFuncSetAttribute(fields_kernel_of<float>(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)c->smem_fields)
-                : cudaFuncSetAttribute(fields_kernel_of<double>(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)c->smem_fields);
+        e = raise_smem_limit(f32 ? (const void*)fields_kernel_of<float>(c) : (const void*)fields_kernel_of<double>(c),
+                             c->smem_fields);
     if (e == cudaSuccess) e = configure_2d(c);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) {

@@ -816,9 +816,9 @@ size_t adj_smem_bytes(int Q, int Z) { return adj_smem_doubles(Q, Z) * sizeof(dou
 size_t adj_moments_smem_bytes(int Q, int Z, int m, int M) { return adj_moments_smem_doubles(Q, Z, m, M) * sizeof(double); }
 
 cudaError_t configure_adjoint(size_t smem_bytes, size_t smem2_bytes) {
-    cudaError_t e = cudaFuncSetAttribute(adj_local_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    cudaError_t e = raise_smem_limit((const void*)adj_local_kernel, smem_bytes);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(adj_moments_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2_bytes);
+    return raise_smem_limit((const void*)adj_moments_kernel, smem2_bytes);
 }
 
 // One stage of the reverse sweep (see the file comment) over the work items

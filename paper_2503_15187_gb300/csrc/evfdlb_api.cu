@@ -16,6 +16,7 @@
 namespace evfdlb {
 size_t stage_smem_bytes_p(int prec, int Q, int Z, int M);
 size_t stage_smem_cap_p(int prec, int Q, int M);
+size_t tile_smem_bytes_p(int prec, int Q, int Z, int M);
 cudaError_t configure_kernels_p(int prec, size_t smem_bytes);
 void launch_stage_p(int prec, int nitems, size_t smem, cudaStream_t st, const SlabDesc* slabs,
                     const WorkItem* items, const double* tables, const void* rtab, const double* taps,
@@ -104,7 +105,8 @@ struct evfdlb_ctx {
     long long NF = 0;           // elements of F (= of G) over all slabs
     long long NN = 0;           // nodes over all slabs
     int Z = 1;                  // node tile of the work items
-    size_t smem = 0;
+    size_t smem = 0;             // shared memory of a stage, and of the kernels without its tables
+    size_t smem_tile = 0;
     int device = 0;
     cudaStream_t user = nullptr;
     cudaStream_t cap = nullptr;  // private stream used only for graph capture
@@ -264,7 +266,7 @@ void queue_step(evfdlb_ctx* c, cudaStream_t st) {
     stage(f1, f0, f2, m1, m2, 0.75, 0.25);                 // u2 = 3/4 u + 1/4 (u1 + dt L(u1))
     stage(f2, f0, f0, m2, m0, 1.0 / 3.0, 2.0 / 3.0);       // u_new = 1/3 u + 2/3 (u2 + dt L(u2)), over u
     if (c->iso)                                            // isothermal slabs: T back to T_iso
-        launch_iso_reset_p(c->prec, n, c->smem, st, c->slabs, c->items, c->tables, c->rtables, f0, m0, c->NF,
+        launch_iso_reset_p(c->prec, n, c->smem_tile, st, c->slabs, c->items, c->tables, c->rtables, f0, m0, c->NF,
                            c->NN, c->Z);
 }
 
@@ -313,6 +315,7 @@ void partition(evfdlb_ctx* c, int Z) {
         for (int i0 = lo; i0 < hi; i0 += Z) c->items_h.push_back(WorkItem{s, i0, std::min(Z, hi - i0), 0});
     }
     c->smem = stage_smem_bytes_p(c->df ? EVFDLB_FP64_DF : c->prec, c->Qmax, Z, c->Mmax);
+    c->smem_tile = tile_smem_bytes_p(c->prec, c->Qmax, Z, c->Mmax);
     if (c->items_cap == 0) c->items_cap = (size_t)c->NN;
     c->tiles_h.assign(c->nbatch, 0);
     for (const WorkItem& w : c->items_h) ++c->tiles_h[w.slab];
@@ -720,7 +723,7 @@ evfdlb_status evfdlb_init(evfdlb_ctx* c, const double* n0, const double* u0, con
             TRY_CUDA(cudaMemsetAsync(c->mom[i], 0, sizeof(double) * kNumMoments * c->NN, c->user));
         }
     }
-    launch_init_p(c->prec, (int)c->items_h.size(), c->smem, c->user, c->slabs, c->items, c->tables, c->rtables, dn,
+    launch_init_p(c->prec, (int)c->items_h.size(), c->smem_tile, c->user, c->slabs, c->items, c->tables, c->rtables, dn,
                   du, dT, c->state[0], c->mom[0], c->NF, c->NN, c->Z, c->err);
     TRY_CUDA(cudaGetLastError());
     if (c->ckpt_every > 0) {   // trajectory origin for the adjoint
@@ -861,7 +864,7 @@ evfdlb_status evfdlb_fields(evfdlb_ctx* c, double* fields, int32_t on_device) {
     if (c->c2) return EVFDLB_E_UNSUPPORTED;
     if (!c->have_state) return EVFDLB_E_STATE;
     double* buf = c->scratch;
-    launch_fields_p(c->prec, (int)c->items_h.size(), c->smem, c->user, c->slabs, c->items, c->rtables, c->taps,
+    launch_fields_p(c->prec, (int)c->items_h.size(), c->smem_tile, c->user, c->slabs, c->items, c->rtables, c->taps,
                     c->rtaps, c->mom[0], buf, c->NN, c->Z, c->err);
     TRY_CUDA(cudaGetLastError());
     evfdlb_status s = copy_out(c, fields, buf, sizeof(double) * EVFDLB_NFIELDS * c->NN, on_device);
@@ -1012,7 +1015,7 @@ evfdlb_status evfdlb_stage(evfdlb_ctx* c, int32_t stage) {
     else {
         queue_stage(c, c->user, f2, f0, f0, m2, m0, 1.0 / 3.0, 2.0 / 3.0);
         if (c->iso)
-            launch_iso_reset_p(c->prec, (int)c->items_h.size(), c->smem, c->user, c->slabs, c->items, c->tables,
+            launch_iso_reset_p(c->prec, (int)c->items_h.size(), c->smem_tile, c->user, c->slabs, c->items, c->tables,
                                c->rtables, f0, m0, c->NF, c->NN, c->Z);
         ++c->steps;
     }
@@ -1061,7 +1064,7 @@ evfdlb_status evfdlb_rhs_vjp(evfdlb_ctx* c, const double* WF, const double* WG, 
     if ((st = copy_in(c, w + c->NF, WG, bytes, on_device)) != EVFDLB_OK) return st;
     TRY_CUDA(cudaMemsetAsync(a.phis, 0, sizeof(double) * c->NN, c->user));
     // the node fields of the state, then one transposed right-hand side
-    launch_fields_p(EVFDLB_FP64, (int)c->items_h.size(), c->smem, c->user, c->slabs, c->items, c->tables, c->taps,
+    launch_fields_p(EVFDLB_FP64, (int)c->items_h.size(), c->smem_tile, c->user, c->slabs, c->items, c->tables, c->taps,
                     c->taps, c->mom[0], a.fld, c->NN, c->Z, c->err);
     adj_stage(c, (const double*)c->state[0], a.fld, c->mom[0], w, nullptr, nullptr, o, 0.0, 1.0, 0, 0.0, 0.0, 0.0);
     launch_adj_phi(c->nbatch, c->user, c->slabs, a.phis, a.phi, a.dphi);

@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <mutex>
 #include <type_traits>
 #include <utility>
 
@@ -39,6 +40,18 @@ inline void launch_pdl(void (*k)(P...), int grid, int threads, size_t smem, cuda
     cfg.attrs = at;
     cfg.numAttrs = 1;
     (void)cudaLaunchKernelEx(&cfg, k, std::forward<A>(args)...);
+}
+
+// Raises the limit on a kernel's dynamic shared memory on the current device to
+// at least `bytes`.  The limit belongs to the kernel, not to the context that
+// asks, so it is never lowered: another context's launches may need more.
+inline cudaError_t raise_smem_limit(const void* kernel, size_t bytes) {
+    static std::mutex m;                               // (looking and setting are two calls)
+    std::lock_guard<std::mutex> lock(m);
+    cudaFuncAttributes a;
+    cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess || (size_t)a.maxDynamicSharedSizeBytes >= bytes) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 __device__ __forceinline__ int gidx(int i, int nx, int bc) {

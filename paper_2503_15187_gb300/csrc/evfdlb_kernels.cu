@@ -38,6 +38,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <initializer_list>
 #include <type_traits>
 #include <utility>
 
@@ -511,7 +512,7 @@ __global__ void __launch_bounds__(StageThreads<double>::value, 2) persist_kernel
 }
 
 cudaError_t configure_persist(size_t smem_bytes) {
-    return cudaFuncSetAttribute(persist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    return raise_smem_limit((const void*)persist_kernel, smem_bytes);
 }
 
 // Resident CTAs of the persistent kernel on the current device (at least one).
@@ -823,12 +824,23 @@ size_t stage_smem_cap_p(int prec, int Q, int M) {
     return full <= kStageSmemLimit ? full : std::max(most, kStageSmemLimit);
 }
 
+// Shared memory of the kernels that read no transform tables (initial state,
+// isothermal reset, fields).
+size_t tile_smem_bytes_p(int prec, int Q, int Z, int M) {
+    return prec == EVFDLB_FP32 ? smem_bytes_t<float>(Q, Z, M) : smem_bytes_t<double>(Q, Z, M);
+}
+
+static cudaError_t raise_smem_limits(std::initializer_list<const void*> kernels, size_t bytes) {
+    for (const void* k : kernels) {
+        const cudaError_t e = raise_smem_limit(k, bytes);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 cudaError_t configure_df(size_t smem_bytes) {
-    cudaError_t e = cudaFuncSetAttribute(stage_kernel<double, true, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem_bytes);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(stage_kernel<double, true, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem_bytes);
+    return raise_smem_limits({(const void*)stage_kernel<double, true, 256>, (const void*)stage_kernel<double, true, 512>},
+                             smem_bytes);
 }
 
 // SMs of the current device (cached per device).
@@ -862,42 +874,25 @@ void launch_stage_df(int nitems, size_t smem, cudaStream_t st, const SlabDesc* s
 
 template <typename R>
 static cudaError_t configure_t(size_t smem_bytes) {
-    cudaError_t e = cudaFuncSetAttribute(stage_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(stage_kernel<R, false, (StageThreads<R>::value == 512 ? 256 : 512)>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(init_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(iso_reset_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
-    if (e != cudaSuccess) return e;
-    if (std::is_same<R, double>::value) {
-        e = cudaFuncSetAttribute(stage_fields_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaFuncSetAttribute(fields_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    cudaError_t e = raise_smem_limits({(const void*)stage_kernel<R>,
+                                       (const void*)stage_kernel<R, false, (StageThreads<R>::value == 512 ? 256 : 512)>,
+                                       (const void*)init_kernel<R>, (const void*)iso_reset_kernel<R>,
+                                       (const void*)fields_kernel<R>},
+                                      smem_bytes);
+    if (e == cudaSuccess && std::is_same<R, double>::value)
+        e = raise_smem_limit((const void*)stage_fields_kernel, smem_bytes);
+    return e;
 }
 
 cudaError_t configure_kernels_p(int prec, size_t smem_bytes) {
     return prec == EVFDLB_FP32 ? configure_t<float>(smem_bytes) : configure_t<double>(smem_bytes);
 }
 
-cudaError_t configure_kernels(size_t smem_bytes) { return configure_t<double>(smem_bytes); }
-
-// Raises (never lowers) the dynamic shared-memory limit of the FP64 stage and
-// isothermal-reset kernels on the current device to at least smem_bytes.
+// The limits of the FP64 stage and isothermal-reset kernels on the current device.
 cudaError_t ensure_stage_smem(size_t smem_bytes) {
-    const void* fns[3] = {(const void*)stage_kernel<double>, (const void*)stage_kernel<double, false, 512>,
-                          (const void*)iso_reset_kernel<double>};
-    for (const void* f : fns) {
-        cudaFuncAttributes a;
-        cudaError_t e = cudaFuncGetAttributes(&a, f);
-        if (e != cudaSuccess) return e;
-        if ((size_t)a.maxDynamicSharedSizeBytes >= smem_bytes) continue;
-        e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    return raise_smem_limits({(const void*)stage_kernel<double>, (const void*)stage_kernel<double, false, 512>,
+                              (const void*)iso_reset_kernel<double>},
+                             smem_bytes);
 }
 
 // The FP64 stage: 8 warps (see StageThreads), or 16 (one CTA an SM) where the work
