@@ -44,6 +44,7 @@ struct Slab2 {
     int nx, ny, Q, relax;
     long long N;          // nodes, nx * ny
     int nft, nfm;         // force and Fischer-Methfessel taps
+    int fm_staged;        // whether k2_fields stages the latter in shared memory
     int Mf, mfm;          // their radii in nodes
     double dx;
 };
@@ -400,12 +401,14 @@ static_assert(kTile2 == 16 && 2 * kFRows == kTile2 && kFPlanHead > kFMaxWarps &&
 // apart (the two row blocks of a warp) fall 16 banks apart
 __host__ __device__ inline int fields_pitch(int W) { return W + ((6 - W % 4) % 4); }
 
+// nfm: the Fischer-Methfessel taps staged beside the densities (0: none)
 template <typename R>
 __host__ __device__ inline size_t fields_smem_bytes(int Mf, int mfm, int nfm, int warps) {
     const int H = Mf > mfm + 2 ? Mf : mfm + 2, W = kTile2 + 2 * H, E = kTile2 + 4, Wr = fields_pitch(W);
     const size_t nr = (size_t)(W + kFRows) * Wr, pf = 2 * (size_t)warps * kTile2 * kTile2;
     return sizeof(R) * ((nr > pf ? nr : pf) + 5 * (size_t)E * E + nfm) + sizeof(int) * (size_t)nfm;
 }
+constexpr size_t kFSmemLimit = 227 * 1024;
 
 template <typename R, int NW>
 __global__ void __launch_bounds__(32 * NW)
@@ -444,10 +447,13 @@ k2_fields(Slab2 s, const Par2<R> pr, const double* __restrict__ mom, const float
             Nr[cy * Wr + cx] = n;
         }
     }
-    // Fischer-Methfessel taps as offsets in the staged density
+    // Fischer-Methfessel taps as offsets in the staged density, where there is
+    // room for them: the disc of sigma = 43 dx has 5800 taps (47 KB in FP32), and with
+    // r_cut = 2.5 sigma the densities alone take 221 KB.  Else they are read from global
+    // memory below.
     R* fw = Ct + E * E;
     int* fo = reinterpret_cast<int*>(fw + s.nfm);
-    for (int t = threadIdx.x; t < s.nfm; t += 32 * NW) {
+    for (int t = threadIdx.x; s.fm_staged && t < s.nfm; t += 32 * NW) {
         fw[t] = fm_w[t];
         fo[t] = fm_off[2 * t + 1] * Wr + fm_off[2 * t];
     }
@@ -473,8 +479,13 @@ k2_fields(Slab2 s, const Par2<R> pr, const double* __restrict__ mom, const float
         const int hy = cy - 2 + H, hx = cx - 2 + H;   // position in the halo array
         R nb = R(0);
         const R* c = Nr + hy * Wr + hx;
+        if (s.fm_staged) {
 #pragma unroll 4
-        for (int t = 0; t < s.nfm; ++t) nb = fma(fw[t], c[fo[t]], nb);
+            for (int t = 0; t < s.nfm; ++t) nb = fma(fw[t], c[fo[t]], nb);
+        } else {
+            for (int t = 0; t < s.nfm; ++t)
+                nb = fma(__ldg(fm_w + t), c[__ldg(fm_off + 2 * t + 1) * Wr + __ldg(fm_off + 2 * t)], nb);
+        }
         const R eta = pr.eta_coef * nb, om = R(1) - eta;
         const R chi = (R(2) - eta) / (R(2) * om * om * om);
         const R n = Nr[hy * Wr + hx];
@@ -1953,9 +1964,13 @@ evfdlb_status create_2d(const evfdlb_params& p, void* stream, Ctx2** out) {
         e = f32 ? cudaMemcpy(c->fm_w, mwf.data(), sizeof(float) * mwf.size(), cudaMemcpyHostToDevice)
                 : cudaMemcpy(c->fm_w, t.mw.data(), sizeof(double) * t.mw.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(c->err, 0, sizeof(unsigned));
-    c->smem_fields = f32 ? fields_smem_bytes<float>(s.Mf, s.mfm, s.nfm, c->field_warps)
-                         : fields_smem_bytes<double>(s.Mf, s.mfm, s.nfm, c->field_warps);
-    if (c->smem_fields > 227 * 1024) e = cudaErrorInvalidValue;   // force disc too wide for a tile
+    auto fields_smem = [&](int nfm) {
+        return f32 ? fields_smem_bytes<float>(s.Mf, s.mfm, nfm, c->field_warps)
+                   : fields_smem_bytes<double>(s.Mf, s.mfm, nfm, c->field_warps);
+    };
+    s.fm_staged = fields_smem(s.nfm) <= kFSmemLimit;
+    c->smem_fields = fields_smem(s.fm_staged ? s.nfm : 0);
+    if (c->smem_fields > kFSmemLimit) e = cudaErrorInvalidValue;   // force disc too wide for a tile
     if (e == cudaSuccess)
         e = raise_smem_limit(f32 ? (const void*)fields_kernel_of<float>(c) : (const void*)fields_kernel_of<double>(c),
                              c->smem_fields);
