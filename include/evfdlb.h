@@ -78,8 +78,9 @@ enum {
  * state and FP64 arithmetic except the WENO-5 faces, which run as double-float
  * pairs (hi, lo floats, ~47 bits) on the FP32 pipe, and the Hermite analysis
  * and synthesis of the stage, which run as products of digit slices on the
- * tensor cores (~56 bits; FP64 slabs with Q > 16 as well); the adjoint returns
- * E_UNSUPPORTED for it. */
+ * tensor cores (~56 bits; FP64 slabs with Q > 16 as well); a context with a
+ * slab of weno_eps < 1e-8, beyond the range of such pairs, runs as FP64; the
+ * adjoint returns E_UNSUPPORTED for FP64_DF. */
 enum { EVFDLB_FP64 = 0, EVFDLB_FP32 = 1, EVFDLB_FP64_DF = 2 };
 /* Force model (Sec. II.A).  EV1: the convolution of Eq. (F1), Simpson taps
  * over |z| <= r_cut.  EV2: its gradient expansion, Eq. (F2),

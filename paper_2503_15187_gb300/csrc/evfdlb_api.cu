@@ -132,7 +132,8 @@ struct evfdlb_ctx {
     bool have_state = false;
     bool poisoned = false;
     bool iso = false;            // some slab has T_iso > 0 (reset after every step)
-    bool df = false;             // FP64_DF: FP64 context whose stages use double-float transforms
+    bool df = false;             // FP64_DF: FP64 context ...
+    bool df_stage = false;       // ... whose stages form their faces in double-float
     // z-split slab (EVFDLB_BC_HALO): G ghost nodes per side, and the RK stage
     // that evfdlb_stage runs next (0 after init / set_state / a whole step)
     bool halo = false;
@@ -219,7 +220,7 @@ void free_ctx(evfdlb_ctx* c) {
 void queue_stage(evfdlb_ctx* c, cudaStream_t st, const void* src, const void* base, void* out, const double* mi,
                  double* mo, double a, double b) {
     const int n = (int)c->items_h.size();
-    if (c->df)
+    if (c->df_stage)
         launch_stage_df(n, c->smem, st, c->slabs, c->items, c->tables, c->taps, (const double*)src,
                         (const double*)base, (double*)out, nullptr, mi, mo, c->NF, c->NN, a, b, 0, c->Z, c->err);
     else
@@ -286,7 +287,7 @@ void queue_step(evfdlb_ctx* c, cudaStream_t st) {
 // room for larger ones, 129 against 124 at 64).
 int default_tile(const evfdlb_ctx* c, int sms) {
     const int one = (int)std::min<long long>(std::max<long long>((c->NN + sms - 1) / sms, 1), kZMax);
-    if (c->df) return c->NN <= (long long)kZMax * sms || c->Qmax <= 8 ? one : 32;
+    if (c->df_stage) return c->NN <= (long long)kZMax * sms || c->Qmax <= 8 ? one : 32;
     if (c->prec == EVFDLB_FP32 && one <= 32) return one;
     std::map<int, long long> lens;              // interior nodes -> slabs
     for (const evfdlb_params& q : c->params) ++lens[q.nx - c->halo_lo - c->halo_hi];
@@ -314,7 +315,7 @@ void partition(evfdlb_ctx* c, int Z) {
         const int lo = c->halo_lo, hi = c->params[s].nx - c->halo_hi;
         for (int i0 = lo; i0 < hi; i0 += Z) c->items_h.push_back(WorkItem{s, i0, std::min(Z, hi - i0), 0});
     }
-    c->smem = stage_smem_bytes_p(c->df ? EVFDLB_FP64_DF : c->prec, c->Qmax, Z, c->Mmax);
+    c->smem = stage_smem_bytes_p(c->df_stage ? EVFDLB_FP64_DF : c->prec, c->Qmax, Z, c->Mmax);
     c->smem_tile = tile_smem_bytes_p(c->prec, c->Qmax, Z, c->Mmax);
     if (c->items_cap == 0) c->items_cap = (size_t)c->NN;
     c->tiles_h.assign(c->nbatch, 0);
@@ -566,6 +567,13 @@ evfdlb_status evfdlb_create(const evfdlb_params* p, int32_t nbatch, const evfdlb
     c->user = (cudaStream_t)cuda_stream;
     c->df = (ps[0].precision == EVFDLB_FP64_DF);
     c->prec = c->df ? EVFDLB_FP64 : ps[0].precision;   // FP64_DF is an FP64 context but for its stages
+    // The double-float faces do not scale their products: where every smoothness
+    // indicator is 4 eps these are (4 eps)^4, which in floats has 12 bits left of its
+    // lower half at eps = 1e-9 and is zero at 1e-12 (every face NaN).  A test in the
+    // kernel, of a face or of a slab, costs every stage 1 to 9 %; so a context with
+    // such an eps runs the FP64 stage.
+    c->df_stage = c->df;
+    for (int s = 0; s < nbatch; ++s) c->df_stage = c->df_stage && ps[s].weno_eps >= 1e-8;
     c->ckpt_every = ps[0].ckpt_every > 0 ? ps[0].ckpt_every : 0;
     c->esize = (c->prec == EVFDLB_FP32) ? sizeof(float) : sizeof(double);
     if (cudaGetDevice(&c->device) != cudaSuccess) { free_ctx(c); return EVFDLB_E_CUDA; }
@@ -667,9 +675,9 @@ evfdlb_status evfdlb_create(const evfdlb_params* p, int32_t nbatch, const evfdlb
     if (e == cudaSuccess)
         e = cudaMemcpy(c->items, c->items_h.data(), sizeof(WorkItem) * c->items_h.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(c->err, 0, sizeof(unsigned));
-    const size_t cap = stage_smem_cap_p(c->df ? EVFDLB_FP64_DF : c->prec, Qmax, Mmax);
+    const size_t cap = stage_smem_cap_p(c->df_stage ? EVFDLB_FP64_DF : c->prec, Qmax, Mmax);
     if (e == cudaSuccess) e = configure_kernels_p(c->prec, cap);
-    if (e == cudaSuccess && c->df) e = configure_df(cap);
+    if (e == cudaSuccess && c->df_stage) e = configure_df(cap);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         evfdlb_status st = cuda_status(e);
@@ -843,7 +851,7 @@ evfdlb_status evfdlb_rhs(evfdlb_ctx* c, double* RF, double* RG, int32_t on_devic
     if (c->c2) return c->c2_state ? rhs_2d(c->c2, RF, RG, on_device) : EVFDLB_E_STATE;
     if (!c->have_state) return EVFDLB_E_STATE;
     if (c->halo) return EVFDLB_E_UNSUPPORTED;
-    if (c->df)
+    if (c->df_stage)
         launch_stage_df((int)c->items_h.size(), c->smem, c->user, c->slabs, c->items, c->tables, c->taps,
                         (const double*)c->state[0], nullptr, nullptr, c->scratch, c->mom[0], nullptr, c->NF,
                         c->NN, 0.0, 1.0, 1, c->Z, c->err);

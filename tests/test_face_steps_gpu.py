@@ -68,6 +68,13 @@ def test_jump_beside_flat(eps, kind):
     check(60, 16, 1.0, 1.0, eps, kind, ev.FP64)
 
 
+@pytest.mark.parametrize("kind", ["smooth", "hat", "spike", "jumps"])
+@pytest.mark.parametrize("eps", EPS)
+def test_jump_beside_flat_double_float(eps, kind):
+    """FP64_DF, whose faces do not scale their products."""
+    check(60, 16, 1.0, 1.0, eps, kind, ev.FP64_DF)
+
+
 @pytest.mark.parametrize("sigma", [1 / 512, 1 / 4096])
 @pytest.mark.parametrize("kind", ["smooth", "hat", "spike"])
 def test_small_unit_of_length(kind, sigma):
