@@ -1151,7 +1151,9 @@ k2_coll_pipe(Slab2 s, const Par2<float> pr, const float2* __restrict__ st, const
 // The WENO-5 walk of Weno5Run on pairs.  With g_0 = 2 s_0 - d_1,
 // g_1 = 6 (s_1 + d_2), g_2 = 3 (d_2 - s_2) (60 times the candidate
 // corrections times their linear weights) the face is
-// v2 + (sum a_r g_r) / (6 (a_0 + 6 a_1 + 3 a_2)).  The divisor is at least
+// v2 + (sum a_r g_r) / (6 (a_0 + 6 a_1 + 3 a_2)).  The sum is formed of g_r / 64,
+// in as many operations, so that in FP32 it does not overflow before that of the
+// weighted corrections would (noise of 4000 in F; without it from 2800 on).  The divisor is at least
 // 10 (4 eps)^4: a normal FP32 number for eps >= kFtzMinEps, where FTZ takes
 // the flushing reciprocal; below, the quotient that also covers subnormals.
 constexpr double kFtzMinEps = 1e-9;
@@ -1179,17 +1181,18 @@ struct Weno5Run2 {
         else return make_float2(__fdividef(a.x, b.x), __fdividef(a.y, b.y));
     }
     __device__ __forceinline__ R2 face() const {
-        // s_0 and the g_r with their signs turned (no negations)
+        // s_0 and the g_r with their signs turned (no negations), the g_r over 64
         const R2 s0 = fma2(splat(R(-3)), d1, d0), s1 = add2(d1, d2), s2 = fma2(splat(R(-3)), d2, d3);
         const R2 e0 = fma2(s0, s0, u0), e1 = fma2(s1, s1, u1), e2 = fma2(s2, s2, u2);
         const R2 E0 = mul2(e0, e0), E1 = mul2(e1, e1), E2 = mul2(e2, e2);
         const R2 a0 = mul2(E1, E2), a1 = mul2(E0, E2), a2 = mul2(E0, E1);
-        const R2 g0 = fma2(splat(R(2)), s0, d1);
-        const R2 g1 = fma2(splat(R(-12)), d2, mul2(splat(R(-6)), d1));
-        const R2 g2 = fma2(splat(R(-12)), d2, mul2(splat(R(3)), d3));
+        const R2 x = mul2(splat(R(1.0 / 64.0)), d1), y = mul2(splat(R(-12.0 / 64.0)), d2);
+        const R2 g0 = fma2(splat(R(2.0 / 64.0)), s0, x);
+        const R2 g1 = fma2(splat(R(-6)), x, y);
+        const R2 g2 = fma2(splat(R(3.0 / 64.0)), d3, y);
         const R2 num = fma2(a0, g0, fma2(a1, g1, mul2(a2, g2)));
         const R2 den = fma2(splat(R(6)), a1, fma2(splat(R(3)), a2, a0));
-        return fma2(splat(R(-1.0 / 6.0)), quotient(num, den), v2);
+        return fma2(splat(R(-64.0 / 6.0)), quotient(num, den), v2);
     }
     __device__ __forceinline__ void shift(R2 w5) {
         const R2 d4 = sub2(w5, v4);
