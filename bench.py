@@ -57,6 +57,17 @@ def stage_flops(Q: int, M: int, m: int) -> float:
     return 2 * Q * per_vel + per_node
 
 
+def stage_fp64_flops(Q: int, M: int, m: int) -> float:
+    """What one stage-kernel launch has the FP64 pipe do per node (Q > 16), two
+    flops an instruction as the probe counts its FMAs:
+      per velocity, node and distribution 32 instructions: face 17 (with its share
+      of a cell's), coefficients 7, combine 5, moment sums 3;
+      per node the force taps 2M+1, the Fischer-Methfessel taps 2m+1, the
+      Hermite moments 3Q, gradients, transport and constants 120.
+    The transforms run on the tensor cores, the rest of the faces on the FP32 pipe."""
+    return 2.0 * (2 * Q * 32 + (2 * M + 1) + (2 * m + 1) + 3 * Q + 120)
+
+
 def fp64_peak_gflops(sm_mhz: float, sms: int = 152) -> float:
     """Nominal FP64 FMA rate of GB300: 2 FP64 FMA per clock per SM (4 flops)."""
     return sms * 4 * sm_mhz * 1e6 / 1e9
@@ -244,8 +255,7 @@ def run_ours(args, rank, world):
     del sd
     M, m = int(round(6.0 / DZ)), int(round(1.0 / DZ))
     launch_ms = statistics.mean(stage_ms)          # measured per stage launch (above)
-    flops = stage_flops_method(Q) * NZ
-    flops_detail = stage_flops(Q, M, m) * NZ
+    flops = stage_fp64_flops(Q, M, m) * NZ
     achieved = flops / (launch_ms * 1e-3) / 1e9
     peak = peak_meas
     peak_nom = fp64_peak_gflops(2070.0)
@@ -270,11 +280,10 @@ def run_ours(args, rank, world):
                      "peak_nominal": peak_nom, "frac_of_nominal": achieved / peak_nom,
                      "peak_nominal_note": "152 SMs x 2 FP64 FMA/clk x 2070 MHz",
                      "flops_per_launch": flops,
-                     "flops_note": "2 (68 + 4Q) per node-velocity (WENO-5 face ~60, analysis 2Q, synthesis 2Q, "
-                                   "collision and RK 8; two distributions); the transforms run on the tensor "
-                                   "cores and part of the faces on the FP32 pipe",
-                     "flops_per_launch_detailed": flops_detail,
-                     "frac_detailed": flops_detail / (launch_ms * 1e-3) / 1e9 / peak,
+                     "flops_note": "instructions left on the FP64 pipe x 2 (bench.stage_fp64_flops); the "
+                                   "transforms run on the tensor cores and part of the faces on the FP32 pipe; "
+                                   "bound by latency between the phases, the pipe 54 % busy under ncu",
+                     "flops_per_launch_method": stage_flops_method(Q) * NZ,
                      "launch_ms": launch_ms, "stage_ms": stage_ms,
                      "launch_note": "CUDA events around each stage launch alone (evfdlb_profile_stage), "
                                     f"mean over {nprof} steps",
