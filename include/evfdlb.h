@@ -73,14 +73,23 @@ enum {
     EVFDLB_BC_HALO_OUTFLOW_LO = 3,
     EVFDLB_BC_HALO_OUTFLOW_HI = 4
 };
-/* Precision.  FP64: every step in FP64.  FP32: FP32 state and per-velocity
- * work, FP64 chi / transport / gradients / conserved sums.  FP64_DF: FP64
- * state and FP64 arithmetic except the WENO-5 faces, which run as double-float
- * pairs (hi, lo floats, ~47 bits) on the FP32 pipe, and the Hermite analysis
- * and synthesis of the stage, which run as products of digit slices on the
- * tensor cores (~56 bits; FP64 slabs with Q > 16 as well); a context with a
- * slab of weno_eps < 1e-8, beyond the range of such pairs, runs as FP64; the
- * adjoint returns E_UNSUPPORTED for FP64_DF. */
+/* Precision.  FP64: FP64 state and FP64 arithmetic but for two parts of a 1D
+ * slab's right-hand side, whose error stays below the rounding of a step:
+ *   - the part of a WENO-5 face that vanishes with the third differences is
+ *     formed of float pairs, about 2^-47 of it (a right-hand side, whose rounding
+ *     is some 2^-52 max|xi| / dx of the state, has 0.9 of the error of FP64 faces on
+ *     smooth profiles, the same at 3 % of grid-scale noise, 1.3 times at 30 %, up to
+ *     1.8 times where the density jumps between nodes; a step the same in all).
+ *     Faces outside the range in which pairs hold that (smoothness indicators of a
+ *     ratio above 2^32, or below 1e-18) are FP64;
+ *   - for Q > 16 the Hermite analysis and synthesis are fixed-point sums of
+ *     digits with one exponent per node and distribution: 2^-57 of the node's
+ *     largest value in the norm sum_k F_k^2 / w_k, where an FP64 sum rounds by 2^-53
+ *     of each term; results below 2^-1022 are zero.
+ * FP32: FP32 state and per-velocity work, FP64 chi / gradients / conserved sums.
+ * FP64_DF: as FP64, with the WENO-5 faces wholly as float pairs and the Hermite
+ * transforms in digits at every Q; a context with a slab of weno_eps < 1e-8, beyond
+ * the range of such pairs, runs as FP64; the adjoint returns E_UNSUPPORTED. */
 enum { EVFDLB_FP64 = 0, EVFDLB_FP32 = 1, EVFDLB_FP64_DF = 2 };
 /* Force model (Sec. II.A).  EV1: the convolution of Eq. (F1), Simpson taps
  * over |z| <= r_cut.  EV2: its gradient expansion, Eq. (F2),
@@ -451,7 +460,8 @@ evfdlb_status evfdlb_coexistence(const evfdlb_params* p, double T, double* n_vap
                                  double* n_liquid);
 
 /* Full-range Gauss-Hermite velocity set of order Q (4 <= Q <= 64): roots of
- * the probabilists' He_Q and weights summing to 1, ascending. */
+ * the probabilists' He_Q and weights summing to 1, ascending; each value within
+ * 0.6 units in the last place (the bits may depend on the host's long double). */
 evfdlb_status evfdlb_velocity_set(int32_t Q, double* xi, double* w);
 
 #ifdef __cplusplus

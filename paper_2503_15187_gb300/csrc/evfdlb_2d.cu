@@ -1754,6 +1754,8 @@ auto with_q(int Q, F f) {
 // itself (the force disc's columns then run side by side: 96x64 26.5 -> 17.4
 // us), 16 up to one and a half tiles per SM (200x200: 27.5 -> 24.2 us), else 8,
 // whose CTAs overlap each other's loads (384x384: 43.7 us against 46.9 and 57.1).
+// The force sum adds the warps' columns in this division's order: a grid's results
+// may differ in the last place between devices with other numbers of SMs.
 int field_warps(const Ctx2* c) {
     const long long tiles = (long long)((c->s.nx + kTile2 - 1) / kTile2) * ((c->s.ny + kTile2 - 1) / kTile2);
     return tiles <= c->sms ? kFMaxWarps : (2 * tiles <= 3LL * c->sms ? 16 : 8);

@@ -275,8 +275,9 @@ void queue_step(evfdlb_ctx* c, cudaStream_t st) {
 // smaller tiles fill the SMs better.  That is estimated: a CTA of Z nodes alone on
 // its SM takes about Z + h units (h: its share of work that does not grow with
 // the tile); a second one adds half of that, as one CTA leaves half of the SM to
-// others; the tiles go round in waves of r CTAs an SM, r by registers and shared
-// memory, and the last wave has what is left.  Measured over Q = 8 .. 32, 3001 ..
+// others; the tiles go round in waves of r CTAs an SM, and the last wave has what
+// is left.  r is 2 (the FP64 and FP32 forms are compiled for two CTAs of 256 threads), or 1
+// where the shared memory does not hold two.  Measured over Q = 8 .. 32, 3001 ..
 // 65536 nodes and seven batches, a stage at the estimate's choice takes, against
 // one tile an SM: FP64 never longer, 12000 x 32 133 -> 89 us, 8192 x 24 54 -> 45,
 // 65536 x 24 393 -> 363, 24 slabs of 200 x 16 42 -> 30; FP32 12000 x 32 48 -> 22,
@@ -284,7 +285,7 @@ void queue_step(evfdlb_ctx* c, cudaStream_t st) {
 // 32 nodes an SM waits on latency at any tile, and FP64_DF has a form of its own for
 // one tile an SM (see launch_stage_df): both keep that; more FP64_DF tiles than SMs
 // share them three at a time up to 32 nodes (65536 x 32: 395 -> 319 us; Q = 8, with
-// room for larger ones, 129 against 124 at 64).
+// room for larger ones, 129 against 124 at 64; other orders were not measured).
 int default_tile(const evfdlb_ctx* c, int sms) {
     const int one = (int)std::min<long long>(std::max<long long>((c->NN + sms - 1) / sms, 1), kZMax);
     if (c->df_stage) return c->NN <= (long long)kZMax * sms || c->Qmax <= 8 ? one : 32;

@@ -996,8 +996,11 @@ __device__ __forceinline__ void warp_pool(int* next, int n, F f) {
 // 64-bit integers, which become doubles by bit operations.  Nothing runs on the
 // FP64 pipe, which bounds the stage and spent a third of it on the sums.  The
 // result carries about 2^-56 of the largest value times the largest entry, below
-// the rounding of an FP64 sum of up to 16 terms (2^-53 each): a step's error
-// against 80-bit arithmetic is that of the plain sums or less.  Columns
+// the rounding of an FP64 sum of up to 16 terms (2^-53 each), whatever the state
+// (see kTsSlices): against 80-bit arithmetic a right-hand side has 0.8 .. 1.1 of the
+// plain sums' error (Q = 17 .. 32; noise and liquid slabs up to 4000 steps on, slabs
+// after a density step, nodes at T = 0.15 .. 1.5 and u up to 4).  Only within the rows of the
+// outermost velocities, 1e-10 of the largest and less, is it a few times theirs.  Columns
 // (nodes) are independent, so results do not depend on the tile.  Stage of
 // 4096 x 32: 44.6 -> 33.8 us, of 65536 x 24 (tile 32): 438 -> 328 us.
 //
@@ -1358,13 +1361,13 @@ __device__ void faces(const SlabDesc& sd, const WorkItem& it, const Smem<R>& s, 
 // the FP32 pipe (pairs hi + lo from the e_r and t_r; normalised products and
 // sums, about 2^-47 each).  17 FP64 operations a face, with its share of a
 // cell's, instead of 31.
-// The error of a face against extended precision is that of the FP64 form
-// or below on smooth profiles (its quotient is good to 2^-46 of the whole
-// difference; 100 000 samples of tanh profiles of every steepness), within
-// 4 % of it on grid-scale noise of 1 % of the value, 1.3 times at 3 %; one step
-// of noisy and liquid slabs, Q = 16 .. 32, against 80-bit arithmetic is equally
-// near in both forms (1.1e-16).  Stage of 4096 x 32: 50.6 -> 46.2 us, of
-// 65536 x 24 (tile 32): 520 -> 439 us.
+// The error of a right-hand side against 80-bit arithmetic, by that of the FP64
+// form: 0.87 .. 0.93 on smooth profiles (the FP64 quotient is good to 2^-46 of the
+// whole difference), 0.97 at grid-scale noise of 1 % of every value, 1.0 at 3 %,
+// 1.2 .. 1.3 at 30 %, 1.2 .. 1.8 on slabs of density jumps (there the FP64 form adds
+// next to nothing to v2, this one the difference of two parts of the jump's size); a step's
+// error, 1.2e-16, is the same in all of these.  Stage of 4096 x 32: 50.6 -> 46.2
+// us, of 65536 x 24 (tile 32): 520 -> 439 us.
 //
 // The e_r are scaled by a power of two to max(e_r) in [1, 2), so that the a_r
 // do not overflow whatever the size of the state or of eps.  The divisor is of

@@ -24,13 +24,17 @@
 //   (4) write the new stage and its raw moment sums for the next stage.
 // FP64 is the GB300's scarcest pipe (about 1/60 of FP32), so the design
 // minimises FP64 instructions: one division per WENO face, per-node work
-// shared by all velocities, no re-reads of the state.
+// shared by all velocities, no re-reads of the state, and off that pipe what keeps
+// its precision elsewhere: the Hermite transforms on the tensor cores, part of
+// each face on the FP32 pipe.
 //
 // Precision variants.  The kernels are templated on R, the type of the stored
 // distributions and of the per-velocity work (WENO faces, Hermite analysis and
 // synthesis, the force convolution, the coefficient recurrences and the RK
-// combine).  R = double is the plain FP64 form.  R = float is the FP32
-// variant; it keeps FP64 for the Fischer-Methfessel average, chi and the
+// combine).  R = double: FP64, with the nonlinear part of a face in double-float
+// (faces_split) and for Q > 16 the transforms as digit products (analysis_task,
+// synthesis_task); FP64_DF: faces wholly in double-float and digit products at every
+// Q.  R = float is the FP32 variant; it keeps FP64 for the Fischer-Methfessel average, chi and the
 // transport coefficients (the equation-of-state part, which is sensitive near
 // liquid packing), the gradients, and the per-node sums of the conserved
 // moments (mass, momentum, energy); the heat-flux sums are FP32.
@@ -672,7 +676,9 @@ sums_kernel(const SlabDesc* __restrict__ slabs, const WorkItem* __restrict__ ite
     }
 }
 
-// Node fields of the current state (diagnostic).
+// Node fields of the current state (evfdlb_fields, evfdlb_rhs_vjp), by node_fields; the
+// FP64 stage forms the same quantities in node_roles with its own operations, so
+// that the two agree to rounding, not in bits.
 template <typename R>
 __global__ void __launch_bounds__(kThreads)
 fields_kernel(const SlabDesc* __restrict__ slabs, const WorkItem* __restrict__ items,
