@@ -1148,7 +1148,7 @@ k2_coll_pipe(Slab2 s, const Par2<float> pr, const float2* __restrict__ st, const
 // on aligned tiles alone) took 345 us and 241 instructions, and 376 us against
 // now 128 us on a 333x250 grid, whose rows are not 16-byte aligned.
 // ---------------------------------------------------------------------------
-// The WENO-5 walk of Weno5Run on pairs.  With g_0 = 2 s_0 - d_1,
+// The WENO-5 walk of Weno5Run on pairs.  With g_0 = 5 d_1 - 2 d_0,
 // g_1 = 6 (s_1 + d_2), g_2 = 3 (d_2 - s_2) (60 times the candidate
 // corrections times their linear weights) the face is
 // v2 + (sum a_r g_r) / (6 (a_0 + 6 a_1 + 3 a_2)).  The sum is formed of g_r / 64,
@@ -1186,9 +1186,9 @@ struct Weno5Run2 {
         const R2 e0 = fma2(s0, s0, u0), e1 = fma2(s1, s1, u1), e2 = fma2(s2, s2, u2);
         const R2 E0 = mul2(e0, e0), E1 = mul2(e1, e1), E2 = mul2(e2, e2);
         const R2 a0 = mul2(E1, E2), a1 = mul2(E0, E2), a2 = mul2(E0, E1);
-        const R2 x = mul2(splat(R(1.0 / 64.0)), d1), y = mul2(splat(R(-12.0 / 64.0)), d2);
-        const R2 g0 = fma2(splat(R(2.0 / 64.0)), s0, x);
-        const R2 g1 = fma2(splat(R(-6)), x, y);
+        const R2 y = mul2(splat(R(-12.0 / 64.0)), d2);
+        const R2 g0 = fma2(splat(R(2.0 / 64.0)), d0, mul2(splat(R(-5.0 / 64.0)), d1));
+        const R2 g1 = fma2(splat(R(-6.0 / 64.0)), d1, y);
         const R2 g2 = fma2(splat(R(3.0 / 64.0)), d3, y);
         const R2 num = fma2(a0, g0, fma2(a1, g1, mul2(a2, g2)));
         const R2 den = fma2(splat(R(6)), a1, fma2(splat(R(3)), a2, a0));
